@@ -135,9 +135,8 @@ enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 
 /* Coarse Poisson solver kinds.  KERNELS: two kernel launches per PCG iteration (graph
  * WHILE loop).  PERSISTENT: the whole solve in one cooperative launch over the GPU with a
- * bounded software grid barrier; in FP64, when every row has at most 16 entries and the
- * mesh fits one 32-row slice per warp, each thread keeps its row and its PCG vectors in
- * registers.  PERSISTENT_MEM: the same without register residency.  CLUSTER: the whole
+ * bounded software grid barrier; in FP64, when the mesh fits one 32-row slice per warp with
+ * at most 16 warps per SM, each thread keeps its row and its PCG vectors in registers.  PERSISTENT_MEM: the same without register residency.  CLUSTER: the whole
  * solve in one launch of one thread-block cluster, vectors in global memory, reductions
  * through distributed shared memory.  ONCHIP (CGP_MIXED only): the FP32 inner solve on one
  * cluster of 8 or 16 CTAs with the FP32 matrix and the vectors held in distributed shared

@@ -161,7 +161,9 @@ static int layout(Solver& s, void* base, size_t* bytes) {
     s.geoc = cv.take<double>((size_t)7 * C.nt);
     s.Kc0f = cv.take<float>(nnzc);
     s.dinvKcf = cv.take<float>(nc);
-    s.cw64 = cv.take<double>(8 * nc);
+    // 8 vectors, or the register-resident solve's words and slots (coarse_rr.cuh; at most one
+    // CTA per SM: max_grid is 8 per SM)
+    s.cw64 = cv.take<double>(8 * nc + 12 * (size_t)(s.max_grid / 8 + 1) + 2);
     if (s.prm.guess == CGP_GUESS_LEARNED) {
         s.phi_guess = cv.take<double>(nc);
         s.mlp.carve(cv, (int)nc, 1);

@@ -11,7 +11,7 @@
 // and a two-int status buffer.
 #include <mutex>
 
-#include "coarse_pcg.cuh"
+#include "coarse_rr.cuh"
 
 namespace cgp {
 
@@ -23,6 +23,8 @@ constexpr size_t kNaCount = 32;                                           // bar
 constexpr size_t kNaPartials = 64;                                        // 2 x kNoAllocMaxCtas x 4
 constexpr size_t kNaWork = kNaPartials + 2 * (size_t)kNoAllocMaxCtas * 4; // 8 x kNoAllocMaxRows
 constexpr size_t kNaDoubles = kNaWork + 8 * (size_t)kNoAllocMaxRows;
+static_assert(12 * (size_t)(kNoAllocMaxCtas + 1) + 2 + 2 * (size_t)kNoAllocMaxRows <= 8 * (size_t)kNoAllocMaxRows,
+              "the register-resident solve's work area fits the vectors'");
 
 // Shared by every call on a device, and kept until the process exits (about 4.3 MB).
 static __device__ __align__(256) double g_noalloc_scratch[kNaDoubles];
@@ -48,6 +50,7 @@ struct NoAllocSlot {
     void* ctx;
     double* ptr;
     int grid;
+    int rr_sms;   // SMs that can hold a CTA of the register-resident solve
 };
 NoAllocSlot g_slot[kMaxDevices] = {};
 std::mutex g_slot_mu;
@@ -92,7 +95,7 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
         return CGP_EINVAL;
     }
     double* base = nullptr;
-    int max_grid = 0;
+    int max_grid = 0, rr_sms = 0;
     {
         std::lock_guard<std::mutex> lock(g_slot_mu);
         NoAllocSlot& sl = g_slot[dev];
@@ -112,11 +115,15 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
             }
             const int g = sms * (per_sm < 2 ? per_sm : 2);
             sl.grid = g < kNoAllocMaxCtas ? g : kNoAllocMaxCtas;
+            CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rr_kernel(kRRMaxWarps), 32 * kRRMaxWarps,
+                                                                   0));
+            sl.rr_sms = per_sm > 0 ? (sms < kNoAllocMaxCtas ? sms : kNoAllocMaxCtas) : 0;
             sl.ptr = (double*)p;
             sl.ctx = ctx;
         }
         base = sl.ptr;
         max_grid = sl.grid;
+        rr_sms = sl.rr_sms;
     }
     int grid = (nslices + kGridThreads / 32 - 1) / (kGridThreads / 32);
     if (grid > max_grid) grid = max_grid;
@@ -145,6 +152,13 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
     a.bar_count = reinterpret_cast<unsigned int*>(base + kNaCount);
     a.bar_err = reinterpret_cast<int*>(base + kNaCount) + 1;
     a.partials = base + kNaPartials;
+    int ctas = 0, warps = 0;
+    if (rr_sms && rr_shape(nslices, rr_sms, &ctas, &warps)) {
+        CGP_CUDA(rr_launch(a, ctas, warps, st));
+        k_noalloc_status<<<1, 1, 0, st>>>(a.st, info);
+        CGP_LAUNCH_CHECK();
+        return CGP_OK;
+    }
     // the barrier counter and its error word must start at zero on every call
     CGP_CUDA(cudaMemsetAsync(base + kNaCount, 0, 2 * sizeof(unsigned int), st));
     cudaLaunchConfig_t cfg = {};

@@ -857,16 +857,15 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
                 return CGP_EINVAL;
             }
         }
-        // register-resident variant: every slice no wider than kRRWidth and one slice per warp
-        s.coarse_rr = false;
-        if (allow_rr) {
-            std::vector<int32_t> ptr(C.nslices + 1);
-            CGP_CUDA(cudaMemcpy(ptr.data(), C.sell_ptr, sizeof(int32_t) * (C.nslices + 1), cudaMemcpyDeviceToHost));
-            int wmax = 0;
-            for (int k = 0; k < C.nslices; ++k) wmax = std::max(wmax, (ptr[k + 1] - ptr[k]) / 32);
-            int per_sm_rr = 0;
-            CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rr, k_pcg_grid_rr, kGridThreads, 0));
-            s.coarse_rr = wmax <= kRRWidth && per_sm_rr > 0 && rr_ctas_needed(C.nslices) <= sms * per_sm_rr;
+        // register-resident variant: one slice per warp, one CTA per SM
+        s.rr_ctas = s.rr_warps = 0;
+        int ctas = 0, warps = 0, per_sm_rr = 0;
+        if (allow_rr && rr_shape(C.nslices, sms, &ctas, &warps)) {
+            CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rr, rr_kernel(warps), 32 * warps, 0));
+            if (per_sm_rr > 0) {
+                s.rr_ctas = ctas;
+                s.rr_warps = warps;
+            }
         }
         // mixed form, AUTO, no room on chip: the grid-wide FP64 solve (one reduction per
         // iteration) is faster on this GPU than the FP32 inner solve (two) with the same grid
@@ -998,10 +997,13 @@ static int coarse_solve(Ctx& c) {
             PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, onchip_kernel(s.onchip.nsub), a, s.onchip)));
             return CGP_OK;
         }
+        if (s.rr_ctas && s.coarse_fp64) {
+            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(rr_launch(a, s.rr_ctas, s.rr_warps, c.st)));
+            return CGP_OK;
+        }
         CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));   // counter + error word
         cudaLaunchConfig_t cfg = {};
-        const bool rr = s.coarse_rr && s.coarse_fp64;
-        cfg.gridDim = dim3(rr ? rr_ctas_needed(C.nslices) : s.coarse_grid, 1, 1);
+        cfg.gridDim = dim3(s.coarse_grid, 1, 1);
         cfg.blockDim = dim3(kGridThreads, 1, 1);
         cfg.stream = c.st;
         cudaLaunchAttribute attr[1];
@@ -1009,8 +1011,7 @@ static int coarse_solve(Ctx& c) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (rr) PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid_rr, a)));
-        else PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid, a)));
+        PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid, a)));
         return CGP_OK;
     }
     CGP_TRY(pcg<1>(c, Ac, s.Kc0, s.dinvKc, s.rc, s.phi, &s.ks[KS_POIS], s.prm.tol_poisson, s.prm.max_it_poisson,
@@ -1709,8 +1710,8 @@ extern "C" int cgp_coarse_info(const cgp_solver* h, int32_t* kind, int32_t* ctas
         if (s.onchip_bytes) {
             k = CGP_COARSE_ONCHIP;
             n = cl = s.cluster_size;
-        } else if (s.coarse_rr && s.coarse_fp64) {
-            n = rr_ctas_needed(s.mesh->lev[s.lc].nslices);
+        } else if (s.rr_ctas && s.coarse_fp64) {
+            n = s.rr_ctas;
         } else {
             k = CGP_COARSE_PERSISTENT_MEM;
             n = s.coarse_grid;
