@@ -70,49 +70,6 @@ struct BatchStepArgs {
     KrylovState* ks;
 };
 
-// deterministic cluster-wide sums of up to 8 values (warp -> CTA -> every CTA's slot array ->
-// each CTA adds the slots in rank order); two slot sets alternate, and every sum ends with a
-// cluster barrier, so a slot is rewritten only after every CTA read it
-struct ClusterSum8 {
-    cgrp_bs::cluster_group cl;
-    double (*slots)[8];
-    double (*wsum)[8];
-    double* bcast;
-    int slot = 0;
-    __device__ ClusterSum8(double (*sl)[8], double (*ws)[8], double* bc)
-        : cl(cgrp_bs::this_cluster()), slots(sl), wsum(ws), bcast(bc) {}
-    template <int NR>
-    __device__ void sum(const double (&v)[NR], double (&tot)[NR]) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            const double s = warp_sum(v[k]);
-            if (lane == 0) wsum[wid][k] = s;
-        }
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const double s = warp_sum(lane < nw ? wsum[lane][k] : 0.0);
-                if (lane == 0) slots[slot][k] = s;
-            }
-        }
-        cl.sync();
-        if (wid == 0) {
-            const int ncl = (int)cl.num_blocks();
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                const double s = warp_sum(lane < ncl ? cl.map_shared_rank(&slots[slot][0], lane)[k] : 0.0);
-                if (lane == 0) bcast[k] = s;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < NR; ++k) tot[k] = bcast[k];
-        slot ^= 1;
-    }
-};
-
 // number of Chebyshev steps for a relative energy-norm error tol with eigenvalue bounds
 // [1/2, 2] (condition 4): 4 * 3^-n <= tol
 __host__ __device__ inline int cheb_steps_for(double tol) {
@@ -198,7 +155,7 @@ __device__ void cluster_chebyshev(const SellView& B, const T* __restrict__ val, 
 template <class T>
 __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, const T* __restrict__ dinv,
                                 const T* __restrict__ b, const BicgVecsT<T>& V, double tol2, int maxit, int restarts,
-                                bool zero_x, ClusterSum8& cs, cgrp_bs::cluster_group& cl, int crank, int csize,
+                                bool zero_x, ClusterSync& cs, cgrp_bs::cluster_group& cl, int crank, int csize,
                                 int& status, double (&rr)[2], double (&bb)[2]) {
     const int n = A.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int tid = crank * blockDim.x + threadIdx.x, nthr = csize * blockDim.x;
@@ -268,17 +225,26 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
                     }
                 }
                 const double accd[2] = {(double)acc[0], (double)acc[1]};
-                double tot[2];
-                cs.sum(accd, tot);
+                double q[2];
+                int flag;   // bit c: not finite, bit 2 + c: breakdown
+                cs.sum_to(accd, q, flag, [&](const double (&t)[2], double (&o)[2]) -> int {
+                    int f = 0;
+                    for (int c = 0; c < 2; ++c) {
+                        o[c] = rho[c] / t[c];
+                        if (!isfinite(t[c])) f |= 1 << c;
+                        else if (t[c] == 0.0) f |= 4 << c;
+                    }
+                    return f;
+                });
                 for (int c = 0; c < 2; ++c) {
                     if (done[c]) continue;
-                    if (!isfinite(tot[c])) {
+                    if (flag >> c & 1) {
                         done[c] = 1;
                         status = CGP_ENONFINITE;
-                    } else if (tot[c] != 0.0) {
-                        alpha[c] = rho[c] / tot[c];
-                    } else {
+                    } else if (flag >> (2 + c) & 1) {
                         broke = true;
+                    } else {
+                        alpha[c] = q[c];
                     }
                 }
             }
@@ -312,10 +278,13 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
                     }
                 }
                 const double accd[4] = {(double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3]};
-                double tot[4];
-                cs.sum(accd, tot);
-                for (int c = 0; c < 2; ++c)
-                    omega[c] = (!done[c] && tot[2 + c] > 0.0 && isfinite(tot[2 + c])) ? tot[c] / tot[2 + c] : 0.0;
+                double q[2];
+                int flag;
+                cs.sum_to(accd, q, flag, [](const double (&t)[4], double (&o)[2]) -> int {
+                    for (int c = 0; c < 2; ++c) o[c] = (t[2 + c] > 0.0 && isfinite(t[2 + c])) ? t[c] / t[2 + c] : 0.0;
+                    return 0;
+                });
+                for (int c = 0; c < 2; ++c) omega[c] = done[c] ? 0.0 : q[c];
             }
             {   // x += alpha y + omega z, r = s - omega t, <rhat, r>, <r, r>
                 T acc[4] = {T(0), T(0), T(0), T(0)};
@@ -331,23 +300,35 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
                     }
                 }
                 const double accd[4] = {(double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3]};
-                double tot[4];
-                cs.sum(accd, tot);
+                double q[6];   // <r, r>, the next rho, the next beta
+                int flag;      // bit c: not finite, bit 2 + c: converged, bit 4 + c: breakdown
+                cs.sum_to(accd, q, flag, [&](const double (&t)[4], double (&o)[6]) -> int {
+                    int f = 0;
+                    for (int c = 0; c < 2; ++c) {
+                        o[c] = t[2 + c];
+                        o[2 + c] = t[c];
+                        o[4 + c] = (t[c] / rho[c]) * (alpha[c] / omega[c]);
+                        if (!isfinite(t[c]) || !isfinite(t[2 + c])) f |= 1 << c;
+                        else if (t[2 + c] <= tol2 * bb[c]) f |= 4 << c;
+                        else if (omega[c] == 0.0 || t[c] == 0.0) f |= 16 << c;
+                    }
+                    return f;
+                });
                 for (int c = 0; c < 2; ++c) {
                     if (done[c]) continue;
-                    if (!isfinite(tot[c]) || !isfinite(tot[2 + c])) {
+                    if (flag >> c & 1) {
                         status = CGP_ENONFINITE;
                         done[c] = 1;
                         continue;
                     }
-                    rr[c] = tot[2 + c];
-                    if (rr[c] <= tol2 * bb[c]) {
+                    rr[c] = q[c];
+                    if (flag >> (2 + c) & 1) {
                         done[c] = 1;
-                    } else if (omega[c] == 0.0 || tot[c] == 0.0) {
+                    } else if (flag >> (4 + c) & 1) {
                         broke = true;
                     } else {
-                        beta[c] = (tot[c] / rho[c]) * (alpha[c] / omega[c]);
-                        rho[c] = tot[c];
+                        beta[c] = q[4 + c];
+                        rho[c] = q[2 + c];
                     }
                 }
             }
@@ -362,14 +343,10 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
 
 static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArgs* __restrict__ args,
                                                                          int ninst, unsigned int* queue) {
-    __shared__ double slots4[2][4];
-    __shared__ double wsum4[kClusterThreads / 32][4];
-    __shared__ double slots8[2][8];
-    __shared__ double wsum8[kClusterThreads / 32][8];
-    __shared__ double bcast8[8];
+    __shared__ ClusterShared<512> sm;
     __shared__ int job;
-    ClusterSync sy(slots4, wsum4);
-    ClusterSum8 cs(slots8, wsum8, bcast8);
+    ClusterSync sy(sm);
+    ClusterSync& cs = sy;
     cgrp_bs::cluster_group& cl = sy.cluster;
     const int crank = (int)cl.block_rank(), csize = (int)cl.num_blocks();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;

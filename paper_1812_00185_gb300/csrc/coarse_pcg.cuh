@@ -18,10 +18,8 @@
 // incoherent L1; read-only data (pattern, values, Jacobi diagonal) goes through the
 // read-only path.
 //
-// The PCG recurrence is Chronopoulos and Gear's: both dot products of an iteration are
-// formed after its vector updates, so one grid-wide reduction (one barrier) per iteration
-// suffices; w = A u is carried by a recurrence and double-buffered because the SpMV of an
-// iteration gathers w at neighbouring rows while its own rows are being rewritten.
+// The FP64 PCG recurrence is Chronopoulos and Gear's with w = A u formed every iteration: one
+// reduction and one plain barrier (u complete before its gather) per iteration.
 //
 // Mixed precision (iterative refinement, CGP_MIXED): the outer residual r = b - A x, its
 // norm and the convergence test are FP64; each inner PCG runs its SpMV and vector updates
@@ -38,6 +36,10 @@ namespace cgrp = cooperative_groups;
 
 constexpr int kClusterThreads = 1024;
 constexpr int kGridThreads = 256;
+// CTAs per SM of the memory-resident grid solve: the passes stream, so bytes in flight count.
+// 1,050,625 rows to 1e-10 (about 4,650 iterations): 331 / 257 / 233 ms with 2 / 3 / 4 (64
+// registers a thread); the update pass with two slices in flight was slower (242 ms)
+constexpr int kGridCtasPerSm = 4;
 constexpr unsigned kSpinLimit = 1u << 24;   // polls of one grid barrier before giving up (~seconds)
 constexpr unsigned kSpinLimitTest = 1u << 14;   // the same under the wait test hook (milliseconds)
 constexpr int kStagnation = 2000;           // FP64 inner iterations without halving the best residual
@@ -52,8 +54,8 @@ struct CoarsePcgArgs {
     double* b;              // rhs (projected in place when `project`)
     double* x;              // solution / initial guess
     const double* x_alt;    // optional second initial guess: used instead of x when its FP64 residual is smaller
-    double* w64;            // FP64 work: 8 vectors of n (r, u, w0, w1, z, q, s, p)
-    float* w32;             // FP32 work: 9 vectors of n (r, u, w0, w1, z, q, s, p, e)
+    double* w64;            // FP64 work: 5 vectors of n (r, u, w, s, p), or rr_work_doubles
+    float* w32;             // FP32 work: 7 vectors of n (r, u, z, q, s, p, e)
     const double* mlump;    // non-null: fix sum m_i x_i = 0 after the solve (pure Neumann)
     KrylovState* st;        // out: iter (inner iterations), rr, bb, status, done; in: mean when project
     double tol2;
@@ -79,56 +81,117 @@ template <class T>
 __device__ __forceinline__ T ldcg(const T* p) { return __ldcg(p); }
 
 // ------------------------------------------------------------------ sync policies
+// Both policies reduce the same way inside a CTA: every thread leaves its values in shared
+// memory and warp r adds the column of value r (blockDim / 32 loads and 5 shuffles), so a
+// reduction costs the narrow FP64 pipe one warp's chain per value instead of 5 NR additions
+// in every warp (a warp-wide FP64 addition holds an SM's pipe for 16 clocks).  And both hand
+// the totals to f(tot, out) on warp 0 alone, which forms the iteration's scalars: an FP64
+// divide in every thread of a 256-thread CTA holds the pipe for about 1,800 clocks.
+// f returns a flag that every thread receives with out.
+constexpr int kSumMax = 4;   // values of one reduction; every CTA has at least as many warps
+
+struct SumShared {
+    double out[2 * kSumMax];
+    int flag;
+};
+
+// (after the caller's values are in part[r][thread]) the CTA's total of value r, in every lane
+// of the calling warp; part has at least blockDim.x columns
+__device__ __forceinline__ double column_sum(const double* __restrict__ part) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (j < nw) t[j] = part[32 * j + lane];
+    for (int k = 4; k < nw; k += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + j < nw) t[j] += part[32 * (k + j) + lane];
+    double s = (t[0] + t[1]) + (t[2] + t[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+struct PassTotals {
+    template <int NR, int NO>
+    __device__ int operator()(const double (&tot)[NR], double (&out)[NO]) const {
+#pragma unroll
+        for (int k = 0; k < NR; ++k) out[k] = tot[k];
+        return 0;
+    }
+};
+
+constexpr int kMaxClusterCtas = 16;
+
+// shared memory of a ClusterSync whose CTA has at most T threads
+template <int T>
+struct ClusterShared {
+    double part[kSumMax][T];
+    double slots[2][kSumMax][kMaxClusterCtas];   // [set][value][CTA of the cluster]
+    SumShared res;
+};
+
 struct ClusterSync {
     cgrp::cluster_group cluster;
-    double (*slots)[4];
-    double (*wsum)[4];
+    double* part;
+    int cols;                                    // columns of part
+    double (*slots)[kSumMax][kMaxClusterCtas];
+    SumShared* res;
     int slot = 0;
-    __device__ ClusterSync(double (*sl)[4], double (*ws)[4]) : cluster(cgrp::this_cluster()), slots(sl), wsum(ws) {}
-    __device__ int part() const { return (int)cluster.block_rank(); }
-    __device__ int parts() const { return (int)cluster.num_blocks(); }
+    template <int T>
+    __device__ explicit ClusterSync(ClusterShared<T>& sm)
+        : cluster(cgrp::this_cluster()), part(&sm.part[0][0]), cols(T), slots(sm.slots), res(&sm.res) {}
+    __device__ int rank() const { return (int)cluster.block_rank(); }
+    __device__ int ranks() const { return (int)cluster.num_blocks(); }
     __device__ bool sync() {
         cluster.sync();
         return true;
     }
-    template <int NR>
-    __device__ bool sum(double (&v)[NR], double (&tot)[NR]) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // every CTA's partial goes into every CTA's slots before the one cluster barrier; two slot
+    // sets alternate, so a set is rewritten only after every CTA has read it (it arrived at the
+    // barrier between)
+    template <int NR, int NO, class F>
+    __device__ bool sum_to(const double (&v)[NR], double (&out)[NO], int& flag, F f) {
+        static_assert(NR <= kSumMax && NO <= 2 * kSumMax, "SumShared sizes");
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, ncl = ranks();
 #pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            double s = warp_sum(v[k]);
-            if (lane == 0) wsum[wid][k] = s;
-        }
+        for (int k = 0; k < NR; ++k) part[k * cols + threadIdx.x] = v[k];
         __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                double s = lane < nw ? wsum[lane][k] : 0.0;
-                s = warp_sum(s);
-                if (lane == 0) slots[slot][k] = s;
-            }
+        if (wid < NR) {
+            const double s = column_sum(part + wid * cols);
+            if (lane < ncl) *cluster.map_shared_rank(&slots[slot][wid][rank()], lane) = s;
         }
         cluster.sync();
-        __shared__ double bcast[4];
         if (wid == 0) {
-            const int ncl = parts();
+            double tot[NR], o[NO];
 #pragma unroll
             for (int k = 0; k < NR; ++k) {
-                double s = 0.0;
-                if (lane < ncl) s = cluster.map_shared_rank(&slots[slot][0], lane)[k];
+                tot[k] = lane < ncl ? slots[slot][k][lane] : 0.0;
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-                if (lane == 0) bcast[k] = s;
+                for (int d = kMaxClusterCtas / 2; d > 0; d >>= 1) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], d);
+                tot[k] = __shfl_sync(0xffffffffu, tot[k], lane & (kMaxClusterCtas - 1));
+            }
+            const int fl = f(tot, o);
+            if (lane == 0) {
+#pragma unroll
+                for (int k = 0; k < NO; ++k) res->out[k] = o[k];
+                res->flag = fl;
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < NR; ++k) tot[k] = bcast[k];
-        __syncthreads();
+        for (int k = 0; k < NO; ++k) out[k] = res->out[k];
+        flag = res->flag;
         slot ^= 1;
         return true;
     }
-    __device__ void finish() { cluster.sync(); }   // no CTA leaves while its shared memory may be read
+    template <int NR>
+    __device__ bool sum(const double (&v)[NR], double (&tot)[NR]) {
+        int flag;
+        return sum_to(v, tot, flag, PassTotals{});
+    }
+    __device__ void finish() { cluster.sync(); }   // no CTA leaves while its shared memory may be written
 };
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -137,20 +200,26 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     return v;
 }
 
+struct GridShared {
+    double part[kSumMax][kGridThreads];
+    double tot[kSumMax];
+    SumShared res;
+};
+
 struct GridSync {
     unsigned* count;
     int* err;
     double* partials;
-    double (*wsum)[4];
+    GridShared& sm;
     unsigned gen = 0;
     int slot = 0;
     unsigned extra = 0;            // arrivals awaited beyond the grid's (1 under the wait test hook)
     unsigned limit = kSpinLimit;
-    __device__ GridSync(unsigned* c, int* e, double* p, double (*ws)[4], int wait_test = 0)
-        : count(c), err(e), partials(p), wsum(ws), extra(wait_test ? 1u : 0u),
+    __device__ GridSync(unsigned* c, int* e, double* p, GridShared& s, int wait_test = 0)
+        : count(c), err(e), partials(p), sm(s), extra(wait_test ? 1u : 0u),
           limit(wait_test ? kSpinLimitTest : kSpinLimit) {}
-    __device__ int part() const { return (int)blockIdx.x; }
-    __device__ int parts() const { return (int)gridDim.x; }
+    __device__ int rank() const { return (int)blockIdx.x; }
+    __device__ int ranks() const { return (int)gridDim.x; }
     __device__ bool sync() {
         __shared__ int ok;
         __syncthreads();
@@ -180,43 +249,56 @@ struct GridSync {
         __syncthreads();
         return ok != 0;
     }
-    template <int NR>
-    __device__ bool sum(double (&v)[NR], double (&tot)[NR]) {
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    // per-CTA partials [set][value][CTA]; after the grid barrier warp r of every CTA adds the
+    // partials of value r in the same order (lane l takes l, l + 32, ...)
+    template <int NR, int NO, class F>
+    __device__ bool sum_to(const double (&v)[NR], double (&out)[NO], int& flag, F f) {
+        static_assert(NR <= kSumMax && NO <= 2 * kSumMax, "SumShared sizes");
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, G = (int)gridDim.x;
 #pragma unroll
-        for (int k = 0; k < NR; ++k) {
-            double s = warp_sum(v[k]);
-            if (lane == 0) wsum[wid][k] = s;
-        }
+        for (int k = 0; k < NR; ++k) sm.part[k][threadIdx.x] = v[k];
         __syncthreads();
-        double* my = partials + ((size_t)slot * gridDim.x + blockIdx.x) * 4;
-        if (wid == 0) {
-#pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                double s = lane < nw ? wsum[lane][k] : 0.0;
-                s = warp_sum(s);
-                if (lane == 0) __stcg(my + k, s);
-            }
+        double* mine = partials + ((size_t)slot * kSumMax + wid) * G;
+        if (wid < NR) {
+            const double s = column_sum(sm.part[wid]);
+            if (lane == 0) __stcg(mine + blockIdx.x, s);
         }
         if (!sync()) return false;
-        // every CTA adds the gridDim partials in the same order: lane l takes l, l+32, ...
-        __shared__ double bcast[4];
-        if (wid == 0) {
-            const double* base = partials + (size_t)slot * gridDim.x * 4;
+        if (wid < NR) {
+            double s = 0.0;
+            for (int b0 = lane; b0 < G; b0 += 32 * 8) {
+                double q[8];
 #pragma unroll
-            for (int k = 0; k < NR; ++k) {
-                double s = 0.0;
-                for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(base + (size_t)b * 4 + k);
-                s = warp_sum(s);
-                if (lane == 0) bcast[k] = s;
+                for (int j = 0; j < 8; ++j) q[j] = b0 + 32 * j < G ? __ldcg(mine + b0 + 32 * j) : 0.0;
+                s += ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) sm.tot[wid] = s;
+        }
+        __syncthreads();
+        if (wid == 0) {
+            double tot[NR], o[NO];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) tot[k] = sm.tot[k];
+            const int fl = f(tot, o);
+            if (lane == 0) {
+#pragma unroll
+                for (int k = 0; k < NO; ++k) sm.res.out[k] = o[k];
+                sm.res.flag = fl;
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < NR; ++k) tot[k] = bcast[k];
-        __syncthreads();
+        for (int k = 0; k < NO; ++k) out[k] = sm.res.out[k];
+        flag = sm.res.flag;
         slot ^= 1;
         return true;
+    }
+    template <int NR>
+    __device__ bool sum(const double (&v)[NR], double (&tot)[NR]) {
+        int flag;
+        return sum_to(v, tot, flag, PassTotals{});
     }
     __device__ void finish() {}
 };
@@ -250,7 +332,7 @@ __device__ __forceinline__ float sell_accum_f(const SellView& A, const float* __
 // ------------------------------------------------------------------ the solve
 template <class T>
 struct InnerVecs {
-    T *r, *u, *w0, *w1, *z, *q, *s, *p, *e;
+    T *r, *u, *w, *z, *q, *s, *p, *e;
 };
 
 // sum_k val(row,k) * g(col(row,k)) in precision T (FP32 values for T = float)
@@ -266,117 +348,80 @@ __device__ __forceinline__ T row_spmv(const SellView& A, const double* __restric
     }
 }
 
-// Inner PCG (Chronopoulos-Gear) on A e = r0 in precision T, starting from e = 0 and from
-// r = r0, u = D^{-1} r0 already in V (written before the last barrier).  gamma0 = <r0,u0>.
-// Returns false on a barrier timeout.  iters counts iterations across calls.
-// outcome: 0 = ended normally (target met, or stagnation), 1 = breakdown before an update
-// (the iterate is intact), 2 = a non-finite value after an update (the iterate is not).
-template <class T, class Sync>
-__device__ bool inner_pcg(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<T>& V, const T* __restrict__ dinv,
-                          int s_begin, int s_end, double gamma, double stop2, int& iters, int& outcome,
-                          double& rr_last, bool& done) {
+// Inner FP64 PCG (Chronopoulos-Gear, w = A u formed every iteration as in coarse_rr.cuh) on
+// A x = b from the residual r and u = D^{-1} r in V (written before the last barrier), with
+// gamma = <r, u>; x itself is V.e.  Two passes over the rows per iteration: w = A u with the
+// reduction, then the vector updates.  Returns false on a barrier timeout.  iters counts
+// iterations across calls.  outcome: 0 = ended normally (target met, or stagnation),
+// 1 = breakdown before an update (the iterate is intact), 2 = a non-finite value after an
+// update (the iterate is not).
+template <class Sync>
+__device__ bool inner_pcg(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<double>& V, const double* __restrict__ dinv,
+                          int s_begin, int s_end, double gamma, double stop2, int& iters, int& outcome) {
     outcome = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
-    // w0 = A u, delta = <w0, u>
-    {
-        double acc[1] = {0.0};
+    double d = 0.0, rr_best = INFINITY, part[3] = {0.0, 0.0, 0.0};
+    int best_k = 0;
+    for (int k = 0;; ++k) {
+        // w = A u, <w, u> (u is complete)
         for (int sl = s_begin + wid; sl < s_end; sl += nw) {
             const int i = sl * 32 + lane;
-            const T wv = row_spmv<T>(A, a.val, a.valf, sl, lane, [&](int j) { return ldcg(V.u + j); });
+            const double wv = row_spmv<double>(A, a.val, a.valf, sl, lane, [&](int j) { return ldcg(V.u + j); });
             if (i < A.n) {
-                __stcg(V.w0 + i, wv);
-                acc[0] += (double)wv * (double)ldcg(V.u + i);
+                __stcg(V.w + i, wv);
+                part[1] += wv * ldcg(V.u + i);
             }
         }
-        double tot[1];
-        if (!sy.template sum<1>(acc, tot)) return false;
-        double delta = tot[0];
-        T* wc = V.w0;
-        T* wn = V.w1;
-        double gamma_prev = 0.0, alpha_prev = 0.0;
-        double rr_best = INFINITY;
-        int best_k = 0;
-        done = false;
-        for (int k = 0; iters < a.maxit; ++k) {
-            double alpha, beta;
-            if (k == 0) {
-                beta = 0.0;
-                alpha = gamma / delta;
-            } else {
-                beta = gamma / gamma_prev;
-                alpha = gamma / (delta - beta * gamma / alpha_prev);
-            }
-            if (!isfinite(alpha) || alpha == 0.0) {
-                outcome = 1;
-                return true;
-            }
-            const T al = (T)alpha, be = (T)beta;
-            double part[3] = {0.0, 0.0, 0.0};
-            for (int sl = s_begin + wid; sl < s_end; sl += nw) {
-                const int i = sl * 32 + lane;
-                const T n_i = row_spmv<T>(A, a.val, a.valf, sl, lane,
-                                          [&](int j) { return __ldg(dinv + j) * ldcg(wc + j); });
-                if (i >= A.n) continue;
-                const T w_i = ldcg(wc + i);
-                const T m_i = __ldg(dinv + i) * w_i;
-                const T z_i = k ? n_i + be * ldcg(V.z + i) : n_i;
-                const T q_i = k ? m_i + be * ldcg(V.q + i) : m_i;
-                const T s_i = k ? w_i + be * ldcg(V.s + i) : w_i;
-                const T p_i = k ? ldcg(V.u + i) + be * ldcg(V.p + i) : ldcg(V.u + i);
-                __stcg(V.z + i, z_i);
-                __stcg(V.q + i, q_i);
-                __stcg(V.s + i, s_i);
-                __stcg(V.p + i, p_i);
-                __stcg(V.e + i, ldcg(V.e + i) + al * p_i);
-                const T r_i = ldcg(V.r + i) - al * s_i;
-                const T u_i = ldcg(V.u + i) - al * q_i;
-                const T wn_i = w_i - al * z_i;
-                __stcg(V.r + i, r_i);
-                __stcg(V.u + i, u_i);
-                __stcg(wn + i, wn_i);
-                part[0] += (double)r_i * (double)u_i;
-                part[1] += (double)wn_i * (double)u_i;
-                part[2] += (double)r_i * (double)r_i;
-            }
-            double t3[3];
-            if (!sy.template sum<3>(part, t3)) return false;
-            ++iters;
-            gamma_prev = gamma;
-            alpha_prev = alpha;
-            gamma = t3[0];
-            delta = t3[1];
-            rr_last = t3[2];
-            if (!isfinite(t3[2]) || !isfinite(t3[0]) || !isfinite(t3[1])) {
-                outcome = 2;
-                return true;
-            }
-            if (t3[0] == 0.0 || t3[2] == 0.0) {   // exact solution reached: nothing left to do
-                done = true;
-                return true;
-            }
-            T* tmp = wc;
-            wc = wn;
-            wn = tmp;
-            if (t3[2] <= stop2) {
-                done = true;
-                return true;
-            }
-            // the recursive residual of this recurrence can stagnate above a very tight
-            // target; hand back to the caller, which restarts from the true residual.  CG
-            // residual norms are not monotone, so only a long run without a new minimum counts.
-            if (t3[2] < 0.5 * rr_best) {
-                rr_best = t3[2];
-                best_k = k;
-            } else if (sizeof(T) == 4 && t3[2] > 1e4 * rr_best) {
-                outcome = 2;   // the FP32 recurrence is drifting away: its iterate is not to be used
-                return true;
-            } else if (k - best_k > (sizeof(T) == 4 ? kStagnation32 : kStagnation)) {
-                return true;   // stagnating: restart from the true residual
-            }
+        // out: alpha, beta, gamma, d; flag: 0 go on, else 1 + outcome
+        double o[4];
+        int flag;
+        if (!sy.sum_to(part, o, flag, [&](const double (&t)[3], double (&q)[4]) -> int {
+                const double tg = k ? t[0] : gamma, trr = k ? t[2] : INFINITY;
+                const double beta = k ? tg / gamma : 0.0;
+                q[3] = k ? t[1] - beta * beta * d : t[1];
+                q[2] = tg;
+                q[1] = beta;
+                q[0] = tg / q[3];
+                if (k && !(isfinite(t[0]) && isfinite(t[1]) && isfinite(t[2]))) return 3;
+                if (k && (t[0] == 0.0 || trr <= stop2)) return 1;
+                // CG residual norms are not monotone: only a long run without halving the
+                // smallest counts as stagnation, and hands back to the true residual
+                if (trr < 0.5 * rr_best) {
+                    rr_best = trr;
+                    best_k = k;
+                }
+                if (!isfinite(q[0]) || q[0] == 0.0) return 2;
+                return k - best_k > kStagnation || iters >= a.maxit ? 1 : 0;
+            }))
+            return false;
+        if (flag) {
+            outcome = flag - 1;
+            return true;
         }
+        gamma = o[2];
+        d = o[3];
+        part[0] = part[1] = part[2] = 0.0;
+        for (int sl = s_begin + wid; sl < s_end; sl += nw) {
+            const int i = sl * 32 + lane;
+            if (i >= A.n) continue;
+            double p_i = ldcg(V.u + i), s_i = ldcg(V.w + i);
+            if (k) {
+                p_i = fma(o[1], ldcg(V.p + i), p_i);
+                s_i = fma(o[1], ldcg(V.s + i), s_i);
+            }
+            const double r_i = fma(-o[0], s_i, ldcg(V.r + i)), u_i = __ldg(dinv + i) * r_i;
+            __stcg(V.p + i, p_i);
+            __stcg(V.s + i, s_i);
+            __stcg(V.e + i, fma(o[0], p_i, ldcg(V.e + i)));
+            __stcg(V.r + i, r_i);
+            __stcg(V.u + i, u_i);
+            part[0] += r_i * u_i;
+            part[2] += r_i * r_i;
+        }
+        ++iters;
+        if (!sy.sync()) return false;   // u is complete before it is gathered
     }
-    return true;
 }
 
 // Inner PCG in its classical form (two reductions per iteration) on A e = r0 in precision
@@ -387,9 +432,8 @@ __device__ bool inner_pcg(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<T>& 
 template <class T, class Sync>
 __device__ bool inner_pcg_classic(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<T>& V,
                                   const T* __restrict__ dinv, int s_begin, int s_end, double rz, double stop2,
-                                  int& iters, int& outcome, bool& done) {
+                                  int& iters, int& outcome) {
     outcome = 0;
-    done = false;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
     T* p_old = V.u;   // the first direction is z = u itself
@@ -413,14 +457,18 @@ __device__ bool inner_pcg_classic(const CoarsePcgArgs& a, Sync& sy, const InnerV
                 pq_acc[0] += (double)pv * (double)qi;
             }
         }
-        double pq[1];
-        if (!sy.template sum<1>(pq_acc, pq)) return false;
-        if (!(pq[0] != 0.0) || !isfinite(pq[0])) {
+        double o1[1];
+        int flag;
+        if (!sy.sum_to(pq_acc, o1, flag, [&](const double (&t)[1], double (&q)[1]) -> int {
+                q[0] = rz / t[0];   // alpha
+                return !(t[0] != 0.0) || !isfinite(t[0]);
+            }))
+            return false;
+        if (flag) {
             outcome = 1;
             return true;
         }
-        const double alpha = rz / pq[0];
-        const T al = (T)alpha;
+        const T al = (T)o1[0];
         // phase B: e += alpha p, r -= alpha q, z = D^{-1} r; <r,z>, <r,r>
         double acc2[2] = {0.0, 0.0};
         for (int sl = s_begin + wid; sl < s_end; sl += nw) {
@@ -434,36 +482,33 @@ __device__ bool inner_pcg_classic(const CoarsePcgArgs& a, Sync& sy, const InnerV
             acc2[0] += (double)rv * (double)zv;
             acc2[1] += (double)rv * (double)rv;
         }
+        // flag: 1 = not finite, 2 = target met (or exact), 3 = the FP32 recurrence is drifting
+        // away (its iterate is not to be used), 4 = stagnating
         double t2[2];
-        if (!sy.template sum<2>(acc2, t2)) return false;
+        if (!sy.sum_to(acc2, t2, flag, [&](const double (&t)[2], double (&q)[2]) -> int {
+                q[0] = t[0];
+                q[1] = t[0] / rz;   // beta
+                if (!isfinite(t[0]) || !isfinite(t[1])) return 1;
+                if (t[0] == 0.0 || t[1] == 0.0 || t[1] <= stop2) return 2;
+                if (t[1] < 0.5 * rr_best) {
+                    rr_best = t[1];
+                    best_k = k;
+                    return 0;
+                }
+                return t[1] > 1e4 * rr_best ? 3 : (k - best_k > kStagnation32 ? 4 : 0);
+            }))
+            return false;
         ++iters;
-        if (!isfinite(t2[0]) || !isfinite(t2[1])) {
-            outcome = 2;
+        if (flag) {
+            outcome = flag == 1 || flag == 3 ? 2 : 0;
             return true;
         }
-        if (t2[0] == 0.0 || t2[1] == 0.0) {
-            done = true;
-            return true;
-        }
-        beta = t2[0] / rz;
         rz = t2[0];
+        beta = t2[1];
         // from now on z lives in V.z, and the directions alternate between V.p and V.s
         z = V.z;
         p_old = p_new;
         p_new = (p_new == V.p) ? V.s : V.p;
-        if (t2[1] <= stop2) {
-            done = true;
-            return true;
-        }
-        if (t2[1] < 0.5 * rr_best) {
-            rr_best = t2[1];
-            best_k = k;
-        } else if (t2[1] > 1e4 * rr_best) {
-            outcome = 2;
-            return true;
-        } else if (k - best_k > kStagnation32) {
-            return true;
-        }
     }
     return true;
 }
@@ -472,17 +517,16 @@ template <class Sync>
 __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
-    const int part = sy.part(), parts = sy.parts();
+    const int part = sy.rank(), parts = sy.ranks();
     const int s_begin = (int)(((int64_t)A.nslices * part) / parts);
     const int s_end = (int)(((int64_t)A.nslices * (part + 1)) / parts);
     const double mean = a.project ? a.st->mean : 0.0;
     const double tol2 = a.tol2;
     const size_t n = (size_t)A.n;
     double* xv = a.x;
-    InnerVecs<double> V64{a.w64, a.w64 + n, a.w64 + 2 * n, a.w64 + 3 * n, a.w64 + 4 * n, a.w64 + 5 * n,
-                          a.w64 + 6 * n, a.w64 + 7 * n, xv};
-    InnerVecs<float> V32{a.w32, a.w32 + n, a.w32 + 2 * n, a.w32 + 3 * n, a.w32 + 4 * n, a.w32 + 5 * n,
-                         a.w32 + 6 * n, a.w32 + 7 * n, a.w32 + 8 * n};
+    InnerVecs<double> V64{a.w64, a.w64 + n, a.w64 + 2 * n, nullptr, nullptr, a.w64 + 3 * n, a.w64 + 4 * n, xv};
+    InnerVecs<float> V32{a.w32, a.w32 + n, nullptr, a.w32 + 2 * n, a.w32 + 3 * n, a.w32 + 4 * n, a.w32 + 5 * n,
+                         a.w32 + 6 * n};
     double bb = 0.0, rr_final = 0.0;
     int iters = 0, status = 0, outer = 0, used_alt = 0;
     bool mixed_now = a.mixed != 0;   // cleared if an FP32 inner solve ever produces a non-finite value
@@ -566,18 +610,14 @@ __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
             status = CGP_ENOTCONV;
             break;
         }
-        bool inner_done = false;
         bool ok;
         int outcome = 0;
-        double rr_in = 0.0;
         if (mixed_now) {
             const double stop2 = fmax(a.inner_tol * a.inner_tol * rr0, 0.25 * tol2 * bb);
-            ok = inner_pcg_classic<float>(a, sy, V32, a.dinvf, s_begin, s_end, tot[2], stop2, iters, outcome,
-                                          inner_done);
+            ok = inner_pcg_classic<float>(a, sy, V32, a.dinvf, s_begin, s_end, tot[2], stop2, iters, outcome);
         } else {
             // FP64: the inner recurrence updates x itself; the next outer pass re-checks the true residual
-            ok = inner_pcg<double>(a, sy, V64, a.dinv, s_begin, s_end, tot[2], 0.25 * tol2 * bb, iters, outcome,
-                                   rr_in, inner_done);
+            ok = inner_pcg(a, sy, V64, a.dinv, s_begin, s_end, tot[2], 0.25 * tol2 * bb, iters, outcome);
         }
         if (!ok) {
             status = CGP_ETIMEOUT;
@@ -642,9 +682,9 @@ __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
 }
 
 static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_cluster(CoarsePcgArgs a) {
-    __shared__ double slots[2][4];
-    __shared__ double wsum[kClusterThreads / 32][4];
-    ClusterSync sy(slots, wsum);
+    __shared__ ClusterShared<kClusterThreads> sm;
+    ClusterSync sy(sm);
+    sy.sync();   // every CTA runs before its shared memory is written
     coarse_pcg_body(a, sy);
 }
 
@@ -653,12 +693,11 @@ static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_cluster(Coars
 // solves each with the ClusterSync body; clusters never wait on one another.
 static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_batch(const CoarsePcgArgs* __restrict__ args, int ninst,
                                                                   unsigned int* queue) {
-    __shared__ double slots[2][4];
-    __shared__ double wsum[kClusterThreads / 32][4];
+    __shared__ ClusterShared<kClusterThreads> sm;
     __shared__ int job;
-    ClusterSync sy(slots, wsum);
+    ClusterSync sy(sm);
     for (;;) {
-        if (sy.part() == 0 && threadIdx.x == 0) job = (int)atomicAdd(queue, 1u);
+        if (sy.rank() == 0 && threadIdx.x == 0) job = (int)atomicAdd(queue, 1u);
         sy.cluster.sync();
         const int j = *sy.cluster.map_shared_rank(&job, 0);
         sy.cluster.sync();   // every CTA has read rank 0's job before it can change
@@ -668,9 +707,9 @@ static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_batch(const C
     }
 }
 
-static __global__ void __launch_bounds__(kGridThreads) k_pcg_grid(CoarsePcgArgs a) {
-    __shared__ double wsum[kGridThreads / 32][4];
-    GridSync sy(a.bar_count, a.bar_err, a.partials, wsum, a.wait_test);
+static __global__ void __launch_bounds__(kGridThreads, kGridCtasPerSm) k_pcg_grid(CoarsePcgArgs a) {
+    __shared__ GridShared sm;
+    GridSync sy(a.bar_count, a.bar_err, a.partials, sm, a.wait_test);
     coarse_pcg_body(a, sy);
 }
 

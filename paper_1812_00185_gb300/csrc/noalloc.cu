@@ -113,7 +113,7 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
                 set_error("cgp_pcg_sell_noalloc: cooperative launch unavailable");
                 return CGP_EINVAL;
             }
-            const int g = sms * (per_sm < 2 ? per_sm : 2);
+            const int g = sms * (per_sm < kGridCtasPerSm ? per_sm : kGridCtasPerSm);
             sl.grid = g < kNoAllocMaxCtas ? g : kNoAllocMaxCtas;
             CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rr_kernel(kRRMaxWarps), 32 * kRRMaxWarps,
                                                                    0));

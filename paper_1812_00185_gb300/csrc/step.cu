@@ -778,7 +778,7 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
         const Level& C = s.mesh->lev[s.lc];
         // one slice per warp is enough; never more CTAs than can be co-resident
         const int need = (C.nslices + kGridThreads / 32 - 1) / (kGridThreads / 32);
-        const int cap = sms * (per_sm < 2 ? per_sm : 2);
+        const int cap = sms * (per_sm < kGridCtasPerSm ? per_sm : kGridCtasPerSm);
         s.coarse_grid = need < cap ? need : cap;
         if (s.coarse_grid < 1) s.coarse_grid = 1;
         // mixed precision: the whole FP32 inner solve on one cluster, if it fits on chip; the
