@@ -161,9 +161,7 @@ static int layout(Solver& s, void* base, size_t* bytes) {
     s.geoc = cv.take<double>((size_t)7 * C.nt);
     s.Kc0f = cv.take<float>(nnzc);
     s.dinvKcf = cv.take<float>(nc);
-    // 8 vectors, or the register-resident solve's words and slots (coarse_rr.cuh; at most one
-    // CTA per SM: max_grid is 8 per SM)
-    s.cw64 = cv.take<double>(8 * nc + 12 * (size_t)(s.max_grid / 8 + 1) + 2);
+    s.cw64 = cv.take<double>(5 * nc + 386);   // 5 vectors, or the register-resident solve's words (coarse_rr.cuh)
     if (s.prm.guess == CGP_GUESS_LEARNED) {
         s.phi_guess = cv.take<double>(nc);
         s.mlp.carve(cv, (int)nc, 1);
@@ -175,7 +173,7 @@ static int layout(Solver& s, void* base, size_t* bytes) {
         s.phi_q = cv.take<double>(nc);
         s.proj = reinterpret_cast<ProjState*>(cv.take<double>((sizeof(ProjState) + 7) / 8));
     }
-    s.cw32 = cv.take<float>(9 * nc);
+    s.cw32 = cv.take<float>(7 * nc);
     if (s.prm.precision == CGP_MIXED) {
         // on-chip plan: at most kOnchipMaxCluster x 16 warps x kOnchipRows slices; entries: the
         // matrix, plus per leaf (rows sorted by length) one slice of the longest row (<= 64),

@@ -1,7 +1,7 @@
 // Register-resident variant of the one-launch FP64 coarse solve (Eq. 23).
 //
-// A cooperative launch of at most one CTA per SM; every warp owns at most one SELL-32 slice
-// (32 rows), and every thread keeps its row's first kRRWidth entries (column and value) and
+// A cooperative launch of thread-block clusters, at most one CTA per SM; every warp owns at most
+// one SELL-32 slice (32 rows), and every thread keeps its row's first kRRWidth entries (column and value) and
 // its PCG vectors (x, r, u, p, s, w) in registers for the whole solve; longer rows re-read
 // their remaining entries.  Same outer loop as coarse_pcg_body (FP64 true residual, restart on
 // stagnation, optional second initial guess, pure-Neumann mean fix).
@@ -22,15 +22,21 @@
 //    the generation it needs.  The reductions keep the buffer safe to overwrite: a row's next
 //    word is stored only after every CTA has published its sums, and those depend on the words
 //    read.
-//  * a reduction is one exchange: each CTA stores {partial sum, generation} words and every
-//    CTA polls all of them, so data and arrival travel together; two slot sets alternate.
-//  * the CTA's sums go through shared memory to three warps (one per sum; 16 + 5 dependent
-//    additions) instead of shuffles in every warp, and alpha and beta are formed by one warp:
-//    FP64 divides in every thread cost more than the SpMV.
-// Measured (GB300), 129^2 rows to 1e-10: 7.8 us an iteration and 4.5 ms a solve (the pipelined
-// kernel with a counting barrier, shuffles and divides in every thread: 15.7-25.0 ms);
-// 66,049 rows, 14 warps a CTA: 11 us an iteration (vectors in memory: 17.4 us).
-// Every CTA adds the partials in the same order, so all hold identical scalars.
+//  * a reduction climbs: the CTA's sums go through shared memory to three warps (one per sum)
+//    and from there to the first CTA of the cluster (st.async on its mbarrier); with several
+//    clusters the first CTAs exchange {sum, generation} words through L2, each polling one
+//    word per cluster; the first CTA's warp 0 forms alpha and beta and sends them down to its
+//    cluster.  (Every CTA polling every CTA's words took 6.5k clocks with 66 CTAs and 8.8k
+//    with 148: the polls delay the stores they wait for.)  Two sets of slots alternate.
+//  * one warp per cluster forms the scalars: FP64 divides in every thread cost more than the
+//    SpMV.  Their divides come down to one reciprocal with two Newton steps, and the checks
+//    (finite, converged, stagnating) compare bit patterns on the integer pipe.
+// Measured (GB300): 3,872 rows, one cluster of 16: 4.6 us an iteration (every CTA polling all:
+// 7.4); 129^2 rows, 9 clusters of 8: 7.0 us, 4.1 ms to 1e-10 (7.8; the pipelined kernel with a
+// counting barrier, shuffles and divides in every thread: 14-25 ms a solve); 66,049 rows, 15
+// warps a CTA: 10.7 us (vectors in memory: 17.4 us).  Of the 14k clocks of the 129^2 case the
+// gather takes 3.4k, the words between clusters 4.6k, the sums and scalars 4k.
+// Every cluster adds the partials in the same order, so all CTAs hold identical scalars.
 // Every poll is bounded: after a limit the reader marks its sums as failed, sets the error
 // word, and all CTAs leave with CGP_ETIMEOUT.
 #pragma once
@@ -41,22 +47,42 @@ namespace cgp {
 
 constexpr int kRRWidth = 8;          // entries of a row held in registers
 constexpr int kRRMaxWarps = 16;      // warps (slices) per CTA: 512 threads of up to 128 registers
-constexpr int kRRMinWarps = 8;       // fewer CTAs to poll: 4 warps took 9.4 us an iteration on 129^2 rows, 8 take 7.9
-constexpr int kRRPoll = 5;           // words a lane of the polling warps loads at a time (5 x 32 CTAs)
+constexpr int kRRMinWarps = 4;       // the reductions use three warps
+constexpr int kRRCluster = 8;        // CTAs per cluster of a launch of several clusters
+constexpr int kRRSingle = 16;        // CTAs of a launch of one cluster (small systems)
+constexpr int kRRMaxClusters = 32;   // clusters of a launch: one polled word per lane
 
-// Shape of the launch for nslices slices on `sms` SMs: as few warps per CTA as keep one CTA
-// per SM, at least kRRMinWarps.  Returns false when the system does not fit.
-inline bool rr_shape(int nslices, int sms, int* ctas, int* warps) {
-    int w = (nslices + sms - 1) / sms;
-    if (w < kRRMinWarps) w = kRRMinWarps;
-    *warps = w;
-    *ctas = (nslices + w - 1) / w;
-    return w <= kRRMaxWarps;
+struct RRShape {
+    int ctas = 0, cluster = 0, warps = 0;   // ctas = 0: the system does not fit
+};
+
+// Launch for nslices slices where `single` (0 or 1) clusters of kRRSingle and `multi` clusters
+// of kRRCluster CTAs of the largest size are co-resident: one cluster up to 8 slices per CTA
+// (no exchange through L2 in the sums), else as few warps per CTA as the clusters allow, at
+// least 8 (fewer CTAs, fewer words).
+inline RRShape rr_shape(int nslices, int single, int multi) {
+    RRShape s;
+    if (single > 0 && nslices <= 8 * kRRSingle) {
+        s.cluster = s.ctas = kRRSingle;
+        s.warps = (nslices + kRRSingle - 1) / kRRSingle;
+        if (s.warps < kRRMinWarps) s.warps = kRRMinWarps;
+        return s;
+    }
+    if (multi > kRRMaxClusters) multi = kRRMaxClusters;
+    if (multi < 1) return s;
+    s.warps = (nslices + kRRCluster * multi - 1) / (kRRCluster * multi);
+    if (s.warps < 8) s.warps = 8;
+    if (s.warps > kRRMaxWarps) return RRShape{};
+    const int need = (nslices + s.warps - 1) / s.warps;
+    s.cluster = kRRCluster;
+    s.ctas = (need + kRRCluster - 1) / kRRCluster * kRRCluster;
+    return s;
 }
 
-// Work area (doubles): slots [2][3][ctas + 1] words, the error word (2 doubles), u words [n].
+// Work area (doubles): words [2][3][kRRMaxClusters], the error word (2 doubles), u words [n].
 // Zeroed before every launch: generation 0 is never awaited.
-inline size_t rr_work_doubles(int n, int ctas) { return 12 * (size_t)(ctas + 1) + 2 + 2 * (size_t)n; }
+constexpr size_t kRRHead = 12 * (size_t)kRRMaxClusters + 2;
+inline size_t rr_work_doubles(int n) { return kRRHead + 2 * (size_t)n; }
 
 // one 16-byte {value, tag} word, single-copy atomic, at L2
 __device__ __forceinline__ void st_word(double* p, double v, unsigned long long tag) {
@@ -70,28 +96,100 @@ __device__ __forceinline__ void ld_word(const double* p, double& v, unsigned lon
                  : "memory");
 }
 
-constexpr unsigned long long kRRFail = 1ull << 63;   // tag bit: the CTA's sums are not valid
+constexpr unsigned long long kRRFail = 1ull << 63;   // tag bit: the sums are not valid
+
+// 16 bytes into another CTA's shared memory, completing 16 bytes on its mbarrier
+__device__ __forceinline__ void st_async16(uint32_t addr, double a, unsigned long long b, uint32_t mbar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(addr),
+                 "l"(__double_as_longlong(a)), "l"(b), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void mbar_init1(uint64_t* mb) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(mb)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* mb, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(mb)),
+                 "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint64_t* mb, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"((uint32_t)__cvta_generic_to_shared(mb)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+constexpr long long kRRWaitCycles = 4000000000LL;    // ~2 s: a wait this long means a lost signal
+constexpr long long kRRWaitCyclesTest = 20000000LL;  // ~10 ms, under the wait test hook
+
+// n / d by Newton's iteration for 1 / d from the 20-bit approximation (two steps: 80 bits, so
+// the quotient is within rounding of the exact one); not finite where d is 0 or not finite
+__device__ __forceinline__ double newton_quotient(double n, double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    r = fma(r, fma(-d, r, 1.0), r);
+    const double e = fma(-d, r, 1.0), q = n * r;
+    return fma(q, e, q);
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+struct RRWord {
+    double v;
+    unsigned long long tag;
+};
 
 struct RRShared {
     double part[3][kRRMaxWarps * 32];
+    RRWord up[2][3][kRRSingle];     // first CTA of the cluster: the CTAs' sums {sum, 1 if not valid}
+    RRWord down[2][3];              // {out0, out1 as bits}, {out2, out3}, {valid, -}
     double tot[3];
-    double out[4];
     int ok[3];
-    int good;
+    uint64_t up_bar[2], down_bar[2];
 };
 
 struct RRSync {
     RRShared& sm;
-    double* slots;
+    double* words;
     int* err;
-    unsigned long long gen = 0, ugen = 0;   // generations of the sums and of the u words
+    unsigned long long ugen = 0;            // generation of the u words
+    unsigned long long gen = 0;             // generation of the sums
     unsigned limit;
-    int extra;                              // slots awaited beyond the grid's (1 under the wait test hook)
+    long long cycles;
+    int test;                               // 1 under the wait test hook: the first CTA of every
+                                            // cluster also awaits 16 bytes that nothing sends
+    int rank, ncl, nclusters, cluster_id;
+    uint32_t up_remote, up_bar_remote;      // the first CTA's up[0][0][rank] and up_bar[0]
 
-    __device__ RRSync(RRShared& s, double* sl, int* e, int wait_test)
-        : sm(s), slots(sl), err(e), limit(wait_test ? kSpinLimitTest : kSpinLimit), extra(wait_test ? 1 : 0) {}
+    __device__ RRSync(RRShared& s, double* w, int* e, int wait_test)
+        : sm(s), words(w), err(e), limit(wait_test ? kSpinLimitTest : kSpinLimit),
+          cycles(wait_test ? kRRWaitCyclesTest : kRRWaitCycles), test(wait_test ? 1 : 0) {
+        cgrp::cluster_group c = cgrp::this_cluster();
+        rank = (int)c.block_rank();
+        ncl = (int)c.num_blocks();
+        nclusters = (int)gridDim.x / ncl;
+        cluster_id = (int)blockIdx.x / ncl;
+        up_remote = cluster_addr(&sm.up[0][0][rank], 0);
+        up_bar_remote = cluster_addr(&sm.up_bar[0], 0);
+        if (threadIdx.x == 0) {
+            for (int k = 0; k < 2; ++k) {
+                mbar_init1(&sm.up_bar[k]);
+                mbar_init1(&sm.down_bar[k]);
+            }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        c.sync();
+    }
 
-    // true when a waiting thread has to give up (its own limit, or another's failure)
+    // true when a thread polling memory has to give up (its own limit, or another's failure)
     __device__ bool expired(unsigned spins) const {
         if (spins > limit) {
             atomicExch(err, 1);
@@ -99,17 +197,32 @@ struct RRSync {
         }
         return (spins & 63) == 0 && *(volatile int*)err;
     }
+    __device__ bool wait(uint64_t* mb, uint32_t parity) const {
+        const long long t0 = clock64();
+        while (!mbar_try(mb, parity))
+            if (clock64() - t0 > cycles) {
+                atomicExch(err, 1);
+                return false;
+            }
+        return true;
+    }
 
-    // Grid-wide sums of (v0, v1, v2), which warp 0 hands to f(t0, t1, t2, out); every thread
-    // gets out[0..3].  `bad`: this thread's values are not valid.  False: some wait ran out.
+    // Grid-wide sums of (v0, v1, v2), which warp 0 of every cluster's first CTA hands to
+    // f(t0, t1, t2, out); every thread gets out[0..3].  `bad`: this thread's values are not
+    // valid.  False (in all threads of the CTA): some wait ran out.
+    // A set of slots is rewritten two reductions later, and a CTA gets there only after its
+    // first CTA has sent the reduction between, that is, after all contributed to it and so
+    // had read what the set held.
     template <class F>
     __device__ bool reduce(double v0, double v1, double v2, int bad, double (&out)[4], F f) {
-        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5, G = (int)gridDim.x;
+        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+        const int par = (int)(gen & 1);
+        const uint32_t phase = (uint32_t)(gen >> 1) & 1u;
+        ++gen;
         sm.part[0][tid] = v0;
         sm.part[1][tid] = v1;
         sm.part[2][tid] = v2;
         const int anybad = __syncthreads_or(bad);
-        ++gen;
         if (wid < 3) {
             // entries beyond the CTA's threads are zero (cleared at the start)
             double t[4];
@@ -121,60 +234,64 @@ struct RRSync {
             double s = (t[0] + t[1]) + (t[2] + t[3]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            // the words of one sum lie side by side, so a warp's poll reads whole lines
-            double* base = slots + 2 * (size_t)(G + 1) * (3 * (gen & 1) + wid);
-            if (lane == 0) st_word(base + 2 * (size_t)blockIdx.x, s, anybad ? gen | kRRFail : gen);
-            double a = 0.0;
-            bool ok = true;
-            for (int b0 = lane; b0 < G + extra; b0 += 32 * kRRPoll) {
-                double v[kRRPoll];
-                unsigned long long tg[kRRPoll];
-#pragma unroll
-                for (int j = 0; j < kRRPoll; ++j) {
-                    v[j] = 0.0;
-                    tg[j] = gen;
-                    if (b0 + 32 * j < G + extra) ld_word(base + 2 * (size_t)(b0 + 32 * j), v[j], tg[j]);
+            if (lane == 0)
+                st_async16(up_remote + (uint32_t)(sizeof(RRWord) * kRRSingle * (3 * par + wid)), s, anybad ? 1ull : 0ull,
+                           up_bar_remote + 8 * par);
+            if (tid == 0) mbar_expect(&sm.down_bar[par], 3 * sizeof(RRWord));
+            if (rank == 0) {
+                if (tid == 0) mbar_expect(&sm.up_bar[par], (uint32_t)sizeof(RRWord) * (3 * ncl + test));
+                bool ok = wait(&sm.up_bar[par], phase);
+                double a = 0.0;
+                if (lane < ncl) {
+                    a = sm.up[par][wid][lane].v;
+                    ok = ok && sm.up[par][wid][lane].tag == 0;
                 }
-                unsigned spins = 0;
-                for (;;) {
-                    bool wait = false;
 #pragma unroll
-                    for (int j = 0; j < kRRPoll; ++j)
-                        if ((tg[j] & ~kRRFail) != gen) {
-                            ld_word(base + 2 * (size_t)(b0 + 32 * j), v[j], tg[j]);
-                            wait |= (tg[j] & ~kRRFail) != gen;
+                for (int o = kRRSingle / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                ok = __all_sync(0xffffffffu, ok);
+                if (nclusters > 1) {
+                    double* base = words + 2 * (size_t)kRRMaxClusters * (3 * par + wid);
+                    if (lane == 0) st_word(base + 2 * cluster_id, a, ok ? gen : gen | kRRFail);
+                    unsigned long long tag = gen;
+                    a = 0.0;
+                    if (lane < nclusters) {
+                        ld_word(base + 2 * lane, a, tag);
+                        for (unsigned spins = 0; (tag & ~kRRFail) != gen;) {
+                            if (expired(++spins)) {
+                                tag = kRRFail;
+                                break;
+                            }
+                            ld_word(base + 2 * lane, a, tag);
                         }
-                    if (!wait) break;
-                    if (expired(++spins)) {
-                        ok = false;
-                        break;
+                    }
+                    ok = __all_sync(0xffffffffu, !(tag & kRRFail));
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                }
+                if (lane == 0) {
+                    sm.tot[wid] = a;
+                    sm.ok[wid] = ok;
+                }
+                asm volatile("bar.sync 1, 96;" ::: "memory");   // the three reducing warps
+                if (wid == 0) {
+                    double o[4] = {0.0, 0.0, 0.0, 0.0};
+                    f(sm.tot[0], sm.tot[1], sm.tot[2], o);
+                    if (lane < ncl) {
+                        const uint32_t dst = cluster_addr(&sm.down[par][0], lane), mb = cluster_addr(&sm.down_bar[par], lane);
+                        st_async16(dst, o[0], (unsigned long long)__double_as_longlong(o[1]), mb);
+                        st_async16(dst + 16, o[2], (unsigned long long)__double_as_longlong(o[3]), mb);
+                        st_async16(dst + 32, 0.0, sm.ok[0] && sm.ok[1] && sm.ok[2] ? 1ull : 0ull, mb);
                     }
                 }
-#pragma unroll
-                for (int j = 0; j < kRRPoll; ++j) ok = ok && !(tg[j] & kRRFail);
-                // a tree over the words of this lane; one that this CTA count does not have is 0
-                if (G > 32) a += ((v[0] + v[1]) + (v[2] + v[3])) + v[4];
-                else a = v[0];
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            ok = __all_sync(0xffffffffu, ok);
-            if (lane == 0) {
-                sm.tot[wid] = a;
-                sm.ok[wid] = ok;
-            }
-            asm volatile("bar.sync 1, 96;" ::: "memory");   // the three reducing warps
-            if (wid == 0) {
-                double o[4] = {0.0, 0.0, 0.0, 0.0};
-                f(sm.tot[0], sm.tot[1], sm.tot[2], o);
-                if (lane < 4) sm.out[lane] = lane == 0 ? o[0] : (lane == 1 ? o[1] : (lane == 2 ? o[2] : o[3]));
-                if (lane == 0) sm.good = sm.ok[0] && sm.ok[1] && sm.ok[2];
             }
         }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 4; ++k) out[k] = sm.out[k];
-        return sm.good != 0;
+        const bool got = wait(&sm.down_bar[par], phase);
+        out[0] = sm.down[par][0].v;
+        out[1] = __longlong_as_double((long long)sm.down[par][0].tag);
+        out[2] = sm.down[par][1].v;
+        out[3] = __longlong_as_double((long long)sm.down[par][1].tag);
+        const bool valid = sm.down[par][2].tag != 0;
+        return __syncthreads_and(got && valid) != 0;
     }
 };
 
@@ -182,12 +299,10 @@ struct RRSync {
 template <int kWarps>
 static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcgArgs a) {
     __shared__ RRShared sm;
-    double* const slots = a.w64;
-    int* const err = reinterpret_cast<int*>(a.w64 + 12 * (size_t)(gridDim.x + 1));
-    double* const ubuf = a.w64 + 12 * (size_t)(gridDim.x + 1) + 2;
+    int* const err = reinterpret_cast<int*>(a.w64 + kRRHead - 2);
+    double* const ubuf = a.w64 + kRRHead;
     for (int k = threadIdx.x; k < 3 * kRRMaxWarps * 32; k += blockDim.x) (&sm.part[0][0])[k] = 0.0;
-    __syncthreads();
-    RRSync sy(sm, slots, err, a.wait_test);
+    RRSync sy(sm, a.w64, err, a.wait_test);   // (ends with a cluster barrier)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
     const int sl = (int)blockIdx.x * nw + wid;              // this warp's slice (one at most)
@@ -330,39 +445,42 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         // ---- inner iterations; o = (alpha, beta, gamma, d) of the coming update, and why to
         // leave in the shared flag: 1 = target met or restart, 2 = not finite
         const double stop2 = 0.25 * a.tol2 * bb;
-        double p_i = 0.0, s_i = 0.0, rg = 0.0, c = 0.0, rr_best = INFINITY;
+        double p_i = 0.0, s_i = 0.0, rg = 0.0, c = 0.0;
+        long long half_best = 0x7ff0000000000000ll;   // bits of half the smallest <r, r> so far
         double gd[2] = {0.0, 0.0};   // gamma and d of the last update
         int best_k = 0, leave = 0;
         for (int k = 0;; ++k) {
-            // warp 0 prepares the next scalars while the words travel: 1 / gamma' and d' / gamma'^2
+            // the scalars' warp prepares 1 / gamma' and d' / gamma'^2 while the words travel
             const double w_i = multiply(u_i, [&] {
-                if (wid == 0 && k) {
+                if (wid == 0 && sy.rank == 0 && k) {
                     rg = 1.0 / gd[0];
                     c = gd[1] * rg * rg;
                 }
             });
             const bool ok = sy.reduce(
                 r_i * u_i, w_i * u_i, r_i * r_i, bad, o, [&](double tg, double td, double trr, double (&q)[4]) {
-                    const double beta = tg * rg;
                     const double dn = td - tg * tg * c;
-                    q[0] = tg / dn;
-                    q[1] = beta;
+                    q[0] = newton_quotient(tg, dn);
+                    q[1] = tg * rg;
                     q[2] = tg;
                     q[3] = dn;
-                    if (k && !(isfinite(tg) && isfinite(td) && isfinite(trr))) {
+                    // (trr is a sum of squares: for such values the bit patterns order as the
+                    // numbers do, and one exponent less is half)
+                    const long long rb = __double_as_longlong(trr);
+                    if (k && !(finite_bits(tg) && finite_bits(td) && finite_bits(trr))) {
                         q[0] = 0.0;
                         q[1] = 2.0;     // not finite after an update
-                    } else if (k && (trr <= stop2 || tg == 0.0 || trr == 0.0)) {
+                    } else if (k && (rb <= __double_as_longlong(stop2) || (__double_as_longlong(tg) << 1) == 0)) {
                         q[0] = 0.0;
                         q[1] = 1.0;
                     } else {
                         // a long run without halving the smallest residual, or a breakdown
                         // before the update: back to the true residual
-                        if (trr < 0.5 * rr_best) {
-                            rr_best = trr;
+                        if (rb < half_best) {
+                            half_best = rb - (1ll << 52);
                             best_k = k;
                         }
-                        if (!isfinite(q[0]) || k - best_k > kStagnation || iters >= a.maxit) {
+                        if (!finite_bits(q[0]) || k - best_k > kStagnation || iters >= a.maxit) {
                             q[0] = 0.0;
                             q[1] = 1.0;
                         }
@@ -403,6 +521,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
             status = CGP_ETIMEOUT;
     }
     if (row) a.x[i] = x_i;
+    cgrp::this_cluster().sync();   // no CTA leaves while its shared memory may be written
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         KrylovState* st = a.st;
         st->iter = iters;
@@ -421,20 +540,55 @@ inline auto rr_kernel(int warps) -> void (*)(CoarsePcgArgs) {
     return warps <= 8 ? k_pcg_grid_rr<8> : k_pcg_grid_rr<kRRMaxWarps>;
 }
 
-// zero the work area (a.w64), then the solve
-inline cudaError_t rr_launch(const CoarsePcgArgs& a, int ctas, int warps, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(a.w64, 0, rr_work_doubles(a.A.n, ctas) * sizeof(double), st);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
+// attributes: clusters of `cluster` CTAs, all CTAs co-resident
+inline void rr_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int ctas, int cluster, int warps,
+                      cudaStream_t st) {
+    cfg = {};
     cfg.gridDim = dim3(ctas, 1, 1);
     cfg.blockDim = dim3(32 * warps, 1, 1);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = 2;
+}
+
+// co-resident clusters: of kRRSingle CTAs with up to 8 warps, of kRRCluster CTAs of the largest size
+inline cudaError_t rr_capacity(int* single, int* multi) {
+    *single = *multi = 0;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    for (int w : {8, kRRMaxWarps}) {
+        const cudaError_t e = cudaFuncSetAttribute(rr_kernel(w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    rr_config(cfg, attr, kRRSingle, kRRSingle, 8, nullptr);
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rr_kernel(warps), a);
+    if (cudaOccupancyMaxActiveClusters(single, rr_kernel(8), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        *single = 0;
+    }
+    rr_config(cfg, attr, kRRCluster, kRRCluster, kRRMaxWarps, nullptr);
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(multi, rr_kernel(kRRMaxWarps), &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        *multi = 0;
+    }
+    return cudaSuccess;
+}
+
+// zero the work area (a.w64), then the solve
+inline cudaError_t rr_launch(const CoarsePcgArgs& a, const RRShape& sh, cudaStream_t st) {
+    const cudaError_t e = cudaMemsetAsync(a.w64, 0, rr_work_doubles(a.A.n) * sizeof(double), st);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    rr_config(cfg, attr, sh.ctas, sh.cluster, sh.warps, st);
+    return cudaLaunchKernelEx(&cfg, rr_kernel(sh.warps), a);
 }
 
 }  // namespace cgp

@@ -23,7 +23,7 @@ constexpr size_t kNaCount = 32;                                           // bar
 constexpr size_t kNaPartials = 64;                                        // 2 x kNoAllocMaxCtas x 4
 constexpr size_t kNaWork = kNaPartials + 2 * (size_t)kNoAllocMaxCtas * 4; // 8 x kNoAllocMaxRows
 constexpr size_t kNaDoubles = kNaWork + 8 * (size_t)kNoAllocMaxRows;
-static_assert(12 * (size_t)(kNoAllocMaxCtas + 1) + 2 + 2 * (size_t)kNoAllocMaxRows <= 8 * (size_t)kNoAllocMaxRows,
+static_assert(kRRHead + 2 * (size_t)kNoAllocMaxRows <= 8 * (size_t)kNoAllocMaxRows,
               "the register-resident solve's work area fits the vectors'");
 
 // Shared by every call on a device, and kept until the process exits (about 4.3 MB).
@@ -50,7 +50,7 @@ struct NoAllocSlot {
     void* ctx;
     double* ptr;
     int grid;
-    int rr_sms;   // SMs that can hold a CTA of the register-resident solve
+    int rr_single, rr_multi;   // co-resident clusters of the register-resident solve
 };
 NoAllocSlot g_slot[kMaxDevices] = {};
 std::mutex g_slot_mu;
@@ -95,7 +95,8 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
         return CGP_EINVAL;
     }
     double* base = nullptr;
-    int max_grid = 0, rr_sms = 0;
+    int max_grid = 0;
+    RRShape shape;
     {
         std::lock_guard<std::mutex> lock(g_slot_mu);
         NoAllocSlot& sl = g_slot[dev];
@@ -115,15 +116,13 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
             }
             const int g = sms * (per_sm < kGridCtasPerSm ? per_sm : kGridCtasPerSm);
             sl.grid = g < kNoAllocMaxCtas ? g : kNoAllocMaxCtas;
-            CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rr_kernel(kRRMaxWarps), 32 * kRRMaxWarps,
-                                                                   0));
-            sl.rr_sms = per_sm > 0 ? (sms < kNoAllocMaxCtas ? sms : kNoAllocMaxCtas) : 0;
+            CGP_CUDA(rr_capacity(&sl.rr_single, &sl.rr_multi));
             sl.ptr = (double*)p;
             sl.ctx = ctx;
         }
         base = sl.ptr;
         max_grid = sl.grid;
-        rr_sms = sl.rr_sms;
+        shape = rr_shape(nslices, sl.rr_single, sl.rr_multi);
     }
     int grid = (nslices + kGridThreads / 32 - 1) / (kGridThreads / 32);
     if (grid > max_grid) grid = max_grid;
@@ -152,9 +151,8 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
     a.bar_count = reinterpret_cast<unsigned int*>(base + kNaCount);
     a.bar_err = reinterpret_cast<int*>(base + kNaCount) + 1;
     a.partials = base + kNaPartials;
-    int ctas = 0, warps = 0;
-    if (rr_sms && rr_shape(nslices, rr_sms, &ctas, &warps)) {
-        CGP_CUDA(rr_launch(a, ctas, warps, st));
+    if (shape.ctas) {
+        CGP_CUDA(rr_launch(a, shape, st));
         k_noalloc_status<<<1, 1, 0, st>>>(a.st, info);
         CGP_LAUNCH_CHECK();
         return CGP_OK;

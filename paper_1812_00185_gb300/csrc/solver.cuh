@@ -68,12 +68,12 @@ struct Solver {
     ProjState* proj = nullptr;
     double* phi_guess = nullptr;  // n_c: the network's prediction of Phi_c
     int* mlp_gate = nullptr;      // the coarse solve's judge of the network (see CoarsePcgArgs::gate)
-    double* cw64 = nullptr;       // coarse one-launch solver work: 8 FP64 vectors of n_c (+ rr_work_doubles' slots)
-    float* cw32 = nullptr;        // and 9 FP32 vectors of n_c
+    double* cw64 = nullptr;       // coarse one-launch solver work: 5 FP64 vectors of n_c, or rr_work_doubles
+    float* cw32 = nullptr;        // and 7 FP32 vectors of n_c
     int coarse_kind = 0;          // CGP_COARSE_KERNELS / _CLUSTER / _PERSISTENT (AUTO resolved)
     int cluster_size = 0;         // CTAs of the one-cluster solver
     int coarse_grid = 0;          // CTAs of the persistent (cooperative) solver
-    int rr_ctas = 0, rr_warps = 0;   // launch of the register-resident FP64 solve (0 = it does not fit)
+    int rr_ctas = 0, rr_cluster = 0, rr_warps = 0;   // launch of the register-resident FP64 solve (0: does not fit)
     double *user_ud = nullptr, *user_f = nullptr;   // CGP_BC_USER: 2*nf each
     bool coarse_fp64 = true;
     cudaStream_t branch = nullptr;                 // second stream of a step (work beside the coarse solve)

@@ -857,15 +857,15 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
                 return CGP_EINVAL;
             }
         }
-        // register-resident variant: one slice per warp, one CTA per SM
-        s.rr_ctas = s.rr_warps = 0;
-        int ctas = 0, warps = 0, per_sm_rr = 0;
-        if (allow_rr && rr_shape(C.nslices, sms, &ctas, &warps)) {
-            CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_rr, rr_kernel(warps), 32 * warps, 0));
-            if (per_sm_rr > 0) {
-                s.rr_ctas = ctas;
-                s.rr_warps = warps;
-            }
+        // register-resident variant: one slice per warp, one CTA per SM, in clusters
+        s.rr_ctas = s.rr_cluster = s.rr_warps = 0;
+        if (allow_rr) {
+            int single = 0, multi = 0;
+            CGP_CUDA(rr_capacity(&single, &multi));
+            const RRShape sh = rr_shape(C.nslices, single, multi);
+            s.rr_ctas = sh.ctas;
+            s.rr_cluster = sh.cluster;
+            s.rr_warps = sh.warps;
         }
         // mixed form, AUTO, no room on chip: the grid-wide FP64 solve (one reduction per
         // iteration) is faster on this GPU than the FP32 inner solve (two) with the same grid
@@ -998,7 +998,8 @@ static int coarse_solve(Ctx& c) {
             return CGP_OK;
         }
         if (s.rr_ctas && s.coarse_fp64) {
-            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(rr_launch(a, s.rr_ctas, s.rr_warps, c.st)));
+            PL(c, CGP_PROF_POIS_CLUSTER,
+               CGP_CUDA(rr_launch(a, RRShape{s.rr_ctas, s.rr_cluster, s.rr_warps}, c.st)));
             return CGP_OK;
         }
         CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));   // counter + error word
