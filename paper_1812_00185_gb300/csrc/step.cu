@@ -212,11 +212,46 @@ __global__ void k_sub_scalar(int n, double* __restrict__ x, const double* __rest
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] -= m;
 }
 
-// Eq. 24, one level: phi[nv_c + e] = (phi[a_e] + phi[b_e]) / 2; coincident vertices keep their value
-__global__ void k_prolong(int n_new, int nv_c, const int32_t* __restrict__ parents, double* __restrict__ phi) {
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n_new; e += gridDim.x * blockDim.x) {
-        const int2 pr = reinterpret_cast<const int2*>(parents)[e];
-        phi[nv_c + e] = 0.5 * (phi[pr.x] + phi[pr.y]);
+// Eq. 24, one level: phi[nv_c + e] = (phi[a_e] + phi[b_e]) / 2; coincident vertices keep their
+// value.  With `out` (cgp_prolong into device memory) every value goes there as well, and with
+// `in` the coarse values come from there (and are stored): a stand-alone prolongation is then
+// one launch a level, without a copy in and a copy out of the whole fine field.
+// Bound by memory: 8 bytes of parents and 8 (16 with out) written per new vertex; four vertices
+// in flight per thread hide the parents -> values chain.
+__global__ void __launch_bounds__(kBlock) k_prolong(int n_new, int nv_c, const int32_t* __restrict__ parents,
+                                                    double* phi, const double* in, double* out) {
+    const int stride = gridDim.x * blockDim.x, t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const int2* __restrict__ pr = reinterpret_cast<const int2*>(parents);
+    const double* src = in ? in : phi;
+    if (in)
+        for (int i = t0; i < nv_c; i += stride) {
+            const double v = in[i];
+            phi[i] = v;
+            out[i] = v;
+        }
+    constexpr int U = 4;
+    for (int e0 = t0; e0 < n_new; e0 += U * stride) {
+        int2 q[U];
+        double a[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            q[u] = make_int2(0, 0);
+            if (e0 + u * stride < n_new) q[u] = __ldg(pr + e0 + u * stride);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            a[u] = src[q[u].x];
+            b[u] = src[q[u].y];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = e0 + u * stride;
+            if (e < n_new) {
+                const double v = 0.5 * (a[u] + b[u]);
+                phi[nv_c + e] = v;
+                if (out) out[nv_c + e] = v;
+            }
+        }
     }
 }
 
@@ -1026,13 +1061,16 @@ static int coarse_solve(Ctx& c) {
     return CGP_OK;
 }
 
-static int prolong_all(Ctx& c) {
+// every level; in / out: the coarse values and the fine field of a stand-alone prolongation
+// (device memory, null inside a step)
+static int prolong_all(Ctx& c, const double* in = nullptr, double* out = nullptr) {
     Solver& s = *c.s;
     for (int l = s.lc; l < s.lf; ++l) {
         const Level& Lc = s.mesh->lev[l];
         const Level& Lf = s.mesh->lev[l + 1];
         const int n_new = Lf.nv - Lc.nv;
-        PL(c, CGP_PROF_PROLONG, k_prolong<<<grid_rows(s, n_new, 1), kBlock, 0, c.st>>>(n_new, Lc.nv, Lf.parents, s.phi));
+        PL(c, CGP_PROF_PROLONG, k_prolong<<<grid_rows(s, n_new, 1), kBlock, 0, c.st>>>(
+                                    n_new, Lc.nv, Lf.parents, s.phi, l == s.lc ? in : nullptr, out));
     }
     CGP_LAUNCH_CHECK();
     return CGP_OK;
@@ -1758,8 +1796,14 @@ extern "C" int cgp_prolong(cgp_solver* h, const double* phi_c, double* phi_f, in
     }
     Solver& s = h->s;
     cudaStream_t st = (cudaStream_t)stream;
-    CGP_TRY(copy_in(s.phi, phi_c, sizeof(double) * s.nc, where, st));
     Ctx c{&s, st, false};
+    // device arrays: straight from phi_c into both s.phi (the solver's field, as before) and
+    // phi_f, unless the two overlap other than from the same start (a vertex's value could
+    // then be overwritten before it is read) or there is no level to prolong over
+    const char *ci = (const char*)phi_c, *fo = (const char*)phi_f;
+    const bool apart = ci == fo || ci + sizeof(double) * s.nc <= fo || fo + sizeof(double) * s.nf <= ci;
+    if (where == CGP_DEVICE && s.lc < s.lf && apart) return prolong_all(c, phi_c, phi_f);
+    CGP_TRY(copy_in(s.phi, phi_c, sizeof(double) * s.nc, where, st));
     CGP_TRY(prolong_all(c));
     CGP_TRY(copy_out(phi_f, s.phi, sizeof(double) * s.nf, where, st));
     if (where == CGP_HOST) CGP_CUDA(cudaStreamSynchronize(st));
