@@ -14,6 +14,8 @@
 // deterministic passes (per-block partials, then a fixed-order sum).
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "flows.cuh"
 #include "mlp.cuh"
 #include "solver.cuh"
@@ -112,9 +114,37 @@ __global__ void k_mlp_nmean(int n, int batch, const int32_t* __restrict__ rowptr
 // per 32-byte sector for each (neighbour, feature); a vertex-major one reads each neighbour's
 // 64 features as one 256-byte run.  The dense layer that produces the features also writes
 // this copy, hv[b][i][f] = relu(a[b][f][i]).
+// Sum over the 1-ring of vertex i (i excluded, CSR order) of the vertex-major rows vb[j], two
+// features per lane; a warp per vertex.  The lanes hold the ring's indices, so eight rows are
+// in flight at a time instead of one row after each index.
+__device__ __forceinline__ int ring_sum64(int i, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                          const float2* __restrict__ vb, int lane, float& ax, float& ay) {
+    const int rb = rowptr[i], cnt = rowptr[i + 1] - rb;
+    int deg = 0;
+    for (int e0 = 0; e0 < cnt; e0 += 32) {
+        const int m = min(32, cnt - e0), c = lane < m ? col[rb + e0 + lane] : i;
+        deg += __popc(__ballot_sync(0xffffffffu, c != i));
+        for (int e = 0; e < m; e += 8) {
+            float2 x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int j = __shfl_sync(0xffffffffu, c, (e + u) & 31);
+                x[u] = make_float2(0.0f, 0.0f);
+                if (e + u < m && j != i) x[u] = vb[(size_t)j * (kHid / 2) + lane];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                ax += x[u].x;
+                ay += x[u].y;
+            }
+        }
+    }
+    return deg;
+}
+
 // m[b][f][i] = mean over the 1-ring (i excluded) of hv[b][j][f] for 32 vertices per block: a
-// warp per vertex (lanes over features, two each, neighbours in CSR order as in
-// k_mlp_nmean), written back feature-major through shared memory
+// warp per vertex (neighbours in CSR order as in k_mlp_nmean), written back feature-major
+// through shared memory
 __global__ void __launch_bounds__(256) k_mlp_nmean64(int n, const int32_t* __restrict__ rowptr,
                                                     const int32_t* __restrict__ col, const float* __restrict__ hv,
                                                     float* __restrict__ m) {
@@ -126,17 +156,7 @@ __global__ void __launch_bounds__(256) k_mlp_nmean64(int n, const int32_t* __res
     for (int v = wid; v < 32; v += 8) {
         const int i = i0 + v;
         float ax = 0.0f, ay = 0.0f;
-        int deg = 0;
-        if (i < n) {
-            for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
-                const int j = col[e];
-                if (j == i) continue;
-                ++deg;
-                const float2 x = vb[(size_t)j * (kHid / 2) + lane];
-                ax += x.x;
-                ay += x.y;
-            }
-        }
+        const int deg = i < n ? ring_sum64(i, rowptr, col, vb, lane, ax, ay) : 0;
         const float inv = deg ? 1.0f / deg : 0.0f;
         tile[2 * lane][v] = ax * inv;
         tile[2 * lane + 1][v] = ay * inv;
@@ -149,17 +169,46 @@ __global__ void __launch_bounds__(256) k_mlp_nmean64(int n, const int32_t* __res
     }
 }
 
+// Its transpose, fused with the ReLU's: gh[b][f][j] += sum over the neighbours i of j of
+// gv[b][i][f] (vertex-major, already divided by i's degree), then gh = 0 where a_prev <= 0.
+// (A feature-major gather of gm read one 4-byte value per 32-byte sector.)
+__global__ void __launch_bounds__(256) k_mlp_nmean64_bwd(int n, const int32_t* __restrict__ rowptr,
+                                                        const int32_t* __restrict__ col, const float* __restrict__ gv,
+                                                        const float* __restrict__ a_prev, float* __restrict__ gh) {
+    __shared__ float tile[kHid][33];
+    const int b = blockIdx.y, i0 = blockIdx.x * 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const float2* vb = reinterpret_cast<const float2*>(gv + (size_t)b * n * kHid);
+    for (int v = wid; v < 32; v += 8) {
+        const int i = i0 + v;
+        float ax = 0.0f, ay = 0.0f;
+        if (i < n) ring_sum64(i, rowptr, col, vb, lane, ax, ay);
+        tile[2 * lane][v] = ax;
+        tile[2 * lane + 1][v] = ay;
+    }
+    __syncthreads();
+    const size_t o = (size_t)b * kHid * n + i0 + lane;
+    if (i0 + lane < n)
+#pragma unroll
+        for (int f = wid; f < kHid; f += 8) {
+            const size_t at = o + (size_t)f * n;
+            gh[at] = a_prev[at] > 0.0f ? gh[at] + tile[f][lane] : 0.0f;
+        }
+}
+
 // a[b][o][i] = sum_k W[o][k] x_k + bias[o], x = [act(h); m] (2*FIN inputs), summed in k
 // order; with VOUT also hv[b][i][o] = relu(a[b][o][i]) (the vertex-major copy the next
 // 1-ring mean gathers).  W (bf16, row-major FOUT x 2*FIN) is staged per block as FP32
 // columns wt[k][o]: lane l of a warp loads 8 consecutive k of row o = l (16 bytes) and
 // writes them down column l, so the transposed writes are free of bank conflicts.  With
 // FOUT >= 32 two threads share a vertex (the first half of the block takes outputs
-// [0, FOUT/2), the second half the rest, so a warp reads one wt row as a broadcast).  Each
-// thread loads its inputs in chunks, the next chunk while it multiplies the current one,
-// so the latency of the feature-major input loads overlaps the FMAs.
+// [0, FOUT/2), the second half the rest, so a warp reads one wt row as a broadcast), and each
+// thread has two vertices, so a weight read from shared memory feeds two FMAs (one read per
+// FMA held the kernel at the shared-memory pipe's rate).  Each thread loads its inputs in
+// chunks, the next chunk while it multiplies the current one, so the latency of the
+// feature-major input loads overlaps the FMAs.
 template <int FOUT>
-__host__ __device__ constexpr int dense_vertices_per_block() { return FOUT >= 32 ? 64 : 128; }   // of 128 threads
+__host__ __device__ constexpr int dense_vertices_per_block() { return 128; }   // of 128 threads
 
 template <int FIN, int FOUT, bool RELU_IN, bool VOUT>
 __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_bfloat16* __restrict__ W,
@@ -168,10 +217,11 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
                                                    float* __restrict__ hv) {
     constexpr int K = 2 * FIN;
     constexpr int VB = dense_vertices_per_block<FOUT>();
-    constexpr int OS = 128 / VB;                        // threads per vertex
+    constexpr int OS = FOUT >= 32 ? 2 : 1;              // threads per vertex
+    constexpr int V = OS * VB / 128;                    // vertices per thread
     constexpr int FO = FOUT / OS;                       // outputs per thread
     constexpr int LD = FOUT == 1 ? 1 : FOUT + 4;        // row stride of wt (16-byte rows)
-    constexpr int KCMAX = FO == 1 ? 32 : 16;
+    constexpr int KCMAX = FO == 1 ? 32 : 8;
     constexpr int KC = FIN < KCMAX ? FIN : KCMAX;       // inputs loaded per chunk
     constexpr int NV8 = K * FOUT / 8;                   // 16-byte pieces of W
     static_assert(FOUT % OS == 0 && (FO == 1 || FO % 4 == 0) && FIN % KC == 0 && K % 8 == 0, "dense layer shape");
@@ -194,31 +244,42 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
         }
     }
     __syncthreads();
-    const int part = threadIdx.x / VB;
-    const int64_t t = blockIdx.x * (int64_t)VB + threadIdx.x % VB;
-    if (t >= (int64_t)n * batch) return;
-    const int b = (int)(t / n), i = (int)(t % n);
+    constexpr int TV = 128 / OS;                        // threads over the vertices
+    const int part = threadIdx.x / TV;
     const int o0 = part * FO;
-    float acc[FO];
+    int b[V], i[V];
+    bool in[V];
+    const float *hb[V], *mb[V];
+    float acc[V][FO];
 #pragma unroll
-    for (int o = 0; o < FO; ++o) acc[o] = bias[o0 + o];
+    for (int v = 0; v < V; ++v) {
+        const int64_t t = blockIdx.x * (int64_t)VB + threadIdx.x % TV + v * TV;
+        in[v] = t < (int64_t)n * batch;
+        b[v] = in[v] ? (int)(t / n) : 0;
+        i[v] = in[v] ? (int)(t % n) : 0;
+        hb[v] = h + (size_t)b[v] * FIN * n + i[v];
+        mb[v] = m + (size_t)b[v] * FIN * n + i[v];
+#pragma unroll
+        for (int o = 0; o < FO; ++o) acc[v][o] = bias[o0 + o];
+    }
     // chunk c holds inputs k = c KC .. c KC + KC - 1: the first FIN / KC chunks come from h
     // (with the ReLU when RELU_IN), the rest from m; two register buffers alternate, so the
     // loads of chunk c + 1 are in flight while chunk c is multiplied
     constexpr int NCH = K / KC;
     static_assert(NCH % 2 == 0, "chunks come in pairs");
-    const float* hb = h + (size_t)b * FIN * n + i;
-    const float* mb = m + (size_t)b * FIN * n + i;
-    auto load = [&](float (&xs)[KC], int c) {
+    auto load = [&](float (&xs)[V][KC], int c) {
         const bool from_h = c < FIN / KC;
-        const float* src = from_h ? hb + (size_t)c * KC * n : mb + (size_t)(c - FIN / KC) * KC * n;
 #pragma unroll
-        for (int u = 0; u < KC; ++u) {
-            const float x = src[(size_t)u * n];
-            xs[u] = (RELU_IN && from_h) ? fmaxf(x, 0.0f) : x;
+        for (int v = 0; v < V; ++v) {
+            const float* src = from_h ? hb[v] + (size_t)c * KC * n : mb[v] + (size_t)(c - FIN / KC) * KC * n;
+#pragma unroll
+            for (int u = 0; u < KC; ++u) {
+                const float x = src[(size_t)u * n];
+                xs[v][u] = (RELU_IN && from_h) ? fmaxf(x, 0.0f) : x;
+            }
         }
     };
-    auto mul = [&](const float (&xs)[KC], int c) {
+    auto mul = [&](const float (&xs)[V][KC], int c) {
 #pragma unroll
         for (int u = 0; u < KC; ++u) {
             const float* wr = &wt[c * KC + u][o0];
@@ -226,18 +287,23 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
 #pragma unroll
                 for (int o = 0; o < FO; o += 4) {
                     const float4 w4 = *reinterpret_cast<const float4*>(wr + o);
-                    acc[o] += w4.x * xs[u];
-                    acc[o + 1] += w4.y * xs[u];
-                    acc[o + 2] += w4.z * xs[u];
-                    acc[o + 3] += w4.w * xs[u];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) {
+                        acc[v][o] += w4.x * xs[v][u];
+                        acc[v][o + 1] += w4.y * xs[v][u];
+                        acc[v][o + 2] += w4.z * xs[v][u];
+                        acc[v][o + 3] += w4.w * xs[v][u];
+                    }
                 }
             } else {
 #pragma unroll
-                for (int o = 0; o < FO; ++o) acc[o] += wr[o] * xs[u];
+                for (int v = 0; v < V; ++v)
+#pragma unroll
+                    for (int o = 0; o < FO; ++o) acc[v][o] += wr[o] * xs[v][u];
             }
         }
     };
-    float xa[KC], xb[KC];
+    float xa[V][KC], xb[V][KC];
     load(xa, 0);
     for (int c = 0; c < NCH; c += 2) {
         load(xb, c + 1);
@@ -245,42 +311,73 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
         if (c + 2 < NCH) load(xa, c + 2);
         mul(xb, c + 1);
     }
-    float* ab = a + (size_t)b * FOUT * n;
 #pragma unroll
-    for (int o = 0; o < FO; ++o) ab[(size_t)(o0 + o) * n + i] = acc[o];
-    if constexpr (VOUT) {
-        float4* vr = reinterpret_cast<float4*>(hv + ((size_t)b * n + i) * FOUT + o0);
+    for (int v = 0; v < V; ++v) {
+        if (!in[v]) continue;
+        float* ab = a + (size_t)b[v] * FOUT * n;
 #pragma unroll
-        for (int o = 0; o < FO; o += 4)
-            vr[o / 4] = make_float4(fmaxf(acc[o], 0.0f), fmaxf(acc[o + 1], 0.0f), fmaxf(acc[o + 2], 0.0f),
-                                    fmaxf(acc[o + 3], 0.0f));
+        for (int o = 0; o < FO; ++o) ab[(size_t)(o0 + o) * n + i[v]] = acc[v][o];
+        if constexpr (VOUT) {
+            float4* vr = reinterpret_cast<float4*>(hv + ((size_t)b[v] * n + i[v]) * FOUT + o0);
+#pragma unroll
+            for (int o = 0; o < FO; o += 4)
+                vr[o / 4] = make_float4(fmaxf(acc[v][o], 0.0f), fmaxf(acc[v][o + 1], 0.0f), fmaxf(acc[v][o + 2], 0.0f),
+                                        fmaxf(acc[v][o + 3], 0.0f));
+        }
     }
-}
-
-// Phi0 = q + s_q * out (double)
-__global__ void k_mlp_predict(int n, int batch, const double* __restrict__ q, const float* __restrict__ out,
-                              const float* __restrict__ scale, double* __restrict__ pred) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n * batch) return;
-    const int b = (int)(t / n);
-    pred[t] = q[t] + (double)scale[2 * b + 1] * (double)out[t];
 }
 
 // ---------------------------------------------------------------- backward kernels
 constexpr double kTargetClip = 10.0;
 
-// g3 = dL/da3 = 2 (a3 - clip((t - q)/s_q)) / (n * batch); loss partials per block
-__global__ void __launch_bounds__(kBlock) k_mlp_loss(int n, int batch, const double* __restrict__ q,
-                                                   const double* __restrict__ tgt, const float* __restrict__ out,
-                                                   const float* __restrict__ scale, float* __restrict__ g3,
-                                                   double* __restrict__ partials, unsigned int* ticket,
-                                                   float* __restrict__ loss) {
+// ---- layer 3 (one output) in training.  Its 1-ring mean commutes with the weights, so no
+// 64-wide mean is formed: with p = W3h . h2 and z = W3m . h2 per vertex,
+//   a3_i = b3 + p_i + mean_{j in N(i)} z_j,
+// and with g3 = dL/da3 and S_j = sum over the neighbours i of j of g3_i / deg(i),
+//   dL/dh2_j = W3h g3_j + W3m S_j,  dW3h = sum_j g3_j h2_j,  dW3m = sum_j S_j h2_j.
+// (The mean, its transpose and the products over it read and wrote 64 values per vertex eight
+// times: 620 us of a step of 32,489 vertices and 8 samples; these four kernels take about 90.)
+__global__ void __launch_bounds__(kBlock) k_mlp_l3_pz(int n, int batch, const __nv_bfloat16* __restrict__ W,
+                                                     const float* __restrict__ a2, float2* __restrict__ pz) {
+    __shared__ float2 w[kHid];
+    if (threadIdx.x < kHid)
+        w[threadIdx.x] = make_float2(__bfloat162float(W[threadIdx.x]), __bfloat162float(W[kHid + threadIdx.x]));
+    __syncthreads();
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= (int64_t)n * batch) return;
+    const float* ab = a2 + (size_t)(t / n) * kHid * n + t % n;
+    float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll 16
+    for (int f = 0; f < kHid; ++f) {
+        const float v = fmaxf(ab[(size_t)f * n], 0.0f);
+        s.x += w[f].x * v;
+        s.y += w[f].y * v;
+    }
+    pz[t] = s;
+}
+
+// a3 from p and z, g3 = dL/da3 = 2 (a3 - clip((t - q)/s_q)) / (n * batch); loss partials per block
+__global__ void __launch_bounds__(kBlock) k_mlp_loss(int n, int batch, const int32_t* __restrict__ rowptr,
+                                                   const int32_t* __restrict__ col, const float* __restrict__ bias,
+                                                   const float2* __restrict__ pz, const double* __restrict__ q,
+                                                   const double* __restrict__ tgt, const float* __restrict__ scale,
+                                                   float* __restrict__ g3, double* __restrict__ partials,
+                                                   unsigned int* ticket, float* __restrict__ loss) {
     double acc[1] = {0.0};
     const int64_t total = (int64_t)n * batch;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(t / n);
+        const int b = (int)(t / n), i = (int)(t % n);
+        float z = 0.0f;
+        int deg = 0;
+        for (int e = rowptr[i]; e < rowptr[i + 1]; ++e) {
+            const int j = col[e];
+            if (j == i) continue;
+            ++deg;
+            z += pz[(size_t)b * n + j].y;
+        }
+        const float out = bias[0] + pz[t].x + z * (deg ? 1.0f / deg : 0.0f);
         const double tn = fmin(fmax((tgt[t] - q[t]) / (double)scale[2 * b + 1], -kTargetClip), kTargetClip);
-        const double d = (double)out[t] - tn;
+        const double d = (double)out - tn;
         acc[0] += d * d;
         g3[t] = (float)(2.0 * d / (double)total);
     }
@@ -288,136 +385,280 @@ __global__ void __launch_bounds__(kBlock) k_mlp_loss(int n, int batch, const dou
     if (grid_sum<1>(acc, partials, ticket, tot) && threadIdx.x == 0) *loss = (float)(tot[0] / (double)total);
 }
 
-// gx = W^T ga: gh (the h part, k < FIN) and gm (the mean part)
+// (g3_j, S_j) per vertex and g2 = dL/da2 = (W3h g3 + W3m S) where a2 > 0
+__global__ void __launch_bounds__(kBlock) k_mlp_l3_bwd(int n, int batch, const int32_t* __restrict__ rowptr,
+                                                      const int32_t* __restrict__ col,
+                                                      const __nv_bfloat16* __restrict__ W, const float* __restrict__ g3,
+                                                      const float* __restrict__ a2, float2* __restrict__ gs,
+                                                      float* __restrict__ g2) {
+    __shared__ float2 w[kHid];
+    if (threadIdx.x < kHid)
+        w[threadIdx.x] = make_float2(__bfloat162float(W[threadIdx.x]), __bfloat162float(W[kHid + threadIdx.x]));
+    __syncthreads();
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= (int64_t)n * batch) return;
+    const int b = (int)(t / n), j = (int)(t % n);
+    const float g = g3[t];
+    float s = 0.0f;
+    for (int e = rowptr[j]; e < rowptr[j + 1]; ++e) {
+        const int i = col[e];
+        if (i != j) s += g3[(size_t)b * n + i] * (1.0f / (float)(rowptr[i + 1] - rowptr[i] - 1));
+    }
+    gs[t] = make_float2(g, s);
+    const size_t at = (size_t)b * kHid * n + j;
+#pragma unroll 16
+    for (int f = 0; f < kHid; ++f) {
+        const size_t x = at + (size_t)f * n;
+        g2[x] = a2[x] > 0.0f ? w[f].x * g + w[f].y * s : 0.0f;
+    }
+}
+
+// per-block partials of dW3h, dW3m, db3: blocks of kRowsPerBlock vertices of one sample; a warp
+// takes every eighth feature, its lanes the vertices
+constexpr int kRowsPerBlock = 1024;
+
+__global__ void __launch_bounds__(256) k_mlp_wgrad3(int n, const float2* __restrict__ gs, const float* __restrict__ a2,
+                                                   float* __restrict__ partials) {
+    __shared__ float2 g[kRowsPerBlock];
+    const int b = blockIdx.y, i0 = blockIdx.x * kRowsPerBlock, cnt = min(kRowsPerBlock, n - i0);
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r = threadIdx.x; r < kRowsPerBlock; r += 256)
+        g[r] = r < cnt ? gs[(size_t)b * n + i0 + r] : make_float2(0.0f, 0.0f);
+    __syncthreads();
+    float* out = partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (2 * kHid + 1);
+    for (int f = wid; f < kHid; f += 8) {
+        const float* ab = a2 + ((size_t)b * kHid + f) * n + i0;
+        float s0 = 0.0f, s1 = 0.0f;
+#pragma unroll 8
+        for (int r = lane; r < kRowsPerBlock; r += 32) {
+            const float v = r < cnt ? fmaxf(ab[r], 0.0f) : 0.0f;
+            s0 += g[r].x * v;
+            s1 += g[r].y * v;
+        }
+        s0 = warp_sum(s0);
+        s1 = warp_sum(s1);
+        if (lane == 0) {
+            out[f] = s0;
+            out[kHid + f] = s1;
+        }
+    }
+    if (wid == 0) {
+        float s = 0.0f;
+        for (int r = lane; r < kRowsPerBlock; r += 32) s += g[r].x;
+        s = warp_sum(s);
+        if (lane == 0) out[2 * kHid] = s;
+    }
+}
+
+// per-block partials of layer 1's 64 x 8 weight gradient and bias, same blocks: the 8 inputs in
+// shared memory, a warp takes 8 outputs in two groups of 4, so an input read feeds 4 FMAs
+__global__ void __launch_bounds__(256) k_mlp_wgrad1(int n, const float* __restrict__ ga, const float* __restrict__ h,
+                                                   const float* __restrict__ m, float* __restrict__ partials) {
+    __shared__ float x[8][kRowsPerBlock];
+    const int b = blockIdx.y, i0 = blockIdx.x * kRowsPerBlock, cnt = min(kRowsPerBlock, n - i0);
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int e = threadIdx.x; e < 8 * kRowsPerBlock; e += 256) {
+        const int k = e / kRowsPerBlock, r = e % kRowsPerBlock;
+        const float* src = (k < 4 ? h : m) + ((size_t)b * 4 + (k & 3)) * n + i0;
+        x[k][r] = r < cnt ? src[r] : 0.0f;
+    }
+    __syncthreads();
+    float* out = partials + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * (kHid * 9);
+    for (int o0 = 4 * wid; o0 < kHid; o0 += 32) {
+        float s[4][9];
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) s[o][k] = 0.0f;
+        const float* gb = ga + ((size_t)b * kHid + o0) * n + i0;
+#pragma unroll 4
+        for (int r = lane; r < kRowsPerBlock; r += 32) {
+            float g[4];
+#pragma unroll
+            for (int o = 0; o < 4; ++o) g[o] = r < cnt ? gb[(size_t)o * n + r] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float v = x[k][r];
+#pragma unroll
+                for (int o = 0; o < 4; ++o) s[o][k] += g[o] * v;
+            }
+#pragma unroll
+            for (int o = 0; o < 4; ++o) s[o][8] += g[o];
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const float t = warp_sum(s[o][k]);
+                if (lane == 0) out[(o0 + o) * 9 + k] = t;
+            }
+    }
+}
+
+// gx = W^T ga: gh (the h part, k < FIN; feature-major) and gv (the mean part divided by the
+// vertex's degree, vertex-major, for k_mlp_nmean64_bwd).  Two vertices per thread, so a weight
+// read from shared memory feeds two FMAs.
 template <int FIN, int FOUT>
-__global__ void __launch_bounds__(128) k_mlp_dense_bwd(int n, int batch, const __nv_bfloat16* __restrict__ W,
+__global__ void __launch_bounds__(128) k_mlp_dense_bwd(int n, int batch, const int32_t* __restrict__ rowptr,
+                                                       const __nv_bfloat16* __restrict__ W,
                                                        const float* __restrict__ ga, float* __restrict__ gh,
-                                                       float* __restrict__ gm) {
-    constexpr int K = 2 * FIN;
-    __shared__ float w[K][FOUT];
+                                                       float* __restrict__ gv) {
+    constexpr int K = 2 * FIN, V = 2, KC = 4;
+    static_assert(FIN % KC == 0, "whole chunks");
+    __shared__ __align__(16) float w[K][FOUT];
     for (int e = threadIdx.x; e < K * FOUT; e += blockDim.x) {
         const int o = e / K, k = e % K;
         w[k][o] = __bfloat162float(W[e]);
     }
     __syncthreads();
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n * batch) return;
-    const int b = (int)(t / n), i = (int)(t % n);
-    const float* gab = ga + (size_t)b * FOUT * n;
-    float g[FOUT];
+    int b[V], i[V];
+    bool in[V];
+    float inv[V], g[V][FOUT];
 #pragma unroll
-    for (int o = 0; o < FOUT; ++o) g[o] = gab[(size_t)o * n + i];
-    float* ghb = gh + (size_t)b * FIN * n;
-    float* gmb = gm + (size_t)b * FIN * n;
-    for (int k = 0; k < K; ++k) {
-        float s = 0.0f;
+    for (int v = 0; v < V; ++v) {
+        const int64_t t = blockIdx.x * (int64_t)(128 * V) + threadIdx.x + 128 * v;
+        in[v] = t < (int64_t)n * batch;
+        b[v] = in[v] ? (int)(t / n) : 0;
+        i[v] = in[v] ? (int)(t % n) : 0;
+        inv[v] = 1.0f / (float)(rowptr[i[v] + 1] - rowptr[i[v]] - 1);
 #pragma unroll
-        for (int o = 0; o < FOUT; ++o) s += w[k][o] * g[o];
-        if (k < FIN) ghb[(size_t)k * n + i] = s;
-        else gmb[(size_t)(k - FIN) * n + i] = s;
+        for (int o = 0; o < FOUT; ++o) g[v][o] = ga[((size_t)b[v] * FOUT + o) * n + i[v]];
+    }
+    for (int k0 = 0; k0 < K; k0 += KC) {
+        float s[V][KC];
+#pragma unroll
+        for (int u = 0; u < KC; ++u) {
+#pragma unroll
+            for (int v = 0; v < V; ++v) s[v][u] = 0.0f;
+#pragma unroll
+            for (int o = 0; o < FOUT; ++o) {
+                const float wv = w[k0 + u][o];
+#pragma unroll
+                for (int v = 0; v < V; ++v) s[v][u] += wv * g[v][o];
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            if (!in[v]) continue;
+            if (k0 < FIN) {
+#pragma unroll
+                for (int u = 0; u < KC; ++u) gh[((size_t)b[v] * FIN + k0 + u) * n + i[v]] = s[v][u];
+            } else {
+                *reinterpret_cast<float4*>(gv + ((size_t)b[v] * n + i[v]) * FIN + (k0 - FIN)) =
+                    make_float4(s[v][0] * inv[v], s[v][1] * inv[v], s[v][2] * inv[v], s[v][3] * inv[v]);
+            }
+        }
     }
 }
 
-// gh[j] += sum over neighbours i of j (i != j) of gm[i] / deg(i); then ga = gh * (a > 0)
-template <int F>
-__global__ void k_mlp_nmean_bwd(int n, int batch, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                                const float* __restrict__ gm, const float* __restrict__ a_prev, float* __restrict__ gh) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= (int64_t)n * batch) return;
-    const int b = (int)(t / n), j = (int)(t % n);
-    const float* gmb = gm + (size_t)b * F * n;
-    float* ghb = gh + (size_t)b * F * n;
-    const float* ab = a_prev + (size_t)b * F * n;
-    float acc[F];
-#pragma unroll
-    for (int f = 0; f < F; ++f) acc[f] = ghb[(size_t)f * n + j];
-    for (int e = rowptr[j]; e < rowptr[j + 1]; ++e) {
-        const int i = col[e];
-        if (i == j) continue;
-        const float inv = 1.0f / (float)(rowptr[i + 1] - rowptr[i] - 1);
-#pragma unroll
-        for (int f = 0; f < F; ++f) acc[f] += gmb[(size_t)f * n + i] * inv;
-    }
-#pragma unroll
-    for (int f = 0; f < F; ++f) ghb[(size_t)f * n + j] = ab[(size_t)f * n + j] > 0.0f ? acc[f] : 0.0f;
-}
-
-// Per-block partial weight gradients: dW[o][k] = sum_rows ga[o] x[k], db[o] = sum ga[o],
-// x = [act(h); m].  Rows = (sample, vertex) pairs; block c takes rows [c*kRowsPerBlock, ...).
-constexpr int kRowsPerBlock = 1024;
+// Weight gradients are reduced in two deterministic passes: per-block partials [block][o][k]
+// (k = 2 FIN: the bias), then a fixed-order sum in FP64.
 constexpr int kTile = 32;
 
-template <int FIN, int FOUT, bool RELU_IN>
-__global__ void __launch_bounds__(256) k_mlp_wgrad(int n, int batch, const float* __restrict__ ga,
-                                                   const float* __restrict__ h, const float* __restrict__ m,
-                                                   float* __restrict__ partials) {
-    constexpr int K = 2 * FIN;
-    constexpr int NOUT = FOUT * (K + 1);
-    constexpr int PER = (NOUT + 255) / 256;
-    __shared__ float gt[FOUT][kTile + 1];
-    __shared__ float xt[K][kTile + 1];
-    float acc[PER];
+// The 64 x 128 weight gradient of layer 2 (and its bias) as a register-tiled product: 256
+// threads hold 8 x 4 outputs each (o = og + 8 j, k = kg + 32 j), so 12 16-byte shared-memory
+// reads feed 128 FMAs; at most kWgradBlocks CTAs, two per SM.  Sums of 32 rows are added to the
+// running ones, which keeps the rounding of a two-level sum.
+constexpr int kWgradBlocks = 304;
+
+inline int wgrad64_rows(int64_t rows) {   // rows per CTA, whole tiles
+    const int64_t r = (rows + kWgradBlocks - 1) / kWgradBlocks;
+    return (int)((r + kTile - 1) / kTile * kTile);
+}
+
+__global__ void __launch_bounds__(256, 2) k_mlp_wgrad64(int n, int batch, int rows, const float* __restrict__ ga,
+                                                       const float* __restrict__ h, const float* __restrict__ m,
+                                                       float* __restrict__ partials) {
+    constexpr int K = 2 * kHid, LD = kTile + 4;   // 16-byte rows on distinct banks
+    __shared__ __align__(16) float gt[kHid][LD];
+    __shared__ __align__(16) float xt[K][LD];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int og = lane & 7, kg = 4 * wid + (lane >> 3);
+    float acc[8][4], accb[8];
 #pragma unroll
-    for (int u = 0; u < PER; ++u) acc[u] = 0.0f;
-    const int64_t total = (int64_t)n * batch;
-    const int64_t r0 = (int64_t)blockIdx.x * kRowsPerBlock;
-    for (int64_t rt = r0; rt < r0 + kRowsPerBlock && rt < total; rt += kTile) {
-        // stage a tile of rows
-        for (int e = threadIdx.x; e < (FOUT + K) * kTile; e += blockDim.x) {
-            const int f = e / kTile, rr = e % kTile;
-            const int64_t row = rt + rr;
-            float v = 0.0f;
-            if (row < total) {
-                const int b = (int)(row / n), i = (int)(row % n);
-                if (f < FOUT) {
-                    v = ga[((size_t)b * FOUT + f) * n + i];
-                } else {
-                    const int k = f - FOUT;
-                    if (k < FIN) {
-                        v = h[((size_t)b * FIN + k) * n + i];
-                        if (RELU_IN) v = fmaxf(v, 0.0f);
-                    } else {
-                        v = m[((size_t)b * FIN + (k - FIN)) * n + i];
-                    }
-                }
-            }
-            if (f < FOUT) gt[f][rr] = v;
-            else xt[f - FOUT][rr] = v;
-        }
-        __syncthreads();
+    for (int j = 0; j < 8; ++j) {
+        accb[j] = 0.0f;
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int qi = threadIdx.x + 256 * u;
-            if (qi < NOUT) {
-                const int o = qi / (K + 1), k = qi % (K + 1);
-                float s = 0.0f;
-                if (k < K) {
-#pragma unroll 8
-                    for (int rr = 0; rr < kTile; ++rr) s += gt[o][rr] * xt[k][rr];
-                } else {
-#pragma unroll 8
-                    for (int rr = 0; rr < kTile; ++rr) s += gt[o][rr];
-                }
-                acc[u] += s;
-            }
-        }
-        __syncthreads();
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
     }
+    const int64_t total = (int64_t)n * batch, r0 = (int64_t)blockIdx.x * rows;
+    for (int64_t rt = r0; rt < r0 + rows && rt < total; rt += kTile) {
+        const int64_t row = rt + lane;
+        const bool in = row < total;
+        const int b = in ? (int)(row / n) : 0, i = in ? (int)(row % n) : 0;
+        const size_t at = (size_t)b * kHid * n + i;
+        float v[24];
 #pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int qi = threadIdx.x + 256 * u;
-        if (qi < NOUT) partials[(size_t)blockIdx.x * NOUT + qi] = acc[u];
+        for (int u = 0; u < 24; ++u) {
+            const int f = wid + 8 * u;   // 0..63: ga, 64..127: h, 128..191: m
+            const float* src = u < 8 ? ga : (u < 16 ? h : m);
+            v[u] = in ? src[at + (size_t)(f & (kHid - 1)) * n] : 0.0f;
+        }
+        __syncthreads();   // the previous tile is consumed
+#pragma unroll
+        for (int u = 0; u < 24; ++u) {
+            const int f = wid + 8 * u;
+            if (u < 8) gt[f][lane] = v[u];
+            else xt[f - kHid][lane] = u < 16 ? fmaxf(v[u], 0.0f) : v[u];
+        }
+        __syncthreads();
+        float s[8][4], sb[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            sb[j] = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[j][q] = 0.0f;
+        }
+#pragma unroll 1
+        for (int r = 0; r < kTile; r += 4) {
+            float4 x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = *reinterpret_cast<const float4*>(&xt[kg + 32 * q][r]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float4 g = *reinterpret_cast<const float4*>(&gt[og + 8 * j][r]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    s[j][q] += g.x * x[q].x;
+                    s[j][q] += g.y * x[q].y;
+                    s[j][q] += g.z * x[q].z;
+                    s[j][q] += g.w * x[q].w;
+                }
+                if (wid == 0) sb[j] += (g.x + g.y) + (g.z + g.w);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            accb[j] += sb[j];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[j][q] += s[j][q];
+        }
+    }
+    float* out = partials + (size_t)blockIdx.x * kHid * (K + 1);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int o = og + 8 * j;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) out[o * (K + 1) + kg + 32 * q] = acc[j][q];
+        if (kg == 0) out[o * (K + 1) + K] = accb[j];
     }
 }
 
 // grad[W offset + o*K + k] / grad[b offset + o] = sum over blocks (fixed order) of the partials
-__global__ void k_mlp_wgrad_reduce(int nblk, int fout, int K, const float* __restrict__ partials,
-                                   float* __restrict__ gW, float* __restrict__ gb) {
-    const int nout = fout * (K + 1);
-    const int qi = blockIdx.x * blockDim.x + threadIdx.x;
-    if (qi >= nout) return;
+// (eight threads per output take every eighth block, then their sums are added in order)
+__global__ void __launch_bounds__(256) k_mlp_wgrad_reduce(int nblk, int fout, int K, const float* __restrict__ partials,
+                                                         float* __restrict__ gW, float* __restrict__ gb) {
+    __shared__ double part[8][32];
+    const int nout = fout * (K + 1), lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+    const int qi = blockIdx.x * 32 + lane;
     double s = 0.0;
-    for (int c = 0; c < nblk; ++c) s += partials[(size_t)c * nout + qi];
+    if (qi < nout)
+#pragma unroll 4
+        for (int c = grp; c < nblk; c += 8) s += partials[(size_t)c * nout + qi];
+    part[grp][lane] = s;
+    __syncthreads();
+    if (grp || qi >= nout) return;
+    for (int k = 1; k < 8; ++k) s += part[k][lane];
     const int o = qi / (K + 1), k = qi % (K + 1);
     if (k < K) gW[o * K + k] = (float)s;
     else gb[o] = (float)s;
@@ -471,14 +712,14 @@ void MlpBuffers::carve(Carve& cv, int n_, int batch) {
     params = cv.take<float>(kMlpParams);
 }
 
-// the training forward pass: every activation kept (feature-major) for mlp_backward
+// the training forward pass up to layer 3's (p, z) (in B.m2): every activation kept
+// (feature-major) for mlp_backward
 static int mlp_forward_train(const MlpBuffers& B, const Level& L, const double* r, const double* q, int batch,
-                             double* pred, cudaStream_t st) {
+                             cudaStream_t st) {
     const int n = B.n;
     const int64_t nb = (int64_t)n * batch;
     const int g = blocks_for(nb);
     const int gh = blocks_for(nb, dense_vertices_per_block<kHid>());
-    const int g1 = blocks_for(nb, dense_vertices_per_block<1>());
     k_mlp_scales<<<dim3(kScaleBlocks, batch), kBlock, 0, st>>>(n, r, q, B.spart);
     k_mlp_scales_fin<<<batch, 32, 0, st>>>(n, kScaleBlocks, B.spart, B.scale);
     k_mlp_features<<<g, kBlock, 0, st>>>(n, batch, r, q, L.xy, B.scale, B.h0);
@@ -487,12 +728,9 @@ static int mlp_forward_train(const MlpBuffers& B, const Level& L, const double* 
                                                            B.m0, B.a1, B.hv);
     const dim3 gm((n + 31) / 32, batch);
     k_mlp_nmean64<<<gm, 256, 0, st>>>(n, L.rowptr, L.col, B.hv, B.m1);
-    k_mlp_dense<kHid, kHid, true, true><<<gh, 128, 0, st>>>(n, batch, B.params_bf + kOffW2, B.params + kOffB2, B.a1,
-                                                             B.m1, B.a2, B.hv);
-    k_mlp_nmean64<<<gm, 256, 0, st>>>(n, L.rowptr, L.col, B.hv, B.m2);
-    k_mlp_dense<kHid, 1, true, false><<<g1, 128, 0, st>>>(n, batch, B.params_bf + kOffW3, B.params + kOffB3, B.a2,
-                                                           B.m2, B.out, nullptr);
-    if (pred) k_mlp_predict<<<g, kBlock, 0, st>>>(n, batch, q, B.out, B.scale, pred);
+    k_mlp_dense<kHid, kHid, true, false><<<gh, 128, 0, st>>>(n, batch, B.params_bf + kOffW2, B.params + kOffB2, B.a1,
+                                                              B.m1, B.a2, nullptr);
+    k_mlp_l3_pz<<<g, kBlock, 0, st>>>(n, batch, B.params_bf + kOffW3, B.a2, reinterpret_cast<float2*>(B.m2));
     CGP_LAUNCH_CHECK();
     return CGP_OK;
 }
@@ -511,7 +749,6 @@ struct cgp_mlp {
     double* partials = nullptr;
     unsigned int* ticket = nullptr;
     int adam_t = 0;
-    int nblk = 0;
 };
 
 extern "C" int cgp_mlp_param_count(void) { return kMlpParams; }
@@ -528,13 +765,13 @@ extern "C" int cgp_mlp_create(const cgp_mesh* mesh, int32_t level, int32_t max_b
     m->level = level;
     const int n = mesh->lev[level].nv;
     const int64_t nb = (int64_t)n * max_batch;
-    m->nblk = (int)((nb + kRowsPerBlock - 1) / kRowsPerBlock);
+    const size_t nblk = (size_t)((n + kRowsPerBlock - 1) / kRowsPerBlock) * max_batch;   // blocks of layers 1 and 3
     auto layout = [&](Carve& cv) {
         m->B.carve(cv, n, max_batch);
         m->grad = cv.take<float>(kMlpParams);
         m->adam_m = cv.take<float>(kMlpParams);
         m->adam_v = cv.take<float>(kMlpParams);
-        m->wpart = cv.take<float>((size_t)m->nblk * kHid * (2 * kHid + 1));
+        m->wpart = cv.take<float>(std::max((size_t)kWgradBlocks * kHid * (2 * kHid + 1), nblk * kHid * 9));
         m->gA = cv.take<float>(kHid * nb);
         m->gB = cv.take<float>(kHid * nb);
         m->gM = cv.take<float>(kHid * nb);
@@ -647,28 +884,32 @@ static int mlp_backward(cgp_mlp* m, const double* r, const double* q, const doub
     MlpBuffers& B = m->B;
     const int n = B.n;
     const int64_t nb = (int64_t)n * batch;
-    CGP_TRY(mlp_forward_train(B, L, r, q, batch, nullptr, st));
-    const int g = blocks_for(nb), g128 = blocks_for(nb, 128);
-    const int nblk = (int)((nb + kRowsPerBlock - 1) / kRowsPerBlock);
+    CGP_TRY(mlp_forward_train(B, L, r, q, batch, st));
+    const int g = blocks_for(nb), g256 = blocks_for(nb, 256);   // two vertices per thread of 128
+    const dim3 gm((n + 31) / 32, batch), gw((n + kRowsPerBlock - 1) / kRowsPerBlock, batch);
+    const int rows64 = wgrad64_rows(nb), nblk64 = (int)((nb + rows64 - 1) / rows64);
+    const int nblk = (int)(gw.x * gw.y);
     int gl = (int)(nb / kBlock + 1);
     if (gl > 1024) gl = 1024;
-    k_mlp_loss<<<gl, kBlock, 0, st>>>(n, batch, q, tgt, B.out, B.scale, m->g3, m->partials, m->ticket, m->loss);
-    // layer 3: dW3, db3; gh2 (direct) and gm2
-    k_mlp_wgrad<kHid, 1, true><<<nblk, 256, 0, st>>>(n, batch, m->g3, B.a2, B.m2, m->wpart);
-    k_mlp_wgrad_reduce<<<blocks_for(2 * kHid + 1), kBlock, 0, st>>>(nblk, 1, 2 * kHid, m->wpart, m->grad + kOffW3,
-                                                                   m->grad + kOffB3);
-    k_mlp_dense_bwd<kHid, 1><<<g128, 128, 0, st>>>(n, batch, B.params_bf + kOffW3, m->g3, m->gA, m->gM);
-    k_mlp_nmean_bwd<kHid><<<g, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, m->gM, B.a2, m->gA);   // gA = dL/da2
+    const float2* pz = reinterpret_cast<const float2*>(B.m2);
+    float2* gs = reinterpret_cast<float2*>(m->gM);   // free until layer 2's mean part
+    k_mlp_loss<<<gl, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, B.params + kOffB3, pz, q, tgt, B.scale, m->g3,
+                                      m->partials, m->ticket, m->loss);
+    // layer 3: gA = dL/da2, then dW3, db3
+    k_mlp_l3_bwd<<<g, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, B.params_bf + kOffW3, m->g3, B.a2, gs, m->gA);
+    k_mlp_wgrad3<<<gw, 256, 0, st>>>(n, gs, B.a2, m->wpart);
+    k_mlp_wgrad_reduce<<<blocks_for(2 * kHid + 1, 32), 256, 0, st>>>(nblk, 1, 2 * kHid, m->wpart, m->grad + kOffW3,
+                                                                    m->grad + kOffB3);
     // layer 2
-    k_mlp_wgrad<kHid, kHid, true><<<nblk, 256, 0, st>>>(n, batch, m->gA, B.a1, B.m1, m->wpart);
-    k_mlp_wgrad_reduce<<<blocks_for(kHid * (2 * kHid + 1)), kBlock, 0, st>>>(nblk, kHid, 2 * kHid, m->wpart,
-                                                                            m->grad + kOffW2, m->grad + kOffB2);
-    k_mlp_dense_bwd<kHid, kHid><<<g128, 128, 0, st>>>(n, batch, B.params_bf + kOffW2, m->gA, m->gB, m->gM);
-    k_mlp_nmean_bwd<kHid><<<g, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, m->gM, B.a1, m->gB);   // gB = dL/da1
+    k_mlp_wgrad64<<<nblk64, 256, 0, st>>>(n, batch, rows64, m->gA, B.a1, B.m1, m->wpart);
+    k_mlp_wgrad_reduce<<<blocks_for(kHid * (2 * kHid + 1), 32), 256, 0, st>>>(nblk64, kHid, 2 * kHid, m->wpart,
+                                                                             m->grad + kOffW2, m->grad + kOffB2);
+    k_mlp_dense_bwd<kHid, kHid><<<g256, 128, 0, st>>>(n, batch, L.rowptr, B.params_bf + kOffW2, m->gA, m->gB, m->gM);
+    k_mlp_nmean64_bwd<<<gm, 256, 0, st>>>(n, L.rowptr, L.col, m->gM, B.a1, m->gB);   // gB = dL/da1
     // layer 1
-    k_mlp_wgrad<4, kHid, false><<<nblk, 256, 0, st>>>(n, batch, m->gB, B.h0, B.m0, m->wpart);
-    k_mlp_wgrad_reduce<<<blocks_for(kHid * 9), kBlock, 0, st>>>(nblk, kHid, 8, m->wpart, m->grad + kOffW1,
-                                                               m->grad + kOffB1);
+    k_mlp_wgrad1<<<gw, 256, 0, st>>>(n, m->gB, B.h0, B.m0, m->wpart);
+    k_mlp_wgrad_reduce<<<blocks_for(kHid * 9, 32), 256, 0, st>>>(nblk, kHid, 8, m->wpart, m->grad + kOffW1,
+                                                                m->grad + kOffB1);
     CGP_LAUNCH_CHECK();
     return CGP_OK;
 }
