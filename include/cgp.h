@@ -128,9 +128,11 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * (a variant, not in the paper): Jacobi plus an additive subdomain coarse correction,
  * M^{-1} = D^{-1} + Z E^+ Z^T with Z the indicator vectors of up to 128 compact vertex
  * subdomains (phi = 0 vertices in none) and E^+ the pseudo-inverse of E = Z^T K_c Z, built
- * once at cgp_assemble; only the ONCHIP coarse solver has it (cgp_assemble fails with
- * CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs, JACOBI elsewhere.
- * The solution is the same to the solve's tolerance; only the iteration count changes. */
+ * once at cgp_assemble; asked for by name, only the ONCHIP coarse solver has it (cgp_assemble
+ * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs, the same
+ * correction in FP64 (one subdomain per CTA) in the register-resident PERSISTENT solve, JACOBI
+ * elsewhere.  The solution is the same to the solve's tolerance; only the iteration count
+ * changes. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 
 /* Coarse Poisson solver kinds.  KERNELS: two kernel launches per PCG iteration (graph

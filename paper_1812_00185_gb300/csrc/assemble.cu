@@ -4,10 +4,12 @@
 // Assembly is vertex-centric: the thread of row i walks the triangles around vertex i
 // (ascending) and adds each element contribution to the CSR slot of the other corner,
 // so every row is written by one thread and the sums are deterministic (no atomics).
+#include <algorithm>
 #include <cstring>
 
 #include "flows.cuh"
 #include "guess_proj.cuh"
+#include "rr_plan.cuh"
 #include "solver.cuh"
 
 namespace cgp {
@@ -161,7 +163,13 @@ static int layout(Solver& s, void* base, size_t* bytes) {
     s.geoc = cv.take<double>((size_t)7 * C.nt);
     s.Kc0f = cv.take<float>(nnzc);
     s.dinvKcf = cv.take<float>(nc);
-    s.cw64 = cv.take<double>(5 * nc + 386);   // 5 vectors, or the register-resident solve's words (coarse_rr.cuh)
+    s.cw64 = cv.take<double>(5 * nc + 1410);   // 5 vectors, or the register-resident solve's words (coarse_rr.cuh)
+    // its plan: a thread per row of at most one slice more per CTA than the rows need, and E^+
+    if (s.prm.precond == CGP_PRECOND_AUTO) {
+        const size_t ctas = std::min<size_t>(kRRMaxSub, (size_t)C.nslices / 8 + 16);
+        s.rr_perm = cv.take<int32_t>(32 * ((size_t)C.nslices + 16 * ctas));
+        s.rr_einv = cv.take<double>(ctas * ctas);
+    }
     if (s.prm.guess == CGP_GUESS_LEARNED) {
         s.phi_guess = cv.take<double>(nc);
         s.mlp.carve(cv, (int)nc, 1);

@@ -75,6 +75,11 @@ struct CoarsePcgArgs {
     // which the network is not evaluated, gate[1] = consecutive steps in which its direction
     // lowered the starting residual by less than 5 %
     int* gate;
+    // plan of the register-resident FP64 solve (rr_plan.cuh), or null and 0
+    const int32_t* perm;
+    const int32_t* rowptr;
+    const double* einv;
+    int nsub;
 };
 
 template <class T>

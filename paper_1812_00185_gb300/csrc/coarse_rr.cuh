@@ -15,6 +15,15 @@
 // the stagnation window: 10,272 iterations to 1e-10 on the channel's 32,489-row system where
 // this form takes 1,243, and 2,878 against 580 on 129^2 vertices.)
 //
+// With a plan (rr_plan.cuh; the solver's default) the rows go to the CTAs as compact subdomains
+// and the preconditioner is Jacobi plus an additive coarse correction, as in the on-chip solve:
+// M^{-1} = D^{-1} + Z E^+ Z^T with Z the CTAs' indicator vectors and E = Z^T K Z, all in FP64.
+// A CTA's sum of w joins the exchange of the other sums; from them s = Z^T r follows by the
+// recurrence of r itself (s -= alpha (Z^T w + beta Z^T s')), every first CTA forms mu = E^+ s
+// for its cluster and sends it down with alpha and beta, and u = D^{-1} r + mu.  Iterations to
+// 1e-10 fall from 580 to 250 (129^2 rows, 72 subdomains), 1,243 to 251 (the channel's 32,489
+// rows, 128), 1,162 to 348 (257^2, 144).
+//
 // What bounds an iteration is latency: two round trips through L2 and the narrow FP64 pipe
 // (a warp-wide FP64 operation holds an SM's pipe for 16 clocks).  Hence:
 //  * u travels without a barrier: a row's owner stores the 16-byte word {u, generation} (one
@@ -31,57 +40,72 @@
 //  * one warp per cluster forms the scalars: FP64 divides in every thread cost more than the
 //    SpMV.  Their divides come down to one reciprocal with two Newton steps, and the checks
 //    (finite, converged, stagnating) compare bit patterns on the integer pipe.
-// Measured (GB300): 3,872 rows, one cluster of 16: 4.6 us an iteration (every CTA polling all:
-// 7.4); 129^2 rows, 9 clusters of 8: 7.0 us, 4.1 ms to 1e-10 (7.8; the pipelined kernel with a
-// counting barrier, shuffles and divides in every thread: 14-25 ms a solve); 66,049 rows, 15
-// warps a CTA: 10.7 us (vectors in memory: 17.4 us).  Of the 14k clocks of the 129^2 case the
-// gather takes 3.4k, the words between clusters 4.6k, the sums and scalars 4k.
+// Measured (GB300): 3,872 rows, one cluster of 16, Jacobi: 4.6 us an iteration (every CTA
+// polling all: 7.4).  129^2 rows, 9 clusters of 8, to 1e-10: 2.4 ms with the plan, 4.1 ms with
+// Jacobi alone, 7.0 us an iteration (14-25 ms: the pipelined kernel with a counting barrier,
+// shuffles and divides in every thread).  66,049 rows, 37 clusters of 4: 348 iterations of
+// 13 us (1,217 of 10 us in memory with Jacobi, 17 us in the pipelined form).  Of the 14k
+// clocks of the 129^2 case with Jacobi the gather takes 3.4k, the words between clusters 4.6k,
+// the sums and scalars 4k.
 // Every cluster adds the partials in the same order, so all CTAs hold identical scalars.
 // Every poll is bounded: after a limit the reader marks its sums as failed, sets the error
 // word, and all CTAs leave with CGP_ETIMEOUT.
 #pragma once
 
 #include "coarse_pcg.cuh"
+#include "rr_plan.cuh"
 
 namespace cgp {
 
 constexpr int kRRWidth = 8;          // entries of a row held in registers
 constexpr int kRRMaxWarps = 16;      // warps (slices) per CTA: 512 threads of up to 128 registers
 constexpr int kRRMinWarps = 4;       // the reductions use three warps
-constexpr int kRRCluster = 8;        // CTAs per cluster of a launch of several clusters
+constexpr int kRRCluster = 8;        // CTAs per cluster of a launch of several clusters: 8, or 4
 constexpr int kRRSingle = 16;        // CTAs of a launch of one cluster (small systems)
-constexpr int kRRMaxClusters = 32;   // clusters of a launch: one polled word per lane
+constexpr int kRRMaxClusters = 64;   // clusters of a launch: two polled words per lane
 
 struct RRShape {
     int ctas = 0, cluster = 0, warps = 0;   // ctas = 0: the system does not fit
 };
 
-// Launch for nslices slices where `single` (0 or 1) clusters of kRRSingle and `multi` clusters
-// of kRRCluster CTAs of the largest size are co-resident: one cluster up to 8 slices per CTA
-// (no exchange through L2 in the sums), else as few warps per CTA as the clusters allow, at
-// least 8 (fewer CTAs, fewer words).
-inline RRShape rr_shape(int nslices, int single, int multi) {
+// co-resident clusters of the largest CTAs: one of kRRSingle CTAs or none; of 8; of 4
+struct RRCapacity {
+    int single = 0, eight = 0, four = 0;
+};
+
+// Launch for nslices slices: one cluster up to 8 slices per CTA (no exchange through L2 in the
+// sums); else clusters of 8 with as few warps per CTA as they allow, at least 8 (fewer CTAs,
+// fewer words); where 16 warps per CTA do not do (fewer clusters of 8 than SMs / 8 fit the
+// GPCs), clusters of 4.
+inline RRShape rr_shape(int nslices, const RRCapacity& cap) {
     RRShape s;
-    if (single > 0 && nslices <= 8 * kRRSingle) {
+    if (cap.single > 0 && nslices <= 8 * kRRSingle) {
         s.cluster = s.ctas = kRRSingle;
         s.warps = (nslices + kRRSingle - 1) / kRRSingle;
         if (s.warps < kRRMinWarps) s.warps = kRRMinWarps;
         return s;
     }
-    if (multi > kRRMaxClusters) multi = kRRMaxClusters;
-    if (multi < 1) return s;
-    s.warps = (nslices + kRRCluster * multi - 1) / (kRRCluster * multi);
-    if (s.warps < 8) s.warps = 8;
-    if (s.warps > kRRMaxWarps) return RRShape{};
-    const int need = (nslices + s.warps - 1) / s.warps;
-    s.cluster = kRRCluster;
-    s.ctas = (need + kRRCluster - 1) / kRRCluster * kRRCluster;
+    for (int size : {kRRCluster, kRRCluster / 2}) {
+        int fit = size == kRRCluster ? cap.eight : cap.four;
+        if (fit > kRRMaxClusters) fit = kRRMaxClusters;
+        if (fit > kRRMaxSub / size) fit = kRRMaxSub / size;
+        if (fit < 1) continue;
+        int w = (nslices + size * fit - 1) / (size * fit);
+        if (w < 8) w = 8;
+        if (w > kRRMaxWarps) continue;
+        const int need = (nslices + w - 1) / w;
+        s.warps = w;
+        s.cluster = size;
+        s.ctas = (need + size - 1) / size * size;
+        return s;
+    }
     return s;
 }
 
-// Work area (doubles): words [2][3][kRRMaxClusters], the error word (2 doubles), u words [n].
-// Zeroed before every launch: generation 0 is never awaited.
-constexpr size_t kRRHead = 12 * (size_t)kRRMaxClusters + 2;
+// Work area (doubles): words [2][3][kRRMaxClusters], words of the CTAs' Z^T w [2][kRRMaxSub], the
+// error word (2 doubles), u words [n].  Zeroed before every launch: generation 0 is never awaited.
+constexpr size_t kRRZWords = 12 * (size_t)kRRMaxClusters;
+constexpr size_t kRRHead = kRRZWords + 4 * (size_t)kRRMaxSub + 2;
 inline size_t rr_work_doubles(int n) { return kRRHead + 2 * (size_t)n; }
 
 // one 16-byte {value, tag} word, single-copy atomic, at L2
@@ -142,17 +166,25 @@ __device__ __forceinline__ double newton_quotient(double n, double d) {
 }
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
+constexpr int kRREinvMax = kRRCluster * kRRMaxSub;   // and kRRSingle^2 is less
+static_assert(kRRSingle * kRRSingle <= kRREinvMax, "rows of E^+ of one cluster");
+
+enum RRCorrection { kRRNone, kRRStart, kRRAdvance };   // reduce: what becomes of s = Z^T r
+
 struct RRWord {
     double v;
     unsigned long long tag;
 };
 
 struct RRShared {
-    double part[3][kRRMaxWarps * 32];
-    RRWord up[2][3][kRRSingle];     // first CTA of the cluster: the CTAs' sums {sum, 1 if not valid}
-    RRWord down[2][3];              // {out0, out1 as bits}, {out2, out3}, {valid, -}
-    double tot[3];
-    int ok[3];
+    double part[4][kRRMaxWarps * 32];
+    RRWord up[2][4][kRRSingle];     // first CTA of the cluster: the CTAs' sums {sum, 1 if not valid}
+    RRWord down[2][3];              // {out0, out1 as bits}, {out2, out3}, {mu, 1 if valid}
+    double tot[3], ab[2];
+    int ok[4], valid;
+    // first CTA of the cluster, with a plan: Z^T w as received, s = Z^T r and Z^T s' (alternating),
+    // and the rows of E^+ of the cluster's CTAs
+    double zt[kRRMaxSub], zs[2][kRRMaxSub], zq[2][kRRMaxSub], einv[kRREinvMax];
     uint64_t up_bar[2], down_bar[2];
 };
 
@@ -166,11 +198,11 @@ struct RRSync {
     long long cycles;
     int test;                               // 1 under the wait test hook: the first CTA of every
                                             // cluster also awaits 16 bytes that nothing sends
-    int rank, ncl, nclusters, cluster_id;
+    int rank, ncl, nclusters, cluster_id, nsub, zpar = 0;
     uint32_t up_remote, up_bar_remote;      // the first CTA's up[0][0][rank] and up_bar[0]
 
-    __device__ RRSync(RRShared& s, double* w, int* e, int wait_test)
-        : sm(s), words(w), err(e), limit(wait_test ? kSpinLimitTest : kSpinLimit),
+    __device__ RRSync(RRShared& s, double* w, int* e, int wait_test, int nsub_)
+        : sm(s), words(w), err(e), nsub(nsub_), limit(wait_test ? kSpinLimitTest : kSpinLimit),
           cycles(wait_test ? kRRWaitCyclesTest : kRRWaitCycles), test(wait_test ? 1 : 0) {
         cgrp::cluster_group c = cgrp::this_cluster();
         rank = (int)c.block_rank();
@@ -207,14 +239,59 @@ struct RRSync {
         return true;
     }
 
+    // the word's value once it carries this generation (tag: kRRFail set when it never does, or
+    // when its writer's sums are not valid)
+    __device__ double poll_word(const double* w, unsigned long long& tag) const {
+        double v;
+        ld_word(w, v, tag);
+        for (unsigned spins = 0; (tag & ~kRRFail) != gen;) {
+            if (expired(++spins)) {
+                tag = kRRFail;
+                break;
+            }
+            ld_word(w, v, tag);
+        }
+        return v;
+    }
+    // warp 3 of a first CTA: lanes < ncl hold the CTAs' z sums; all nsub of them into sm.zt
+    __device__ void exchange_z(double a, bool ok, int par) {
+        const int lane = threadIdx.x & 31;
+        if (nclusters == 1) {
+            if (lane < ncl) sm.zt[lane] = a;
+        } else {
+            double* base = words + kRRZWords + 2 * (size_t)kRRMaxSub * par;
+            if (lane < ncl) st_word(base + 2 * (cluster_id * ncl + lane), a, ok ? gen : gen | kRRFail);
+            double v[kRRMaxSub / 32];
+            unsigned long long tag[kRRMaxSub / 32];
+#pragma unroll
+            for (int j = 0; j < kRRMaxSub / 32; ++j) {   // all five in flight before the first is awaited
+                tag[j] = gen;
+                v[j] = 0.0;
+                if (lane + 32 * j < nsub) ld_word(base + 2 * (lane + 32 * j), v[j], tag[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < kRRMaxSub / 32; ++j) {
+                if ((tag[j] & ~kRRFail) != gen) v[j] = poll_word(base + 2 * (lane + 32 * j), tag[j]);
+                if (lane + 32 * j < nsub) sm.zt[lane + 32 * j] = v[j];
+                ok = ok && !(tag[j] & kRRFail);
+            }
+            ok = __all_sync(0xffffffffu, ok);
+        }
+        if (lane == 0) sm.ok[3] = ok;
+    }
+
     // Grid-wide sums of (v0, v1, v2), which warp 0 of every cluster's first CTA hands to
     // f(t0, t1, t2, out); every thread gets out[0..3].  `bad`: this thread's values are not
-    // valid.  False (in all threads of the CTA): some wait ran out.
+    // valid.  False (in all threads of the CTA): some wait ran out.  With a plan, z of all
+    // threads of a CTA is added up too: kRRStart takes the sums as s, kRRAdvance as Z^T w of the
+    // coming update s -= alpha (Z^T w + beta Z^T s') (alpha, beta = out[0], out[1]), and mu is
+    // this CTA's entry of E^+ s.
     // A set of slots is rewritten two reductions later, and a CTA gets there only after its
     // first CTA has sent the reduction between, that is, after all contributed to it and so
     // had read what the set held.
     template <class F>
-    __device__ bool reduce(double v0, double v1, double v2, int bad, double (&out)[4], F f) {
+    __device__ bool reduce(double v0, double v1, double v2, double z, RRCorrection corr, int bad, double (&out)[4],
+                           double& mu, F f) {
         const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
         const int par = (int)(gen & 1);
         const uint32_t phase = (uint32_t)(gen >> 1) & 1u;
@@ -222,8 +299,10 @@ struct RRSync {
         sm.part[0][tid] = v0;
         sm.part[1][tid] = v1;
         sm.part[2][tid] = v2;
+        const int nv = nsub ? 4 : 3;
+        if (nsub) sm.part[3][tid] = z;
         const int anybad = __syncthreads_or(bad);
-        if (wid < 3) {
+        if (wid < nv) {
             // entries beyond the CTA's threads are zero (cleared at the start)
             double t[4];
 #pragma unroll
@@ -235,61 +314,102 @@ struct RRSync {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane == 0)
-                st_async16(up_remote + (uint32_t)(sizeof(RRWord) * kRRSingle * (3 * par + wid)), s, anybad ? 1ull : 0ull,
+                st_async16(up_remote + (uint32_t)(sizeof(RRWord) * kRRSingle * (4 * par + wid)), s, anybad ? 1ull : 0ull,
                            up_bar_remote + 8 * par);
             if (tid == 0) mbar_expect(&sm.down_bar[par], 3 * sizeof(RRWord));
             if (rank == 0) {
-                if (tid == 0) mbar_expect(&sm.up_bar[par], (uint32_t)sizeof(RRWord) * (3 * ncl + test));
+                if (tid == 0) mbar_expect(&sm.up_bar[par], (uint32_t)sizeof(RRWord) * (nv * ncl + test));
                 bool ok = wait(&sm.up_bar[par], phase);
                 double a = 0.0;
                 if (lane < ncl) {
                     a = sm.up[par][wid][lane].v;
                     ok = ok && sm.up[par][wid][lane].tag == 0;
                 }
-#pragma unroll
-                for (int o = kRRSingle / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
                 ok = __all_sync(0xffffffffu, ok);
-                if (nclusters > 1) {
-                    double* base = words + 2 * (size_t)kRRMaxClusters * (3 * par + wid);
-                    if (lane == 0) st_word(base + 2 * cluster_id, a, ok ? gen : gen | kRRFail);
-                    unsigned long long tag = gen;
-                    a = 0.0;
-                    if (lane < nclusters) {
-                        ld_word(base + 2 * lane, a, tag);
-                        for (unsigned spins = 0; (tag & ~kRRFail) != gen;) {
-                            if (expired(++spins)) {
-                                tag = kRRFail;
-                                break;
-                            }
-                            ld_word(base + 2 * lane, a, tag);
-                        }
-                    }
-                    ok = __all_sync(0xffffffffu, !(tag & kRRFail));
+                if (wid == 3) {
+                    exchange_z(a, ok, par);
+                } else {
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    for (int o = kRRSingle / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    if (nclusters > 1) {
+                        double* base = words + 2 * (size_t)kRRMaxClusters * (3 * par + wid);
+                        if (lane == 0) st_word(base + 2 * cluster_id, a, ok ? gen : gen | kRRFail);
+                        unsigned long long t0 = gen, t1 = gen;
+                        a = 0.0;
+                        if (lane < nclusters) a = poll_word(base + 2 * lane, t0);
+                        if (lane + 32 < nclusters) a += poll_word(base + 2 * (lane + 32), t1);
+                        ok = __all_sync(0xffffffffu, !((t0 | t1) & kRRFail));
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    }
+                    if (lane == 0) {
+                        sm.tot[wid] = a;
+                        sm.ok[wid] = ok;
+                    }
                 }
-                if (lane == 0) {
-                    sm.tot[wid] = a;
-                    sm.ok[wid] = ok;
-                }
-                asm volatile("bar.sync 1, 96;" ::: "memory");   // the three reducing warps
+                asm volatile("bar.sync 1, %0;" ::"r"(32 * nv) : "memory");   // the reducing warps
                 if (wid == 0) {
                     double o[4] = {0.0, 0.0, 0.0, 0.0};
                     f(sm.tot[0], sm.tot[1], sm.tot[2], o);
+                    const bool valid = sm.ok[0] && sm.ok[1] && sm.ok[2] && (!nsub || sm.ok[3]);
                     if (lane < ncl) {
                         const uint32_t dst = cluster_addr(&sm.down[par][0], lane), mb = cluster_addr(&sm.down_bar[par], lane);
                         st_async16(dst, o[0], (unsigned long long)__double_as_longlong(o[1]), mb);
                         st_async16(dst + 16, o[2], (unsigned long long)__double_as_longlong(o[3]), mb);
-                        st_async16(dst + 32, 0.0, sm.ok[0] && sm.ok[1] && sm.ok[2] ? 1ull : 0ull, mb);
+                        if (!nsub) st_async16(dst + 32, 0.0, valid ? 1ull : 0ull, mb);
+                    }
+                    if (lane == 0) {
+                        sm.ab[0] = o[0];
+                        sm.ab[1] = o[1];
+                        sm.valid = valid;
                     }
                 }
             }
+        }
+        // the correction, on up to eight warps of the first CTA
+        if (nsub && rank == 0 && wid < 8) {
+            const int nb = nw < 8 ? nw : 8;
+            asm volatile("bar.sync 2, %0;" ::"r"(32 * nb) : "memory");   // zt, ab and valid are there
+            double sv[kRRMaxSub / 32];
+#pragma unroll
+            for (int j = 0; j < kRRMaxSub / 32; ++j) {
+                const int k = lane + 32 * j;
+                sv[j] = 0.0;
+                if (k < nsub && corr != kRRNone) {
+                    double q = 0.0;
+                    if (corr == kRRStart) {
+                        sv[j] = sm.zt[k];
+                    } else {
+                        q = fma(sm.ab[1], sm.zq[zpar][k], sm.zt[k]);
+                        sv[j] = fma(-sm.ab[0], q, sm.zs[zpar][k]);
+                    }
+                    if (wid == 0) {
+                        sm.zq[zpar ^ 1][k] = q;
+                        sm.zs[zpar ^ 1][k] = sv[j];
+                    }
+                }
+            }
+            for (int c = wid; c < ncl; c += nb) {
+                double m = 0.0;
+                if (corr != kRRNone) {
+#pragma unroll
+                    for (int j = 0; j < kRRMaxSub / 32; ++j)
+                        if (lane + 32 * j < nsub) m = fma(sm.einv[c * nsub + lane + 32 * j], sv[j], m);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+                }
+                if (lane == 0)
+                    st_async16(cluster_addr(&sm.down[par][2], c), m, sm.valid ? 1ull : 0ull,
+                               cluster_addr(&sm.down_bar[par], c));
+            }
+            if (corr != kRRNone) zpar ^= 1;
         }
         const bool got = wait(&sm.down_bar[par], phase);
         out[0] = sm.down[par][0].v;
         out[1] = __longlong_as_double((long long)sm.down[par][0].tag);
         out[2] = sm.down[par][1].v;
         out[3] = __longlong_as_double((long long)sm.down[par][1].tag);
+        mu = sm.down[par][2].v;
         const bool valid = sm.down[par][2].tag != 0;
         return __syncthreads_and(got && valid) != 0;
     }
@@ -301,33 +421,49 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
     __shared__ RRShared sm;
     int* const err = reinterpret_cast<int*>(a.w64 + kRRHead - 2);
     double* const ubuf = a.w64 + kRRHead;
-    for (int k = threadIdx.x; k < 3 * kRRMaxWarps * 32; k += blockDim.x) (&sm.part[0][0])[k] = 0.0;
-    RRSync sy(sm, a.w64, err, a.wait_test);   // (ends with a cluster barrier)
+    for (int k = threadIdx.x; k < 4 * kRRMaxWarps * 32; k += blockDim.x) (&sm.part[0][0])[k] = 0.0;
+    if (a.nsub) {
+        const cgrp::cluster_group c = cgrp::this_cluster();
+        if (c.block_rank() == 0)
+            for (int k = threadIdx.x; k < (int)c.num_blocks() * a.nsub; k += blockDim.x)
+                sm.einv[k] = __ldg(a.einv + (size_t)blockIdx.x * a.nsub + k);
+    }
+    RRSync sy(sm, a.w64, err, a.wait_test, a.nsub);   // (ends with a cluster barrier)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
-    const int sl = (int)blockIdx.x * nw + wid;              // this warp's slice (one at most)
-    const bool has = sl < A.nslices;
-    const int i = sl * 32 + lane;
-    const bool row = has && i < A.n;
+    // ---- this thread's row: from the plan, or one slice per warp; its entry k is at base + 32 k
+    int i, base = 0, w_ = 0;
+    bool row, in_space = false;
+    if (a.perm) {
+        const int g = __ldg(a.perm + blockIdx.x * blockDim.x + threadIdx.x);
+        row = g != -1;
+        in_space = g >= 0;
+        i = g >= 0 ? g : -2 - g;
+        if (row) {
+            base = __ldg(A.ptr + (i >> 5)) + (i & 31);
+            w_ = __ldg(a.rowptr + i + 1) - __ldg(a.rowptr + i);
+        }
+    } else {
+        const int sl = (int)blockIdx.x * nw + wid;
+        i = sl * 32 + lane;
+        row = i < A.n;
+        if (sl < A.nslices) {
+            base = __ldg(A.ptr + sl) + lane;
+            w_ = (__ldg(A.ptr + sl + 1) - base + lane) >> 5;
+        }
+    }
     // ---- row data, loaded once
     int col[kRRWidth];
     double av[kRRWidth];
-    int w_ = 0;
     double dinv_i = 0.0;
 #pragma unroll
     for (int k = 0; k < kRRWidth; ++k) {
         col[k] = 0;
         av[k] = 0.0;
-    }
-    if (has) {
-        const int base = __ldg(A.ptr + sl);
-        w_ = (__ldg(A.ptr + sl + 1) - base) >> 5;
-#pragma unroll
-        for (int k = 0; k < kRRWidth; ++k)
-            if (k < w_) {
-                col[k] = __ldg(A.col + base + 32 * k + lane);
-                av[k] = __ldg(a.val + base + 32 * k + lane);
-            }
+        if (k < w_) {
+            col[k] = __ldg(A.col + base + 32 * k);
+            av[k] = __ldg(a.val + base + 32 * k);
+        }
     }
     if (row) {
         dinv_i = __ldg(a.dinv + i);
@@ -373,7 +509,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                 s1 += av[k + 1] * v[k + 1];
             }
         for (int k = kRRWidth; k < w_ && !bad; ++k) {   // entries beyond the registers
-            const int e = __ldg(A.ptr + sl) + 32 * k + lane;
+            const int e = base + 32 * k;
             const int c = __ldg(A.col + e);
             double x;
             unsigned long long tg;
@@ -396,21 +532,17 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
     };
     double x_i = (row && !a.zero_x) ? a.x[i] : 0.0;
     int iters = 0, status = 0, outer = 0, used_alt = 0;
-    double bb = 0.0, rr_final = 0.0, o[4];
+    double bb = 0.0, rr_final = 0.0, mu = 0.0, o[4];
     bool converged = false;
     // ---- the judge of a second initial guess compares FP64 residuals
     if (a.x_alt && !a.zero_x) {
         const double ax = multiply(x_i, nothing);
         double aa = 0.0, y = 0.0;
-        if (has)
-            for (int k = 0; k < w_; ++k) {
-                const int e = __ldg(A.ptr + sl) + 32 * k + lane;
-                aa += __ldg(a.val + e) * __ldg(a.x_alt + __ldg(A.col + e));
-            }
+        for (int k = 0; k < w_; ++k) aa += __ldg(a.val + base + 32 * k) * __ldg(a.x_alt + __ldg(A.col + base + 32 * k));
         if (row) y = __ldg(a.x_alt + i);
         const double b_i = row ? a.b[i] : 0.0;
         const double e0 = row ? (b_i - ax) * (b_i - ax) : 0.0, e1 = row ? (b_i - aa) * (b_i - aa) : 0.0;
-        if (!sy.reduce(e0, e1, 0.0, bad, o, plain)) {
+        if (!sy.reduce(e0, e1, 0.0, 0.0, kRRNone, bad, o, mu, plain)) {
             status = CGP_ETIMEOUT;
         } else if (o[1] < o[0]) {
             used_alt = 1;
@@ -418,13 +550,12 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         }
     }
     while (status == 0) {
-        // ---- outer: r = b - A x, u = D^{-1} r
+        // ---- outer: r = b - A x, u = M^{-1} r
         double r_i = 0.0;
         const double ax = (a.zero_x && outer == 0) ? 0.0 : multiply(x_i, nothing);
         const double b_i = row ? a.b[i] : 0.0;
         if (row) r_i = b_i - ax;
-        double u_i = dinv_i * r_i;
-        if (!sy.reduce(r_i * r_i, b_i * b_i, 0.0, bad, o, plain)) {
+        if (!sy.reduce(r_i * r_i, b_i * b_i, 0.0, in_space ? r_i : 0.0, kRRStart, bad, o, mu, plain)) {
             status = CGP_ETIMEOUT;
             break;
         }
@@ -442,6 +573,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
             status = CGP_ENOTCONV;
             break;
         }
+        double u_i = fma(dinv_i, r_i, in_space ? mu : 0.0);   // M^{-1} r
         // ---- inner iterations; o = (alpha, beta, gamma, d) of the coming update, and why to
         // leave in the shared flag: 1 = target met or restart, 2 = not finite
         const double stop2 = 0.25 * a.tol2 * bb;
@@ -458,7 +590,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                 }
             });
             const bool ok = sy.reduce(
-                r_i * u_i, w_i * u_i, r_i * r_i, bad, o, [&](double tg, double td, double trr, double (&q)[4]) {
+                r_i * u_i, w_i * u_i, r_i * r_i, in_space ? w_i : 0.0, kRRAdvance, bad, o, mu, [&](double tg, double td, double trr, double (&q)[4]) {
                     const double dn = td - tg * tg * c;
                     q[0] = newton_quotient(tg, dn);
                     q[1] = tg * rg;
@@ -499,7 +631,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                 s_i = fma(o[1], s_i, w_i);
                 x_i = fma(o[0], p_i, x_i);
                 r_i = fma(-o[0], s_i, r_i);
-                u_i = dinv_i * r_i;
+                u_i = fma(dinv_i, r_i, in_space ? mu : 0.0);
             }
             ++iters;
             gd[0] = o[2];
@@ -515,7 +647,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
     // ---- pure-Neumann mean fix
     if (a.mlump && status != CGP_ETIMEOUT) {
         const double m = row ? __ldg(a.mlump + i) : 0.0;
-        if (sy.reduce(m * x_i, m, 0.0, bad, o, [](double t0, double t1, double, double (&q)[4]) { q[0] = t0 / t1; }))
+        if (sy.reduce(m * x_i, m, 0.0, 0.0, kRRNone, bad, o, mu, [](double t0, double t1, double, double (&q)[4]) { q[0] = t0 / t1; }))
             x_i -= o[0];
         else
             status = CGP_ETIMEOUT;
@@ -557,27 +689,27 @@ inline void rr_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], i
     cfg.numAttrs = 2;
 }
 
-// co-resident clusters: of kRRSingle CTAs with up to 8 warps, of kRRCluster CTAs of the largest size
-inline cudaError_t rr_capacity(int* single, int* multi) {
-    *single = *multi = 0;
+inline cudaError_t rr_capacity(RRCapacity* cap) {
+    *cap = RRCapacity{};
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     for (int w : {8, kRRMaxWarps}) {
         const cudaError_t e = cudaFuncSetAttribute(rr_kernel(w), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
     }
-    rr_config(cfg, attr, kRRSingle, kRRSingle, 8, nullptr);
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(single, rr_kernel(8), &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        *single = 0;
-    }
-    rr_config(cfg, attr, kRRCluster, kRRCluster, kRRMaxWarps, nullptr);
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(multi, rr_kernel(kRRMaxWarps), &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        *multi = 0;
-    }
+    auto count = [&](int cluster, int warps) {
+        int n = 0;
+        rr_config(cfg, attr, cluster, cluster, warps, nullptr);
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, rr_kernel(warps), &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        return n;
+    };
+    cap->single = count(kRRSingle, 8);
+    cap->eight = count(kRRCluster, kRRMaxWarps);
+    cap->four = count(kRRCluster / 2, kRRMaxWarps);
     return cudaSuccess;
 }
 

@@ -50,7 +50,7 @@ struct NoAllocSlot {
     void* ctx;
     double* ptr;
     int grid;
-    int rr_single, rr_multi;   // co-resident clusters of the register-resident solve
+    RRCapacity rr;   // co-resident clusters of the register-resident solve
 };
 NoAllocSlot g_slot[kMaxDevices] = {};
 std::mutex g_slot_mu;
@@ -116,13 +116,13 @@ extern "C" int cgp_pcg_sell_noalloc(int32_t n, int32_t nslices, const int32_t* s
             }
             const int g = sms * (per_sm < kGridCtasPerSm ? per_sm : kGridCtasPerSm);
             sl.grid = g < kNoAllocMaxCtas ? g : kNoAllocMaxCtas;
-            CGP_CUDA(rr_capacity(&sl.rr_single, &sl.rr_multi));
+            CGP_CUDA(rr_capacity(&sl.rr));
             sl.ptr = (double*)p;
             sl.ctx = ctx;
         }
         base = sl.ptr;
         max_grid = sl.grid;
-        shape = rr_shape(nslices, sl.rr_single, sl.rr_multi);
+        shape = rr_shape(nslices, sl.rr);
     }
     int grid = (nslices + kGridThreads / 32 - 1) / (kGridThreads / 32);
     if (grid > max_grid) grid = max_grid;

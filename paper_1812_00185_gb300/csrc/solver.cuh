@@ -75,6 +75,9 @@ struct Solver {
     int coarse_grid = 0;          // CTAs of the persistent (cooperative) solver
     int rr_ctas = 0, rr_cluster = 0, rr_warps = 0;   // launch of the register-resident FP64 solve (0: does not fit)
     double *user_ud = nullptr, *user_f = nullptr;   // CGP_BC_USER: 2*nf each
+    int rr_nsub = 0;              // subdomains of its plan (rr_plan.cuh; 0: Jacobi alone)
+    int32_t* rr_perm = nullptr;
+    double* rr_einv = nullptr;
     bool coarse_fp64 = true;
     cudaStream_t branch = nullptr;                 // second stream of a step (work beside the coarse solve)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;      // the coarse solve's inner iterations run in FP64

@@ -895,12 +895,35 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
         // register-resident variant: one slice per warp, one CTA per SM, in clusters
         s.rr_ctas = s.rr_cluster = s.rr_warps = 0;
         if (allow_rr) {
-            int single = 0, multi = 0;
-            CGP_CUDA(rr_capacity(&single, &multi));
-            const RRShape sh = rr_shape(C.nslices, single, multi);
+            RRCapacity cap;
+            CGP_CUDA(rr_capacity(&cap));
+            const RRShape sh = rr_shape(C.nslices, cap);
             s.rr_ctas = sh.ctas;
             s.rr_cluster = sh.cluster;
             s.rr_warps = sh.warps;
+            // its subdomain plan, where the preconditioner is left to the library.  Not on one
+            // cluster: with 16 subdomains the cavity's 33^2 rows took 110 iterations instead of
+            // 152, but each 40 % longer (4 steps 6.25 instead of 5.60 ms)
+            s.rr_nsub = 0;
+            if (sh.ctas > kRRSingle && p.precond == CGP_PRECOND_AUTO && !s.onchip_bytes && s.rr_perm) {
+                std::vector<int32_t> rowptr(C.nv + 1), ptr(C.nslices + 1), col(C.nnz_sell);
+                std::vector<double> xy(2 * (size_t)C.nv), val(C.nnz_sell);
+                std::vector<uint8_t> in_space(C.nv);
+                CGP_CUDA(cudaStreamSynchronize(st));   // the assembled K_c
+                CGP_CUDA(cudaMemcpy(rowptr.data(), C.rowptr, sizeof(int32_t) * (C.nv + 1), cudaMemcpyDeviceToHost));
+                CGP_CUDA(cudaMemcpy(ptr.data(), C.sell_ptr, sizeof(int32_t) * (C.nslices + 1), cudaMemcpyDeviceToHost));
+                CGP_CUDA(cudaMemcpy(col.data(), C.sell_col, sizeof(int32_t) * C.nnz_sell, cudaMemcpyDeviceToHost));
+                CGP_CUDA(cudaMemcpy(xy.data(), C.xy, sizeof(double) * 2 * C.nv, cudaMemcpyDeviceToHost));
+                CGP_CUDA(cudaMemcpy(val.data(), s.Kc0, sizeof(double) * C.nnz_sell, cudaMemcpyDeviceToHost));
+                CGP_CUDA(cudaMemcpy(in_space.data(), C.tag, C.nv, cudaMemcpyDeviceToHost));
+                for (auto& t : in_space) t = (t & CGP_PHI_ZERO) ? 0 : 1;
+                RRHostPlan P;
+                if (rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh.ctas, 32 * sh.warps, s.pure_neumann, P)) {
+                    CGP_CUDA(cudaMemcpy(s.rr_perm, P.perm.data(), sizeof(int32_t) * P.perm.size(), cudaMemcpyHostToDevice));
+                    CGP_CUDA(cudaMemcpy(s.rr_einv, P.einv.data(), sizeof(double) * P.einv.size(), cudaMemcpyHostToDevice));
+                    s.rr_nsub = P.nsub;
+                }
+            }
         }
         // mixed form, AUTO, no room on chip: the grid-wide FP64 solve (one reduction per
         // iteration) is faster on this GPU than the FP32 inner solve (two) with the same grid
@@ -968,6 +991,10 @@ CoarsePcgArgs coarse_args(Solver& s) {
     a.partials = s.coarse_partials;
     a.wait_test = s.wait_test;
     a.gate = s.onchip_bytes ? s.mlp_gate : nullptr;
+    a.nsub = s.rr_nsub;
+    a.perm = s.rr_nsub ? s.rr_perm : nullptr;
+    a.einv = s.rr_einv;
+    a.rowptr = C.rowptr;
     return a;
 }
 
@@ -1732,7 +1759,7 @@ extern "C" int cgp_coarse_subdomains(const cgp_solver* h, int32_t* nsub) {
         set_error("null solver");
         return CGP_EINVAL;
     }
-    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : 0;
+    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub : 0);
     return CGP_OK;
 }
 

@@ -1,6 +1,7 @@
 """Solver parameter sets of the named forms, and training of the learned guess on a workload.
 
-A *form* is one way of running the same CGP step: ``fp64`` (every solve in FP64),
+A *form* is one way of running the same CGP step: ``fp64`` (every solve in FP64, the coarse
+one with Jacobi alone, as the other FP64 forms: the plain method),
 ``mixed`` (FP32-inner / FP64-outer refinement, previous increment as the coarse guess),
 ``mixed_zero`` (the same from a zero guess), ``mixed_jacobi`` (Jacobi alone in the on-chip
 coarse solve), ``mixed_proj`` / ``fp64_proj`` (the coarse guess projected onto the last
@@ -37,7 +38,8 @@ def workload_params(w, form, use_graph=1, tol_inner=0.0, mass_mode=0, chi=None, 
                           max_it_mass=1000, precision=cg.CGP_MIXED if mixed else cg.CGP_FP64,
                           guess=guess, bc_kind=w.bc, bc_param=w.bc_param, use_graph=use_graph,
                           tol_inner=tol_inner,
-                          precond=cg.CGP_PRECOND_JACOBI if form == "mixed_jacobi" else cg.CGP_PRECOND_AUTO,
+                          precond=cg.CGP_PRECOND_JACOBI if form == "mixed_jacobi" or not mixed else
+                          cg.CGP_PRECOND_AUTO,
                           mass_mode=mass_mode)
 
 

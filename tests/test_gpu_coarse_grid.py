@@ -49,11 +49,14 @@ CASES = {
 }
 
 
+@pytest.mark.parametrize("precond", ["auto", "jacobi"])
 @pytest.mark.parametrize("name", CASES)
-def test_fp64_coarse_solve_meets_its_tolerance(lib, name):
+def test_fp64_coarse_solve_meets_its_tolerance(lib, name, precond):
     from paper_1812_00185_gb300 import binding as cg
     base, levels = CASES[name]()
-    m, s, A, fixed = _system(cg, base, levels)
+    m, s, A, fixed = _system(cg, base, levels, precond=cg.CGP_PRECOND_AUTO if precond == "auto" else
+                             cg.CGP_PRECOND_JACOBI)
+    assert s.coarse_subdomains() == 0 or precond == "auto"
     b = _rhs(A.shape[0], fixed, 7)
     phi, it, rc = cg.cgp_poisson_solve(s.handle, b)
     assert rc == cg.CGP_OK and it > 0
