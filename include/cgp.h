@@ -298,13 +298,15 @@ void cgp_solver_destroy(cgp_solver* s);
  *    instances from a queue, largest first, and run each instance's whole step of Eqs. 21-26
  *    (momentum rows and FP64 BiCGStab, coarse right-hand side and the instance's coarse PCG,
  *    prolongation, Chebyshev mass solves of Eqs. 25-26 with the eigenvalue bounds [1/2, 2] of
- *    Jacobi-scaled P1 mass matrices, pressure update), reducing through distributed shared
+ *    Jacobi-scaled P1 mass matrices, FP32 steps inside FP64 refinement in mixed instances,
+ *    pressure update), reducing through distributed shared
  *    memory; the launch is captured in a CUDA graph;
  *  - graph branches (CGP_BATCH_BRANCHES): one CUDA graph per step with every instance's
  *    momentum solve and coarse right-hand side on its own stream, ONE persistent launch for
  *    all the coarse Poisson problems, then every instance's correction and update.
  * cluster_size (0 = autotune, else 1, 2, 4, 8) and threads (0 = autotune, else 256, 512,
- * 1024) fix the persistent launch's shape; the autotuner times each candidate on the
+ * 1024) fix the persistent launch's shape; the autotuner (which for large instances also tries
+ * clusters of 16) times each candidate on the
  * instances' first step (whole step) or first coarse problems (branches), restoring their
  * state after each trial.  The batch allocates its own device memory (launch arguments, a
  * queue counter and the saved state); the solvers must outlive it.  Synchronises `stream`. */

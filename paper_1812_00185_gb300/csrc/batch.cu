@@ -18,6 +18,7 @@
 // autotuner that times every candidate on the batch's own first coarse problems (the
 // instances' coarse state is saved and restored around the trials).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "solver.cuh"
@@ -28,7 +29,7 @@ struct cgp_batch {
     int whole = 0;                          // 1: whole-step persistent launch, 0: graph branches
     void* d_step_args = nullptr;            // BatchStepArgs[n], device (whole-step form)
     double* d_state = nullptr;              // saved U, U_prev, P, phi, t, stats, Krylov states (autotuning)
-    std::vector<Solver*> inst;              // in launch order (largest coarse level first)
+    std::vector<Solver*> inst;              // in launch order (longest step first)
     std::vector<cudaStream_t> streams;
     std::vector<cudaEvent_t> events;
     cudaStream_t origin = nullptr;
@@ -36,6 +37,7 @@ struct cgp_batch {
     unsigned int* d_queue = nullptr;
     double* d_save = nullptr;               // saved rhs and Phi_c of every instance (autotuning)
     int csize = 1, threads = 256, nclusters = 1;
+    int floats = 0;                         // dynamic shared memory of the whole-step launch
     std::vector<float> trial_ms;            // per candidate, -1 if it does not fit
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -142,9 +144,14 @@ int save_state(cgp_batch* b, bool restore, cudaStream_t st) {
     return CGP_OK;
 }
 
+// (the last two are no choice of the caller's: clusters of 16 CTAs, tried by the autotuner when
+// the largest instance gives every thread of 8 CTAs more than kWideRows rows.  Such an instance
+// is the launch's critical path: its momentum iterations read more through L2 than 8 SMs take.
+// 32 uneven cavities up to 256^2: 15.7 ms a step with 15 clusters of 8 x 512, 13.4 with 7 of 16.)
 const int kStepCand[][2] = {{1, 256}, {1, 512}, {1, 1024}, {2, 256}, {2, 512}, {2, 1024}, {4, 256}, {4, 512},
-                            {4, 1024}, {8, 256}, {8, 512}, {8, 1024}};
+                            {4, 1024}, {8, 256}, {8, 512}, {8, 1024}, {16, 256}, {16, 512}};
 constexpr int kNumStepCand = sizeof(kStepCand) / sizeof(kStepCand[0]);
+constexpr int kWideRows = 8;
 
 int autotune_whole(cgp_batch* b, int fixed_csize, int fixed_threads, cudaStream_t st) {
     CGP_TRY(save_state(b, false, st));
@@ -155,16 +162,21 @@ int autotune_whole(cgp_batch* b, int fixed_csize, int fixed_threads, cudaStream_
     float best = 1e30f;
     int rc = CGP_OK;
     const int n = (int)b->inst.size();
+    int widest = 0;
+    for (const Solver* s : b->inst) widest = std::max(widest, s->nf);
     for (int k = 0; k < kNumStepCand && rc == CGP_OK; ++k) {
         const int cs = kStepCand[k][0], th = kStepCand[k][1];
         if ((fixed_csize && cs != fixed_csize) || (fixed_threads && th != fixed_threads)) continue;
+        if (cs > 8 && widest <= 8 * 512 * kWideRows) continue;
         int ncl = 0;
-        if ((rc = batch_step_clusters(cs, th, &ncl)) != CGP_OK) break;
+        int floats = 0;
+        if ((rc = batch_step_shared(b->inst.data(), n, cs, &floats)) != CGP_OK) break;
+        if ((rc = batch_step_clusters(cs, th, floats, &ncl)) != CGP_OK) break;
         if (ncl < 1) continue;
         if (ncl > n) ncl = n;
         if ((rc = save_state(b, true, st)) != CGP_OK) break;
         cudaEventRecord(e0, st);
-        if ((rc = launch_batch_step(b->d_step_args, n, b->d_queue, cs, th, ncl, st)) != CGP_OK) break;
+        if ((rc = launch_batch_step(b->d_step_args, n, b->d_queue, cs, th, floats, ncl, st)) != CGP_OK) break;
         cudaEventRecord(e1, st);
         if (cudaEventSynchronize(e1) != cudaSuccess) {
             set_error("batched step trial failed: %s", cudaGetErrorString(cudaGetLastError()));
@@ -178,6 +190,7 @@ int autotune_whole(cgp_batch* b, int fixed_csize, int fixed_threads, cudaStream_
             best = ms;
             b->csize = cs;
             b->threads = th;
+            b->floats = floats;
             b->nclusters = ncl;
         }
     }
@@ -198,7 +211,8 @@ int autotune_whole(cgp_batch* b, int fixed_csize, int fixed_threads, cudaStream_
 int build_graph_whole(cgp_batch* b) {
     cudaStream_t o = b->origin;
     CGP_CUDA(cudaStreamBeginCapture(o, cudaStreamCaptureModeThreadLocal));
-    int rc = launch_batch_step(b->d_step_args, (int)b->inst.size(), b->d_queue, b->csize, b->threads, b->nclusters, o);
+    int rc = launch_batch_step(b->d_step_args, (int)b->inst.size(), b->d_queue, b->csize, b->threads, b->floats, b->nclusters,
+                               o);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(o, &g);
     if (rc != CGP_OK || e != cudaSuccess) {
@@ -285,8 +299,11 @@ extern "C" int cgp_batch_create_mode(cgp_solver* const* solvers, int32_t n, int3
         }
         b->inst.push_back(&solvers[i]->s);
     }
-    // largest coarse problem first: the queue hands the long solves out early
-    std::stable_sort(b->inst.begin(), b->inst.end(), [](const Solver* x, const Solver* y) { return x->nc > y->nc; });
+    // the longest steps first, so that the queue hands them out early.  Clocks of a step on 8
+    // CTAs: about 200 per fine row (assembly, momentum, mass solves) and 110k per square root of
+    // the coarse rows (the iterations of the coarse solve)
+    auto cost = [](const Solver* s) { return 200.0 * s->nf + 1.1e5 * std::sqrt((double)s->nc); };
+    std::stable_sort(b->inst.begin(), b->inst.end(), [&](const Solver* x, const Solver* y) { return cost(x) > cost(y); });
     cudaStream_t st = (cudaStream_t)stream;
     auto fail = [&](int rc) {
         cgp_batch_destroy(b);

@@ -20,8 +20,11 @@
 //              steps need no inner products and their number follows from the tolerance
 //              (error <= 4 * 3^-n of the initial one in the energy norm)
 //   Eq. 26     the rotational term (D U~, and the same Chebyshev solve on M) and the update
-// In a mixed instance the momentum BiCGStab's inner iterations run in FP32: on this GPU the
-// narrow FP64 pipe is the busiest unit of the cluster's FP64 iterations.
+// In a mixed instance the momentum BiCGStab's inner iterations and the Chebyshev steps run in
+// FP32: on this GPU the narrow FP64 pipe is the busiest unit of the cluster's FP64 iterations.
+// Clocks of a 66k-row instance's step on 8 CTAs (iterations in
+// brackets): momentum 5.5M (20 iterations), coarse solve at 4,225 rows 7.5M (450; 10.4M with
+// its vectors in memory), the two mass solves 4.3M (5.8M in FP64), assembly 1.0M.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -51,6 +54,8 @@ struct BatchStepArgs {
     int64_t nnz;
     float *A32, *dinvA32;
     float* fv[10];
+    const float *M0f, *Mf, *dinvM0f, *dinvMf;   // FP32 mass matrices and Jacobi diagonals
+    double tol_mass2;
     // coarse level and its solve
     SellView Ac;
     const double *Cxc, *Cyc, *Kc, *cxy;
@@ -82,68 +87,228 @@ __host__ __device__ inline int cheb_steps_for(double tol) {
     return n;
 }
 
+// The step's coefficients of the semi-iteration with these bounds (theta = 1.25, delta = 0.75):
+// d' = c1 d + c2 D^-1 r.  A table: the recurrence's two FP64 divides in every thread cost 7k
+// clocks a step.
+struct ChebTable {
+    double c1[200], c2[200];
+    constexpr ChebTable() : c1(), c2() {
+        const double delta = 0.75, sigma = 1.25 / 0.75;
+        double rho = 1.0 / sigma;
+        for (int k = 0; k < 200; ++k) {
+            const double next = 1.0 / (2.0 * sigma - rho);
+            c1[k] = next * rho;
+            c2[k] = 2.0 * next / delta;
+            rho = next;
+        }
+    }
+};
+static __constant__ ChebTable kChebTable = ChebTable();
+
 // Mixed instances: the momentum system runs up to kBatchIrSweeps FP64-residual sweeps around
 // an FP32 BiCGStab (each asked for kBatchInnerTol of its right-hand side, or what is left to
-// the tolerance), then the FP64 BiCGStab unless a sweep's residual already met the tolerance.
-constexpr int kBatchIrSweeps = 3;
+// the tolerance) while they gain at least a decade each, then the FP64 BiCGStab unless a
+// sweep's residual already met the tolerance.  (With three sweeps, two of 32 cavities at a
+// tolerance of 1e-12 were left just above it and spent 15M clocks in the FP64 iteration.)
+constexpr int kBatchIrSweeps = 8;
 constexpr double kBatchInnerTol = 1e-4;
 constexpr int kBatchInnerMaxit = 200;
 
-// Chebyshev semi-iteration for B x = rhs (NC interleaved components), x = 0 at the start;
-// Jacobi preconditioning, bounds [1/2, 2] of D^-1 B; one cluster barrier per step.  (It stays
-// FP64 in mixed instances too: FP32 sweeps inside FP64 refinement took longer here, the
-// cluster's steps being bound by latency rather than by the FP64 pipe.)
-template <int NC, class T = double>
-__device__ void cluster_chebyshev(const SellView& B, const T* __restrict__ val, const T* __restrict__ dinv,
-                                  const T* __restrict__ rhs, T* __restrict__ x, T* __restrict__ r,
-                                  T* __restrict__ d0, T* __restrict__ d1, int steps, int crank, int csize,
-                                  cgrp_bs::cluster_group& cl) {
-    const double theta = 1.25, delta = 0.75, sigma = theta / delta;
-    const int n = B.n, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5, wid = threadIdx.x >> 5;
-    for (int i = crank * blockDim.x + threadIdx.x; i < n; i += csize * blockDim.x) {
-        const T di = dinv[i];
+// rows sl[0 .. U-1] (slices; one past the end: none) of the two- or one-component product A u,
+// the pattern and value loads of all U slices in flight together
+template <int U, int NC, class T>
+__device__ __forceinline__ void spmv_slices(const SellView& A, const T* __restrict__ val, const T* __restrict__ u,
+                                            const int (&sl)[U], int lane, T (&ax)[U][NC]) {
+    int base[U], w[U], wmax = 0;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const T ri = rhs[NC * i + c];
-            x[NC * i + c] = T(0);
-            r[NC * i + c] = ri;
-            d0[NC * i + c] = di * ri / T(theta);
+    for (int q = 0; q < U; ++q) {
+        base[q] = w[q] = 0;
+        if (sl[q] < A.nslices) {
+            base[q] = __ldg(A.ptr + sl[q]);
+            w[q] = (__ldg(A.ptr + sl[q] + 1) - base[q]) >> 5;
         }
     }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+        wmax = max(wmax, w[q]);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ax[q][c] = T(0);
+    }
+    for (int k0 = 0; k0 < wmax; k0 += 8) {
+        int cj[U][8];
+        T av[U][8];
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                cj[q][k] = 0;
+                av[q][k] = T(0);
+                if (k0 + k < w[q]) {
+                    const int e = base[q] + 32 * (k0 + k) + lane;
+                    cj[q][k] = __ldg(A.col + e);
+                    av[q][k] = __ldg(val + e);
+                }
+            }
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k0 + k < w[q]) {
+                    T xv[NC];
+                    ldv<NC>(u, cj[q][k], xv);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) ax[q][c] += av[q][k] * xv[c];
+                }
+    }
+}
+
+// `steps` Chebyshev steps on B e = r (NC interleaved components) from e = 0, with Jacobi and the
+// bounds [1/2, 2] of D^-1 B; one cluster barrier per step.  r is overwritten.
+template <int NC, class T>
+__device__ void cluster_cheb_steps(const SellView& B, const T* __restrict__ val, const T* __restrict__ dinv, T* r, T* e,
+                                   T* d0, T* d1, int steps, int crank, int csize, cgrp_bs::cluster_group& cl) {
+    constexpr int U = sizeof(T) == 4 ? 2 : 1;   // slices in flight per warp (registers)
+    const int n = B.n, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5, wid = threadIdx.x >> 5;
+    const int stride = csize * nwarp;
+    for (int i = crank * blockDim.x + threadIdx.x; i < n; i += csize * blockDim.x) {
+        T rv[NC], dv[NC], zero[NC];
+        ldv<NC>(r, i, rv);
+        const T di = dinv[i] * T(0.8);   // 1 / theta
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            dv[c] = di * rv[c];
+            zero[c] = T(0);
+        }
+        stv<NC>(d0, i, dv);
+        stv<NC>(e, i, zero);
+    }
     cl.sync();
-    double rho = 1.0 / sigma;
     T* dc = d0;
     T* dn = d1;
     for (int k = 0; k < steps; ++k) {
-        const double rho_n = 1.0 / (2.0 * sigma - rho);
-        const T c1 = (T)(rho_n * rho), c2 = (T)(2.0 * rho_n / delta);
-        for (int sl = crank * nwarp + wid; sl < B.nslices; sl += csize * nwarp) {
-            const int i = sl * 32 + lane;
-            T wv[NC];
+        const T c1 = (T)kChebTable.c1[k], c2 = (T)kChebTable.c2[k];
+        for (int s0 = crank * nwarp + wid; s0 < B.nslices; s0 += U * stride) {
+            int sl[U];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) wv[c] = T(0);
-            sell_accum<NC>(B, val, sl, lane, [&](int j, T (&o)[NC]) {
+            for (int q = 0; q < U; ++q) sl[q] = s0 + q * stride;
+            T dv[U][NC], rv[U][NC], ev[U][NC], di[U], wv[U][NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) o[c] = dc[NC * j + c];
-            }, wv);
-            if (i < n) {
-                const T di = dinv[i];
+            for (int q = 0; q < U; ++q) {
+                const int i = sl[q] * 32 + lane;
+                if (i < n) {
+                    ldv<NC>(dc, i, dv[q]);
+                    ldv<NC>(r, i, rv[q]);
+                    ldv<NC>(e, i, ev[q]);
+                    di[q] = dinv[i];
+                }
+            }
+            spmv_slices<U, NC>(B, val, dc, sl, lane, wv);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const T dd = dc[NC * i + c];
-                    x[NC * i + c] += dd;
-                    const T rn = r[NC * i + c] - wv[c];
-                    r[NC * i + c] = rn;
-                    dn[NC * i + c] = c1 * dd + c2 * di * rn;
+            for (int q = 0; q < U; ++q) {
+                const int i = sl[q] * 32 + lane;
+                if (i < n) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        ev[q][c] += dv[q][c];
+                        rv[q][c] -= wv[q][c];
+                        dv[q][c] = c1 * dv[q][c] + c2 * di[q] * rv[q][c];
+                    }
+                    stv<NC>(e, i, ev[q]);
+                    stv<NC>(r, i, rv[q]);
+                    stv<NC>(dn, i, dv[q]);
                 }
             }
         }
         cl.sync();
-        rho = rho_n;
         T* t = dc;
         dc = dn;
         dn = t;
     }
+}
+
+// B x = rhs in FP64 by one run of the semi-iteration
+template <int NC>
+__device__ __noinline__ void cluster_chebyshev(const SellView& B, const double* __restrict__ val, const double* __restrict__ dinv,
+                                  const double* __restrict__ rhs, double* x, double* r, double* d0, double* d1,
+                                  int steps, int crank, int csize, cgrp_bs::cluster_group& cl) {
+    // (each thread copies the rows that it initialises in cluster_cheb_steps)
+    for (int i = crank * blockDim.x + threadIdx.x; i < B.n; i += csize * blockDim.x) {
+        double v[NC];
+        ldv<NC>(rhs, i, v);
+        stv<NC>(r, i, v);
+    }
+    cluster_cheb_steps<NC, double>(B, val, dinv, r, x, d0, d1, steps, crank, csize, cl);
+}
+
+// B x = rhs of a mixed instance: sweeps of the FP64 residual and kBatchChebSteps FP32 steps
+// (each reduces the error to below 1e-5) until the residual meets the tolerance; false when
+// kBatchChebSweeps did not get there (the caller then runs the FP64 semi-iteration).  A step of
+// a 66k-row instance on 8 CTAs is bound by the FP64 pipe in FP64 (130k clocks), by latency in
+// FP32.
+constexpr int kBatchChebSteps = 12, kBatchChebSweeps = 6;
+
+template <int NC>
+__device__ __noinline__ bool cluster_cheb_mixed(const SellView& B, const double* __restrict__ val, const float* __restrict__ val32,
+                                   const float* __restrict__ dinv32, const double* __restrict__ rhs, double* x,
+                                   float* r32, float* e, float* d0, float* d1, double tol2, ClusterSync& cs, int crank,
+                                   int csize, cgrp_bs::cluster_group& cl, int& steps) {
+    const int n = B.n, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5, wid = threadIdx.x >> 5;
+    double bb[NC];
+    steps = 0;
+    for (int sw = 0; sw <= kBatchChebSweeps; ++sw) {
+        double acc[2 * NC];
+#pragma unroll
+        for (int c = 0; c < 2 * NC; ++c) acc[c] = 0.0;
+        for (int sl = crank * nwarp + wid; sl < B.nslices; sl += csize * nwarp) {
+            const int i = sl * 32 + lane;
+            double ax[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ax[c] = 0.0;
+            if (sw) sell_accum<NC>(B, val, sl, lane, [&](int j, double (&o)[NC]) { ldv<NC>(x, j, o); }, ax);
+            if (i < n) {
+                double bv[NC], zero[NC];
+                float rf[NC];
+                ldv<NC>(rhs, i, bv);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const double rv = bv[c] - ax[c];
+                    rf[c] = (float)rv;
+                    zero[c] = 0.0;
+                    acc[c] += rv * rv;
+                    acc[NC + c] += bv[c] * bv[c];
+                }
+                stv<NC>(r32, i, rf);
+                if (!sw) stv<NC>(x, i, zero);
+            }
+        }
+        double tot[2 * NC];
+        cs.sum(acc, tot);   // (r32 is complete: a cluster barrier)
+        bool all = true, finite_all = true;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            if (!sw) bb[c] = tot[NC + c];
+            all = all && tot[c] <= tol2 * bb[c];
+            finite_all = finite_all && isfinite(tot[c]);
+        }
+        if (all) return true;
+        if (!finite_all || sw == kBatchChebSweeps) return false;
+        cluster_cheb_steps<NC, float>(B, val32, dinv32, r32, e, d0, d1, kBatchChebSteps, crank, csize, cl);
+        steps += kBatchChebSteps;
+        for (int sl = crank * nwarp + wid; sl < B.nslices; sl += csize * nwarp) {
+            const int i = sl * 32 + lane;
+            if (i < n) {
+                double xv[NC];
+                float ev[NC];
+                ldv<NC>(x, i, xv);
+                ldv<NC>(e, i, ev);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) xv[c] += (double)ev[c];
+                stv<NC>(x, i, xv);
+            }
+        }
+        cl.sync();
+    }
+    return false;
 }
 
 // BiCGStab with Jacobi for the two velocity components of one instance, on its cluster.  T:
@@ -153,12 +318,15 @@ __device__ void cluster_chebyshev(const SellView& B, const T* __restrict__ val, 
 // times.  Converged when <r, r> <= tol2 <b, b> for each component.  Returns the iterations;
 // status, the last <r, r> and <b, b> go out.
 template <class T>
-__device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, const T* __restrict__ dinv,
+__device__ __noinline__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, const T* __restrict__ dinv,
                                 const T* __restrict__ b, const BicgVecsT<T>& V, double tol2, int maxit, int restarts,
                                 bool zero_x, ClusterSync& cs, cgrp_bs::cluster_group& cl, int crank, int csize,
                                 int& status, double (&rr)[2], double (&bb)[2]) {
     const int n = A.n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int tid = crank * blockDim.x + threadIdx.x, nthr = csize * blockDim.x;
+    // rows (vector passes) and slices (products) in flight per thread: the passes are bound by
+    // latency, a thread walking 16 rows of a 66k-row instance one after the other
+    constexpr int U = sizeof(T) == 4 ? 2 : 1, R = sizeof(T) == 4 ? 4 : 1, R2 = sizeof(T) == 4 ? 2 : 1;
     double rho[2] = {0.0, 0.0}, alpha[2] = {0.0, 0.0}, omega[2] = {0.0, 0.0}, beta[2] = {0.0, 0.0};
     int done[2] = {0, 0}, it = 0;
     status = 0;
@@ -197,30 +365,53 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
         }
         bool broke = false;
         while (!(done[0] && done[1]) && it < maxit && !broke) {
-            // p = r + beta (p - omega v), y = D^-1 p
-            for (int i = tid; i < n; i += nthr) {
-                const T di = dinv[i];
+            // p = r + beta (p - omega v), y = D^-1 p.  (Vectors of a component that is done
+            // may hold anything from here on; only its x is kept.)
+            for (int i0 = tid; i0 < n; i0 += R * nthr) {
+                T rv[R][2], pv[R][2], vv[R][2], di[R];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    if (done[c]) continue;
-                    const T pv = V.r[2 * i + c] + (T)beta[c] * (V.p[2 * i + c] - (T)omega[c] * V.v[2 * i + c]);
-                    V.p[2 * i + c] = pv;
-                    V.y[2 * i + c] = di * pv;
+                for (int q = 0; q < R; ++q) {
+                    const int i = i0 + q * nthr;
+                    if (i < n) {
+                        ldv<2>(V.r, i, rv[q]);
+                        ldv<2>(V.p, i, pv[q]);
+                        ldv<2>(V.v, i, vv[q]);
+                        di[q] = dinv[i];
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const int i = i0 + q * nthr;
+                    if (i < n) {
+                        T yv[2];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            pv[q][c] = rv[q][c] + (T)beta[c] * (pv[q][c] - (T)omega[c] * vv[q][c]);
+                            yv[c] = di[q] * pv[q][c];
+                        }
+                        stv<2>(V.p, i, pv[q]);
+                        stv<2>(V.y, i, yv);
+                    }
                 }
             }
             cl.sync();
             {   // v = A y, alpha = rho / <rhat, v>
                 T acc[2] = {T(0), T(0)};
-                for (int sl = crank * nwarp + wid; sl < A.nslices; sl += csize * nwarp) {
-                    const int i = sl * 32 + lane;
-                    T ax[2];
-                    spmv2_row(A, val, V.y, sl, lane, ax);
-                    if (i < n) {
+                for (int s0 = crank * nwarp + wid; s0 < A.nslices; s0 += U * csize * nwarp) {
+                    int sl[U];
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            if (done[c]) continue;
-                            V.v[2 * i + c] = ax[c];
-                            acc[c] += V.rhat[2 * i + c] * ax[c];
+                    for (int q = 0; q < U; ++q) sl[q] = s0 + q * csize * nwarp;
+                    T ax[U][2];
+                    spmv_slices<U, 2>(A, val, V.y, sl, lane, ax);
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        const int i = sl[q] * 32 + lane;
+                        if (i < n) {
+                            T rh[2];
+                            ldv<2>(V.rhat, i, rh);
+                            stv<2>(V.v, i, ax[q]);
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) acc[c] += rh[c] * ax[q][c];
                         }
                     }
                 }
@@ -250,30 +441,53 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
             }
             if (broke) break;
             // s = r - alpha v, z = D^-1 s
-            for (int i = tid; i < n; i += nthr) {
-                const T di = dinv[i];
+            for (int i0 = tid; i0 < n; i0 += R * nthr) {
+                T rv[R][2], vv[R][2], di[R];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    if (done[c]) continue;
-                    const T sv = V.r[2 * i + c] - (T)alpha[c] * V.v[2 * i + c];
-                    V.s[2 * i + c] = sv;
-                    V.z[2 * i + c] = di * sv;
+                for (int q = 0; q < R; ++q) {
+                    const int i = i0 + q * nthr;
+                    if (i < n) {
+                        ldv<2>(V.r, i, rv[q]);
+                        ldv<2>(V.v, i, vv[q]);
+                        di[q] = dinv[i];
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < R; ++q) {
+                    const int i = i0 + q * nthr;
+                    if (i < n) {
+                        T zv[2];
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            rv[q][c] -= (T)alpha[c] * vv[q][c];
+                            zv[c] = di[q] * rv[q][c];
+                        }
+                        stv<2>(V.s, i, rv[q]);
+                        stv<2>(V.z, i, zv);
+                    }
                 }
             }
             cl.sync();
             {   // t = A z, omega = <t, s> / <t, t>
                 T acc[4] = {T(0), T(0), T(0), T(0)};
-                for (int sl = crank * nwarp + wid; sl < A.nslices; sl += csize * nwarp) {
-                    const int i = sl * 32 + lane;
-                    T ax[2];
-                    spmv2_row(A, val, V.z, sl, lane, ax);
-                    if (i < n) {
+                for (int s0 = crank * nwarp + wid; s0 < A.nslices; s0 += U * csize * nwarp) {
+                    int sl[U];
 #pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            if (done[c]) continue;
-                            V.t[2 * i + c] = ax[c];
-                            acc[c] += ax[c] * V.s[2 * i + c];
-                            acc[2 + c] += ax[c] * ax[c];
+                    for (int q = 0; q < U; ++q) sl[q] = s0 + q * csize * nwarp;
+                    T ax[U][2];
+                    spmv_slices<U, 2>(A, val, V.z, sl, lane, ax);
+#pragma unroll
+                    for (int q = 0; q < U; ++q) {
+                        const int i = sl[q] * 32 + lane;
+                        if (i < n) {
+                            T sv[2];
+                            ldv<2>(V.s, i, sv);
+                            stv<2>(V.t, i, ax[q]);
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                acc[c] += ax[q][c] * sv[c];
+                                acc[2 + c] += ax[q][c] * ax[q][c];
+                            }
                         }
                     }
                 }
@@ -288,15 +502,34 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
             }
             {   // x += alpha y + omega z, r = s - omega t, <rhat, r>, <r, r>
                 T acc[4] = {T(0), T(0), T(0), T(0)};
-                for (int i = tid; i < n; i += nthr) {
+                for (int i0 = tid; i0 < n; i0 += R2 * nthr) {
+                    T xv[R2][2], yv[R2][2], zv[R2][2], sv[R2][2], tv[R2][2], rh[R2][2];
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        if (done[c]) continue;
-                        V.x[2 * i + c] += (T)alpha[c] * V.y[2 * i + c] + (T)omega[c] * V.z[2 * i + c];
-                        const T rv = V.s[2 * i + c] - (T)omega[c] * V.t[2 * i + c];
-                        V.r[2 * i + c] = rv;
-                        acc[c] += V.rhat[2 * i + c] * rv;
-                        acc[2 + c] += rv * rv;
+                    for (int q = 0; q < R2; ++q) {
+                        const int i = i0 + q * nthr;
+                        if (i < n) {
+                            ldv<2>(V.x, i, xv[q]);
+                            ldv<2>(V.y, i, yv[q]);
+                            ldv<2>(V.z, i, zv[q]);
+                            ldv<2>(V.s, i, sv[q]);
+                            ldv<2>(V.t, i, tv[q]);
+                            ldv<2>(V.rhat, i, rh[q]);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < R2; ++q) {
+                        const int i = i0 + q * nthr;
+                        if (i < n) {
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) {
+                                if (!done[c]) xv[q][c] += (T)alpha[c] * yv[q][c] + (T)omega[c] * zv[q][c];
+                                sv[q][c] -= (T)omega[c] * tv[q][c];
+                                acc[c] += rh[q][c] * sv[q][c];
+                                acc[2 + c] += sv[q][c] * sv[q][c];
+                            }
+                            stv<2>(V.x, i, xv[q]);
+                            stv<2>(V.r, i, sv[q]);
+                        }
                     }
                 }
                 const double accd[4] = {(double)acc[0], (double)acc[1], (double)acc[2], (double)acc[3]};
@@ -341,11 +574,15 @@ __device__ int cluster_bicgstab(const SellView& A, const T* __restrict__ val, co
     return it;
 }
 
-static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArgs* __restrict__ args,
-                                                                         int ninst, unsigned int* queue) {
+// (the phases are calls: inlined side by side they spilled 1.6 KB a thread)
+static __device__ __noinline__ void coarse_pcg_call(const CoarsePcgArgs& a, ClusterSync& sy) { coarse_pcg_body(a, sy); }
+
+static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArgs* __restrict__ args, int ninst,
+                                                              unsigned int* queue, int dyn_floats) {
+    extern __shared__ float dyn[];   // the coarse CG's vectors (inner_cg_shared)
     __shared__ ClusterShared<512> sm;
     __shared__ int job;
-    ClusterSync sy(sm);
+    ClusterSync sy(sm, dyn_floats ? dyn : nullptr, dyn_floats);
     ClusterSync& cs = sy;
     cgrp_bs::cluster_group& cl = sy.cluster;
     const int crank = (int)cl.block_rank(), csize = (int)cl.num_blocks();
@@ -391,6 +628,7 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
             cl.sync();
             const BicgVecsT<float> W{a.fv[0], a.fv[1], a.fv[2], a.fv[3], a.fv[4], a.fv[5], a.fv[6], a.fv[7], a.fv[8]};
             float* r32 = a.fv[9];
+            double far_last = INFINITY;
             for (int sw = 0; sw < kBatchIrSweeps; ++sw) {
                 double acc[4] = {0.0, 0.0, 0.0, 0.0};
                 for (int sl = crank * nwarp + wid; sl < a.Af.nslices; sl += csize * nwarp) {
@@ -420,6 +658,11 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
                     polish = false;
                     break;
                 }
+                // a sweep that gained less than a decade is the last (components of one matrix:
+                // the larger residual relative to its target decides)
+                const double far = fmax(bb[0] > 0.0 ? rr[0] / bb[0] : 0.0, bb[1] > 0.0 ? rr[1] / bb[1] : 0.0);
+                if (far > 0.01 * far_last) break;
+                far_last = far;
                 // the inner solve aims at kBatchInnerTol, or at what is left to the tolerance
                 // (a factor 2 of margin in the norm) when that is less
                 double t2 = kBatchInnerTol * kBatchInnerTol, need = 1.0;
@@ -472,7 +715,7 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
             if (crank == 0 && threadIdx.x == 0) a.ks[KS_POIS].mean = a.pure_neumann ? tot[0] / a.Ac.n : 0.0;
             cl.sync();
         }
-        coarse_pcg_body(a.coarse, sy);   // ends with a cluster barrier
+        coarse_pcg_call(a.coarse, sy);   // ends with a cluster barrier
         // ---- Eq. 24: prolongation, one level after the other
         for (int l = 0; l + 1 < a.nlev; ++l) {
             const int nc_l = a.nv[l], n_new = a.nv[l + 1] - a.nv[l];
@@ -497,8 +740,15 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
             }
         }
         cl.sync();
-        if (!a.lumped)
-            cluster_chebyshev<2>(a.Af, a.M0, a.dinvM0, a.g, a.delta, a.c0, a.c1, a.c2, a.cheb_steps, crank, csize, cl);
+        int it_corr = 0, it_mass = 0;   // Chebyshev steps
+        if (!a.lumped) {
+            if (!(a.A32 && cluster_cheb_mixed<2>(a.Af, a.M0, a.M0f, a.dinvM0f, a.g, a.delta, a.fv[0], a.fv[1], a.fv[2],
+                                                 a.fv[3], a.tol_mass2, cs, crank, csize, cl, it_corr))) {
+                cluster_chebyshev<2>(a.Af, a.M0, a.dinvM0, a.g, a.delta, a.c0, a.c1, a.c2, a.cheb_steps, crank, csize,
+                                     cl);
+                it_corr += a.cheb_steps;
+            }
+        }
         // ---- Eq. 26: the rotational term q with M q = D U~ (or its lumped form)
         if (a.chi) {
             for (int sl = crank * nwarp + wid; sl < a.Af.nslices; sl += csize * nwarp) {
@@ -513,9 +763,14 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
                 }
             }
             cl.sync();
-            if (!a.lumped)
-                cluster_chebyshev<1>(a.Af, a.M, a.dinvM, a.div, a.qrot, a.c0, a.c1, a.c2, a.cheb_steps, crank, csize,
-                                     cl);
+            if (!a.lumped) {
+                if (!(a.A32 && cluster_cheb_mixed<1>(a.Af, a.M, a.Mf, a.dinvMf, a.div, a.qrot, a.fv[0], a.fv[1], a.fv[2],
+                                                     a.fv[3], a.tol_mass2, cs, crank, csize, cl, it_mass))) {
+                    cluster_chebyshev<1>(a.Af, a.M, a.dinvM, a.div, a.qrot, a.c0, a.c1, a.c2, a.cheb_steps, crank, csize,
+                                         cl);
+                    it_mass += a.cheb_steps;
+                }
+            }
         }
         // ---- end of the step
         for (int i = tid; i < nf; i += nthr) {
@@ -540,8 +795,7 @@ static __global__ void __launch_bounds__(512, 1) k_batch_step(const BatchStepArg
             DeviceStats* st = a.stats;
             st->steps += 1;
             st->sum_outer += ks[KS_POIS].pad[0];
-            const int its[KS_COUNT] = {it, ks[KS_POIS].iter, a.lumped ? 0 : a.cheb_steps,
-                                       (a.chi && !a.lumped) ? a.cheb_steps : 0};
+            const int its[KS_COUNT] = {it, ks[KS_POIS].iter, it_corr, it_mass};
             for (int k = 0; k < KS_COUNT; ++k) {
                 st->last_it[k] = its[k];
                 st->sum_it[k] += its[k];

@@ -28,6 +28,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "krylov.cuh"
 
 namespace cgp {
@@ -143,10 +145,13 @@ struct ClusterSync {
     int cols;                                    // columns of part
     double (*slots)[kSumMax][kMaxClusterCtas];
     SumShared* res;
+    float* dyn;        // dynamic shared memory for inner_cg_shared (null: none), and its floats
+    int dyn_floats;
     int slot = 0;
     template <int T>
-    __device__ explicit ClusterSync(ClusterShared<T>& sm)
-        : cluster(cgrp::this_cluster()), part(&sm.part[0][0]), cols(T), slots(sm.slots), res(&sm.res) {}
+    __device__ explicit ClusterSync(ClusterShared<T>& sm, float* d = nullptr, int nd = 0)
+        : cluster(cgrp::this_cluster()), part(&sm.part[0][0]), cols(T), slots(sm.slots), res(&sm.res), dyn(d),
+          dyn_floats(nd) {}
     __device__ int rank() const { return (int)cluster.block_rank(); }
     __device__ int ranks() const { return (int)cluster.num_blocks(); }
     __device__ bool sync() {
@@ -518,6 +523,102 @@ __device__ bool inner_pcg_classic(const CoarsePcgArgs& a, Sync& sy, const InnerV
     return true;
 }
 
+// Floats of shared memory inner_cg_shared needs per CTA: u of all rows, and r, w, p, s, e of
+// the CTA's own.
+__host__ __device__ inline int shared_cg_floats(int nslices, int ctas) {
+    return 32 * nslices + 5 * 32 * ((nslices + ctas - 1) / ctas);
+}
+
+// Inner FP32 CG of one cluster with its vectors in shared memory, in Chronopoulos and Gear's
+// form with w = A u formed every iteration: every CTA holds u of all rows, and a row's owner
+// stores its new u into every CTA (distributed shared memory), so the SpMV gathers locally;
+// r, w, p, s, e of the own rows stay in the CTA, the matrix streams through L1.  One reduction
+// and one plain cluster barrier per iteration.  (inner_pcg_classic, with its vectors in global
+// memory and two reductions, took 16k clocks an iteration on at most 1,089 rows and 22k on
+// 4,225, on 8 CTAs.)  Dot products are accumulated in FP64 as there; same outcome codes.
+__device__ inline void inner_cg_shared(const CoarsePcgArgs& a, ClusterSync& sy, const InnerVecs<float>& V, int s_begin,
+                                       int s_end, double gamma, double stop2, int& iters, int& outcome) {
+    outcome = 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5, ncl = sy.ranks();
+    const SellView& A = a.A;
+    const int own = 32 * ((A.nslices + ncl - 1) / ncl);
+    float* const u = sy.dyn;
+    float* const r = u + 32 * A.nslices;
+    float *const w = r + own, *const p = w + own, *const s = p + own, *const e = s + own;
+    auto publish = [&](int i, float v) {
+        for (int c = 0; c < ncl; ++c) sy.cluster.map_shared_rank(u, c)[i] = v;
+    };
+    for (int sl = s_begin + wid; sl < s_end; sl += nw) {
+        const int i = sl * 32 + lane, l = i - 32 * s_begin;
+        const bool in = i < A.n;
+        r[l] = in ? ldcg(V.r + i) : 0.0f;
+        p[l] = s[l] = e[l] = 0.0f;
+        publish(i, in ? ldcg(V.u + i) : 0.0f);
+    }
+    sy.sync();
+    double d = 0.0, rg = 0.0, c = 0.0, rr_best = INFINITY, part[3] = {0.0, 0.0, 0.0};
+    int best_k = 0;
+    for (int k = 0;; ++k) {
+        if (wid == 0 && k) {   // 1 / gamma' and d' / gamma'^2, off the reduction's chain
+            rg = 1.0 / gamma;
+            c = d * rg * rg;
+        }
+        for (int sl = s_begin + wid; sl < s_end; sl += nw) {
+            const int i = sl * 32 + lane, l = i - 32 * s_begin;
+            const float wv = sell_accum_f(A, a.valf, sl, lane, [&](int j) { return u[j]; });
+            w[l] = wv;
+            if (i < A.n) part[1] += (double)wv * (double)u[i];
+        }
+        // out: alpha, beta, gamma, d; flag: 0 go on, else 1 + outcome
+        double o[4];
+        int flag;
+        const double gamma0 = gamma;
+        sy.sum_to(part, o, flag, [&](const double (&t)[3], double (&q)[4]) -> int {
+            const double tg = k ? t[0] : gamma0, trr = k ? t[2] : INFINITY;
+            q[3] = t[1] - tg * tg * c;
+            q[2] = tg;
+            q[1] = tg * rg;
+            q[0] = tg / q[3];
+            if (k && !(isfinite(t[0]) && isfinite(t[1]) && isfinite(t[2]))) return 3;
+            if (k && (t[0] == 0.0 || trr <= stop2)) return 1;
+            if (trr < 0.5 * rr_best) {
+                rr_best = trr;
+                best_k = k;
+            } else if (trr > 1e4 * rr_best) {
+                return 3;   // the FP32 recurrence is drifting away: its iterate is not to be used
+            }
+            if (!isfinite(q[0]) || q[0] == 0.0) return 2;
+            return k - best_k > kStagnation32 || iters >= a.maxit ? 1 : 0;
+        });
+        if (flag) {
+            outcome = flag - 1;
+            break;
+        }
+        gamma = o[2];
+        d = o[3];
+        const float al = (float)o[0], be = (float)o[1];
+        part[0] = part[1] = part[2] = 0.0;
+        for (int sl = s_begin + wid; sl < s_end; sl += nw) {
+            const int i = sl * 32 + lane, l = i - 32 * s_begin;
+            const float pv = fmaf(be, p[l], u[i]), sv = fmaf(be, s[l], w[l]);
+            const float rv = fmaf(-al, sv, r[l]), uv = i < A.n ? __ldg(a.dinvf + i) * rv : 0.0f;
+            p[l] = pv;
+            s[l] = sv;
+            e[l] = fmaf(al, pv, e[l]);
+            r[l] = rv;
+            publish(i, uv);
+            part[0] += (double)rv * (double)uv;
+            part[2] += (double)rv * (double)rv;
+        }
+        ++iters;
+        sy.sync();   // u is complete before it is gathered
+    }
+    for (int sl = s_begin + wid; sl < s_end; sl += nw) {
+        const int i = sl * 32 + lane;
+        if (i < A.n) __stcg(V.e + i, e[i - 32 * s_begin]);
+    }
+}
+
 template <class Sync>
 __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -619,7 +720,16 @@ __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
         int outcome = 0;
         if (mixed_now) {
             const double stop2 = fmax(a.inner_tol * a.inner_tol * rr0, 0.25 * tol2 * bb);
-            ok = inner_pcg_classic<float>(a, sy, V32, a.dinvf, s_begin, s_end, tot[2], stop2, iters, outcome);
+            bool shared = false;
+            if constexpr (std::is_same<Sync, ClusterSync>::value)
+                shared = sy.dyn && shared_cg_floats(A.nslices, parts) <= sy.dyn_floats;
+            if (shared) {
+                if constexpr (std::is_same<Sync, ClusterSync>::value)
+                    inner_cg_shared(a, sy, V32, s_begin, s_end, tot[2], stop2, iters, outcome);
+                ok = true;
+            } else {
+                ok = inner_pcg_classic<float>(a, sy, V32, a.dinvf, s_begin, s_end, tot[2], stop2, iters, outcome);
+            }
         } else {
             // FP64: the inner recurrence updates x itself; the next outer pass re-checks the true residual
             ok = inner_pcg(a, sy, V64, a.dinv, s_begin, s_end, tot[2], 0.25 * tol2 * bb, iters, outcome);

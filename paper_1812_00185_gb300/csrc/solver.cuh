@@ -155,9 +155,10 @@ int launch_batch_coarse(const void* d_args, int ninst, unsigned int* queue, int 
 size_t batch_step_args_size();
 bool batch_step_eligible(const Solver& s);
 void fill_batch_step_args(Solver& s, void* dst);
-int batch_step_clusters(int csize, int threads, int* nclusters);
-int launch_batch_step(const void* d_args, int ninst, unsigned int* queue, int csize, int threads, int nclusters,
-                      cudaStream_t st);
+int batch_step_shared(Solver* const* inst, int ninst, int csize, int* floats);
+int batch_step_clusters(int csize, int threads, int floats, int* nclusters);
+int launch_batch_step(const void* d_args, int ninst, unsigned int* queue, int csize, int threads, int floats,
+                      int nclusters, cudaStream_t st);
 int choose_coarse_solver(Solver& s, cudaStream_t st);
 int init_state(Solver* s, cudaStream_t st);
 

@@ -1425,6 +1425,11 @@ void fill_batch_step_args(Solver& s, void* dst) {
         a.dinvA32 = s.dinvAf;
         for (int k = 0; k < 9; ++k) a.fv[k] = s.fv[k];
         a.fv[9] = s.frhs;
+        a.M0f = s.M0f;
+        a.Mf = s.Mf;
+        a.dinvM0f = s.dinvM0f;
+        a.dinvMf = s.dinvMf;
+        a.tol_mass2 = s.prm.tol_mass * s.prm.tol_mass;
     }
     a.tdev = s.tdev;
     a.stats = s.stats;
@@ -1432,15 +1437,33 @@ void fill_batch_step_args(Solver& s, void* dst) {
     memcpy(dst, &a, sizeof(a));
 }
 
-int batch_step_clusters(int csize, int threads, int* nclusters) {
-    static bool attr_set = false;
-    if (!attr_set) {
-        CGP_CUDA(cudaFuncSetAttribute(k_batch_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        attr_set = true;
+// dynamic shared memory of the launch: the largest need of a mixed instance's coarse CG that
+// fits beside the kernel's static arrays (instances beyond it keep their vectors in memory)
+int batch_step_shared(Solver* const* inst, int ninst, int csize, int* floats) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    CGP_CUDA(cudaGetDevice(&dev));
+    CGP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CGP_CUDA(cudaFuncGetAttributes(&fa, k_batch_step));
+    const int most = (optin - (int)fa.sharedSizeBytes - 1024) / (int)sizeof(float);
+    *floats = 0;
+    for (int i = 0; i < ninst; ++i) {
+        const Solver& s = *inst[i];
+        if (s.coarse_fp64) continue;
+        const int need = shared_cg_floats(s.mesh->lev[s.lc].nslices, csize);
+        if (need <= most && need > *floats) *floats = need;
     }
+    CGP_CUDA(cudaFuncSetAttribute(k_batch_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CGP_CUDA(cudaFuncSetAttribute(k_batch_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  most * (int)sizeof(float)));
+    return CGP_OK;
+}
+
+int batch_step_clusters(int csize, int threads, int floats, int* nclusters) {
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(csize, nullptr, attr);
     cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = floats * sizeof(float);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k_batch_step, &cfg) != cudaSuccess) {
         cudaGetLastError();
@@ -1450,14 +1473,15 @@ int batch_step_clusters(int csize, int threads, int* nclusters) {
     return CGP_OK;
 }
 
-int launch_batch_step(const void* d_args, int ninst, unsigned int* queue, int csize, int threads, int nclusters,
-                      cudaStream_t st) {
+int launch_batch_step(const void* d_args, int ninst, unsigned int* queue, int csize, int threads, int floats,
+                      int nclusters, cudaStream_t st) {
     CGP_CUDA(cudaMemsetAsync(queue, 0, sizeof(unsigned int), st));
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = cluster_config(csize, st, attr);
     cfg.gridDim = dim3(csize * nclusters, 1, 1);
     cfg.blockDim = dim3(threads, 1, 1);
-    CGP_CUDA(cudaLaunchKernelEx(&cfg, k_batch_step, (const BatchStepArgs*)d_args, ninst, queue));
+    cfg.dynamicSmemBytes = floats * sizeof(float);
+    CGP_CUDA(cudaLaunchKernelEx(&cfg, k_batch_step, (const BatchStepArgs*)d_args, ninst, queue, floats));
     return CGP_OK;
 }
 
