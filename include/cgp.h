@@ -280,7 +280,7 @@ enum {
     CGP_PROF_F32_BICG_V, CGP_PROF_F32_BICG_S, CGP_PROF_F32_BICG_T, CGP_PROF_F32_BICG_X,
     /* p updates of the FP64 PCG loops (three kernels per iteration) */
     CGP_PROF_POIS_PUPD, CGP_PROF_CORR_PUPD, CGP_PROF_MASS_PUPD,
-    /* CGP_MIXED: FP32 Chebyshev steps of the Eq. 26 and Eq. 25 mass-matrix solves */
+    /* Chebyshev steps of the Eq. 26 and Eq. 25 mass-matrix solves (FP32 in CGP_MIXED, else FP64) */
     CGP_PROF_CHEB_MASS, CGP_PROF_CHEB_CORR,
     /* projection guess of the coarse solve (CGP_GUESS_PROJ, CGP_GUESS_LEARNED) */
     CGP_PROF_PROJ, CGP_PROF_COUNT
