@@ -130,8 +130,9 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * subdomains (phi = 0 vertices in none) and E^+ the pseudo-inverse of E = Z^T K_c Z, built
  * once at cgp_assemble; asked for by name, only the ONCHIP coarse solver has it (cgp_assemble
  * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs, the same
- * correction in FP64 (one subdomain per CTA) in the register-resident PERSISTENT solve, JACOBI
- * elsewhere.  The solution is the same to the solve's tolerance; only the iteration count
+ * correction in FP64 in the PERSISTENT solve of more than one cluster (one subdomain per CTA,
+ * or about one per SM where the vectors stay in memory, up to 4 million rows and not with the
+ * learned guess), JACOBI elsewhere.  The solution is the same to the solve's tolerance; only the iteration count
  * changes. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 

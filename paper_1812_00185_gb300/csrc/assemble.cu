@@ -169,6 +169,18 @@ static int layout(Solver& s, void* base, size_t* bytes) {
         const size_t ctas = std::min<size_t>(kRRMaxSub, (size_t)C.nslices / 8 + 16);
         s.rr_perm = cv.take<int32_t>(32 * ((size_t)C.nslices + 16 * ctas));
         s.rr_einv = cv.take<double>(ctas * ctas);
+        if (gp_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
+            const size_t slots = gp_slots(nc), ent = gp_entries(nnzc);
+            s.gp_perm = cv.take<int32_t>(slots);
+            s.gp_slot = cv.take<int32_t>(nc);
+            s.gp_ptr = cv.take<int32_t>(slots / 32 + 1);
+            s.gp_first = cv.take<int32_t>((size_t)s.max_grid + 1);
+            s.gp_col = cv.take<int32_t>(ent);
+            s.gp_val = cv.take<double>(ent);
+            s.gp_dinv = cv.take<double>(slots);
+            s.gp_einv = cv.take<double>((size_t)kRRMaxSub * kRRMaxSub);
+            s.gp_vec = cv.take<double>(6 * slots);
+        }
     }
     if (s.prm.guess == CGP_GUESS_LEARNED) {
         s.phi_guess = cv.take<double>(nc);

@@ -1,7 +1,9 @@
-// Host plan of the register-resident FP64 coarse solve (see rr_plan.cuh).
+// Host plans of the FP64 coarse solves over compact subdomains (see rr_plan.cuh).
 #include <algorithm>
 #include <cmath>
-#include <numeric>
+#include <system_error>
+#include <thread>
+#include <utility>
 
 #include "rr_plan.cuh"
 
@@ -9,9 +11,14 @@ namespace cgp {
 
 namespace {
 
-// assigns idx[lo, hi) to the parts p0 .. p1 - 1, at most `cap` each
-void bisect(std::vector<int32_t>& idx, const std::vector<double>& xy, int lo, int hi, int p0, int p1, int cap,
-            std::vector<int32_t>& first) {
+struct Point {
+    double x[2];
+    int32_t id;
+};
+
+// p[lo, hi) into the parts p0 .. p1 - 1 of at most `cap` points, halving the longer side of the
+// bounding box.  The two halves of a large piece go to two threads.
+void bisect(Point* p, int lo, int hi, int p0, int p1, int cap, int32_t* first) {
     if (p1 - p0 == 1) {
         first[p0] = lo;
         return;
@@ -19,9 +26,8 @@ void bisect(std::vector<int32_t>& idx, const std::vector<double>& xy, int lo, in
     double mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
     for (int k = lo; k < hi; ++k)
         for (int d = 0; d < 2; ++d) {
-            const double v = xy[2 * (size_t)idx[k] + d];
-            mn[d] = std::min(mn[d], v);
-            mx[d] = std::max(mx[d], v);
+            mn[d] = std::min(mn[d], p[k].x[d]);
+            mx[d] = std::max(mx[d], p[k].x[d]);
         }
     const int axis = mx[1] - mn[1] > mx[0] - mn[0] ? 1 : 0;
     const int parts = p1 - p0, left = parts / 2, here = hi - lo;
@@ -29,47 +35,47 @@ void bisect(std::vector<int32_t>& idx, const std::vector<double>& xy, int lo, in
     take = std::max<int64_t>(take, here - (int64_t)cap * (parts - left));
     take = std::min<int64_t>(take, (int64_t)cap * left);
     const int mid = lo + (int)take;
-    std::nth_element(idx.begin() + lo, idx.begin() + mid, idx.begin() + hi, [&](int32_t a, int32_t b) {
-        const double x = xy[2 * (size_t)a + axis], y = xy[2 * (size_t)b + axis];
-        return x < y || (x == y && a < b);
+    std::nth_element(p + lo, p + mid, p + hi, [axis](const Point& a, const Point& b) {
+        return a.x[axis] < b.x[axis] || (a.x[axis] == b.x[axis] && a.id < b.id);
     });
-    bisect(idx, xy, lo, mid, p0, p0 + left, cap, first);
-    bisect(idx, xy, mid, hi, p0 + left, p1, cap, first);
-}
-
-}  // namespace
-
-bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
-             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
-             const std::vector<uint8_t>& in_space, int ctas, int threads, bool neumann, RRHostPlan& P) {
-    P = RRHostPlan{};
-    const int m = ctas;
-    if (m < 2 || m > kRRMaxSub || (int64_t)m * threads < n) return false;
-    std::vector<int32_t> idx(n), first(m + 1, n), sub(n);
-    std::iota(idx.begin(), idx.end(), 0);
-    bisect(idx, xy, 0, n, 0, m, threads, first);
-    std::vector<int32_t> perm((size_t)m * threads, -1);
-    for (int c = 0; c < m; ++c) {
-        // rows of one length side by side, so that a warp's lanes have the same entry count
-        std::sort(idx.begin() + first[c], idx.begin() + first[c + 1], [&](int32_t a, int32_t b) {
-            const int la = rowptr[a + 1] - rowptr[a], lb = rowptr[b + 1] - rowptr[b];
-            return la > lb || (la == lb && a < b);
-        });
-        for (int k = first[c]; k < first[c + 1]; ++k) {
-            const int i = idx[k];
-            sub[i] = in_space[i] ? c : -1;
-            perm[(size_t)c * threads + (k - first[c])] = in_space[i] ? i : -2 - i;
+    std::thread other;
+    if (here > 100000) {
+        try {
+            other = std::thread(bisect, p, lo, mid, p0, p0 + left, cap, first);
+        } catch (const std::system_error&) {   // no thread to be had: one after the other
         }
     }
+    if (!other.joinable()) bisect(p, lo, mid, p0, p0 + left, cap, first);
+    bisect(p, mid, hi, p0 + left, p1, cap, first);
+    if (other.joinable()) other.join();
+}
+
+std::vector<Point> points(int n, const std::vector<double>& xy) {
+    std::vector<Point> p(n);
+    for (int i = 0; i < n; ++i) p[i] = {{xy[2 * (size_t)i], xy[2 * (size_t)i + 1]}, i};
+    return p;
+}
+
+// E = Z^T K Z of the subdomains sub[i] (-1: outside the space)
+std::vector<double> galerkin(int n, int m, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
+                             const std::vector<int32_t>& sell_col, const std::vector<double>& val,
+                             const std::vector<int32_t>& sub) {
     std::vector<double> E((size_t)m * m, 0.0);
     for (int i = 0; i < n; ++i) {
         if (sub[i] < 0) continue;
+        double* row = E.data() + (size_t)sub[i] * m;
         for (int k = 0; k < rowptr[i + 1] - rowptr[i]; ++k) {
             const int64_t e = (int64_t)sell_ptr[i >> 5] + 32 * k + (i & 31);
             const int j = sub[sell_col[e]];
-            if (j >= 0) E[(size_t)sub[i] * m + j] += val[e];
+            if (j >= 0) row[j] += val[e];
         }
     }
+    return E;
+}
+
+// pseudo-inverse of the Galerkin matrix E (neumann: constants are its null space); false when a
+// pivot is not safely positive
+bool inverse(int m, std::vector<double> E, bool neumann, std::vector<double>& inv) {
     double trace = 0.0;
     for (int j = 0; j < m; ++j) trace += E[(size_t)j * m + j];
     if (!(trace > 0.0) || !std::isfinite(trace)) return false;
@@ -98,7 +104,8 @@ bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
             }
         }
     }
-    std::vector<double> inv((size_t)m * m), y(m);
+    inv.assign((size_t)m * m, 0.0);
+    std::vector<double> y(m);
     for (int c = 0; c < m; ++c) {
         for (int j = 0; j < m; ++j) {
             double s = j == c ? 1.0 : 0.0;
@@ -118,8 +125,113 @@ bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
                 0.5 * (inv[(size_t)j * m + k] + inv[(size_t)k * m + j]);
     for (double x : inv)
         if (!std::isfinite(x)) return false;
+    return true;
+}
+
+}  // namespace
+
+bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
+             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
+             const std::vector<uint8_t>& in_space, int ctas, int threads, bool neumann, RRHostPlan& P) {
+    P = RRHostPlan{};
+    const int m = ctas;
+    if (m < 2 || m > kRRMaxSub || (int64_t)m * threads < n) return false;
+    std::vector<Point> pts = points(n, xy);
+    std::vector<int32_t> first(m + 1, n), sub(n);
+    bisect(pts.data(), 0, n, 0, m, threads, first.data());
+    std::vector<int32_t> perm((size_t)m * threads, -1);
+    for (int c = 0; c < m; ++c) {
+        // rows of one length side by side, so that a warp's lanes have the same entry count
+        std::sort(pts.begin() + first[c], pts.begin() + first[c + 1], [&](const Point& a, const Point& b) {
+            const int la = rowptr[a.id + 1] - rowptr[a.id], lb = rowptr[b.id + 1] - rowptr[b.id];
+            return la > lb || (la == lb && a.id < b.id);
+        });
+        for (int k = first[c]; k < first[c + 1]; ++k) {
+            const int i = pts[k].id;
+            sub[i] = in_space[i] ? c : -1;
+            perm[(size_t)c * threads + (k - first[c])] = in_space[i] ? i : -2 - i;
+        }
+    }
+    std::vector<double> inv;
+    if (!inverse(m, galerkin(n, m, rowptr, sell_ptr, sell_col, val, sub), neumann, inv)) return false;
     P.nsub = m;
     P.perm.swap(perm);
+    P.einv.swap(inv);
+    return true;
+}
+
+bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
+             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
+             const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P) {
+    P = GpHostPlan{};
+    const int m = std::min(nsub, kRRMaxSub);
+    if (m < 2 || n < 32 * m) return false;
+    std::vector<Point> pts = points(n, xy);
+    std::vector<int32_t> first(m + 1, n), sub(n);
+    bisect(pts.data(), 0, n, 0, m, (n + m - 1) / m + 1, first.data());
+    for (int c = 0; c < m; ++c)
+        for (int k = first[c]; k < first[c + 1]; ++k) sub[pts[k].id] = in_space[pts[k].id] ? c : -1;
+    std::vector<double> inv;
+    if (!inverse(m, galerkin(n, m, rowptr, sell_ptr, sell_col, val, sub), neumann, inv)) return false;
+    // the order within a subdomain: rows longer than most first (their slices are wider), then by
+    // the cells of a grid of about 48 rows each, so that a slice's columns lie close together
+    std::vector<int64_t> hist(64, 0);
+    for (int i = 0; i < n; ++i) ++hist[std::min(63, rowptr[i + 1] - rowptr[i])];
+    const int usual = (int)(std::max_element(hist.begin(), hist.end()) - hist.begin());
+    P.slot_of.assign(n, 0);
+    P.ptr.push_back(0);
+    std::vector<int32_t> slices(m + 1, 0), key, count;
+    for (int c = 0; c < m; ++c) {
+        const int lo = first[c], rows = first[c + 1] - lo;
+        double mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
+        for (int k = lo; k < lo + rows; ++k)
+            for (int d = 0; d < 2; ++d) {
+                mn[d] = std::min(mn[d], pts[k].x[d]);
+                mx[d] = std::max(mx[d], pts[k].x[d]);
+            }
+        const int side = std::max(1, (int)std::sqrt(rows / 48.0));
+        auto cell = [&](int k, int d) {
+            const double w = mx[d] - mn[d];
+            return w > 0.0 ? std::min(side - 1, (int)((pts[k].x[d] - mn[d]) / w * side)) : 0;
+        };
+        key.assign(rows, 0);
+        count.assign(2 * side * side + 1, 0);
+        for (int k = 0; k < rows; ++k) {
+            const int cx = cell(lo + k, 0), cy = cell(lo + k, 1), len = rowptr[pts[lo + k].id + 1] - rowptr[pts[lo + k].id];
+            key[k] = (len > usual ? 0 : side * side) + cy * side + (cy & 1 ? side - 1 - cx : cx);
+            ++count[key[k] + 1];
+        }
+        for (size_t q = 1; q < count.size(); ++q) count[q] += count[q - 1];
+        const int s0 = (int)P.ptr.size() - 1, ns = (rows + 31) / 32;
+        P.perm.resize(32 * (size_t)(s0 + ns), -1);
+        for (int k = 0; k < rows; ++k) {
+            const int slot = 32 * s0 + count[key[k]]++;
+            P.perm[slot] = pts[lo + k].id;
+            P.slot_of[pts[lo + k].id] = slot;
+        }
+        for (int q = 0; q < ns; ++q) {
+            int w = 0;
+            for (int l = 0; l < 32; ++l) {
+                const int i = P.perm[32 * (size_t)(s0 + q) + l];
+                if (i >= 0) w = std::max(w, rowptr[i + 1] - rowptr[i]);
+            }
+            const int64_t end = (int64_t)P.ptr.back() + 32 * w;
+            if (end > INT32_MAX) {
+                P = GpHostPlan{};
+                return false;
+            }
+            P.ptr.push_back((int32_t)end);
+        }
+        slices[c + 1] = s0 + ns;
+    }
+    P.nslices = (int)P.ptr.size() - 1;
+    // CTAs per subdomain: as many as give every warp of theirs a slice
+    P.per = std::max(1, std::min(max_per, P.nslices / (8 * m)));
+    for (int c = 0; c < m; ++c)
+        for (int q = 0; q < P.per; ++q)
+            P.first.push_back(slices[c] + (int32_t)((int64_t)(slices[c + 1] - slices[c]) * q / P.per));
+    P.first.push_back(P.nslices);
+    P.nsub = m;
     P.einv.swap(inv);
     return true;
 }

@@ -1,5 +1,6 @@
-// Host plan of the register-resident FP64 coarse solve (coarse_rr.cuh): which row every thread
-// holds, and the coarse space of its preconditioner.
+// Host plans of the FP64 coarse solves over compact subdomains: the register-resident one
+// (coarse_rr.cuh: which row every thread holds) and the memory-resident one (coarse_gp.cuh: the
+// order of the rows), with the coarse space of their preconditioner.
 #pragma once
 
 #include <cstdint>
@@ -8,6 +9,14 @@
 namespace cgp {
 
 constexpr int kRRMaxSub = 160;   // subdomains (one per CTA): five per lane of a warp
+
+// The memory-resident solve has a plan for systems of more slices than any launch of the
+// register-resident one holds by design (16 per SM of about 150), up to a size whose host plan
+// (about 0.1 s per million rows, once per solver) is soon earned back.
+constexpr int kGpMinSlices = 2048, kGpMaxSlices = 1 << 17;
+inline bool gp_wanted(int nslices) { return nslices > kGpMinSlices && nslices <= kGpMaxSlices; }
+inline size_t gp_slots(int64_t n) { return (size_t)n + 32 * (size_t)kRRMaxSub; }
+inline size_t gp_entries(int64_t nnz_sell) { return (size_t)nnz_sell + (size_t)nnz_sell / 4 + 32 * 64 * (size_t)kRRMaxSub; }
 
 struct RRHostPlan {
     int nsub = 0;                  // 0: no plan (the slices in order, Jacobi alone)
@@ -23,5 +32,21 @@ struct RRHostPlan {
 bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
              const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
              const std::vector<uint8_t>& in_space, int ctas, int threads, bool neumann, RRHostPlan& P);
+
+// Plan of the memory-resident solve: nsub compact subdomains of whole 32-row slices, `per` CTAs
+// each, and the slices' widths in the new order.
+struct GpHostPlan {
+    int nsub = 0, per = 0, nslices = 0;
+    std::vector<int32_t> perm;      // slot -> row, or -1 (padding)
+    std::vector<int32_t> slot_of;   // row -> slot
+    std::vector<int32_t> ptr;       // nslices + 1: first entry of every slice
+    std::vector<int32_t> first;     // nsub per + 1: first slice of every CTA
+    std::vector<double> einv;
+};
+
+// False (P.nsub = 0) when E is not safely invertible.
+bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
+             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
+             const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P);
 
 }  // namespace cgp

@@ -78,6 +78,10 @@ struct Solver {
     int rr_nsub = 0;              // subdomains of its plan (rr_plan.cuh; 0: Jacobi alone)
     int32_t* rr_perm = nullptr;
     double* rr_einv = nullptr;
+    // plan of the memory-resident FP64 solve (rr_plan.cuh; gp_nsub = 0: none) and its arrays
+    int gp_nsub = 0, gp_ctas = 0, gp_nslices = 0;
+    int32_t *gp_perm = nullptr, *gp_slot = nullptr, *gp_ptr = nullptr, *gp_first = nullptr, *gp_col = nullptr;
+    double *gp_val = nullptr, *gp_dinv = nullptr, *gp_einv = nullptr, *gp_vec = nullptr;
     bool coarse_fp64 = true;
     cudaStream_t branch = nullptr;                 // second stream of a step (work beside the coarse solve)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;      // the coarse solve's inner iterations run in FP64

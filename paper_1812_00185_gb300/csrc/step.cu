@@ -3,8 +3,10 @@
 // Krylov loops are conditional WHILE nodes driven by the kernels themselves.
 #include <algorithm>
 #include <cstring>
+#include <new>
 
 #include "coarse_pcg.cuh"
+#include "coarse_gp.cuh"
 #include "coarse_rr.cuh"
 #include "coarse_onchip.cuh"
 #include "flows.cuh"
@@ -829,6 +831,55 @@ static cudaLaunchConfig_t cluster_config(int csize, cudaStream_t st, cudaLaunchA
     return cfg;
 }
 
+// Host plan of the FP64 coarse solve over compact subdomains (rr_plan.cuh): of the register-
+// resident launch `sh`, or (null) of the memory-resident solve.  No plan (Jacobi alone) where the
+// coarse matrix cannot be inverted safely.
+static int subdomain_plan(Solver& s, const RRShape* sh, int sms, cudaStream_t st) {
+    const Level& C = s.mesh->lev[s.lc];
+    std::vector<int32_t> rowptr(C.nv + 1), ptr(C.nslices + 1), col(C.nnz_sell);
+    std::vector<double> xy(2 * (size_t)C.nv), val(C.nnz_sell);
+    std::vector<uint8_t> in_space(C.nv);
+    CGP_CUDA(cudaStreamSynchronize(st));   // the assembled K_c
+    CGP_CUDA(cudaMemcpy(rowptr.data(), C.rowptr, sizeof(int32_t) * (C.nv + 1), cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(ptr.data(), C.sell_ptr, sizeof(int32_t) * (C.nslices + 1), cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(col.data(), C.sell_col, sizeof(int32_t) * C.nnz_sell, cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(xy.data(), C.xy, sizeof(double) * 2 * C.nv, cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(val.data(), s.Kc0, sizeof(double) * C.nnz_sell, cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(in_space.data(), C.tag, C.nv, cudaMemcpyDeviceToHost));
+    for (auto& t : in_space) t = (t & CGP_PHI_ZERO) ? 0 : 1;
+    auto up = [](auto* dst, const auto& v) {
+        return cudaMemcpy(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
+    };
+    if (sh) {
+        RRHostPlan P;
+        if (!rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh->ctas, 32 * sh->warps, s.pure_neumann, P)) return CGP_OK;
+        CGP_CUDA(up(s.rr_perm, P.perm));
+        CGP_CUDA(up(s.rr_einv, P.einv));
+        s.rr_nsub = P.nsub;
+        return CGP_OK;
+    }
+    int per_sm = 0;
+    CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_grid_plan, kGridThreads, 0));
+    GpHostPlan G;
+    if (per_sm < 1 || !gp_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sms, std::min(per_sm, kGridCtasPerSm),
+                               s.pure_neumann, G))
+        return CGP_OK;
+    if (G.perm.size() > gp_slots(C.nv) || (size_t)G.ptr.back() > gp_entries(C.nnz_sell)) return CGP_OK;
+    CGP_CUDA(up(s.gp_perm, G.perm));
+    CGP_CUDA(up(s.gp_slot, G.slot_of));
+    CGP_CUDA(up(s.gp_ptr, G.ptr));
+    CGP_CUDA(up(s.gp_first, G.first));
+    CGP_CUDA(up(s.gp_einv, G.einv));
+    k_gp_matrix<<<blocks_for((int64_t)G.perm.size()), kBlock, 0, st>>>(
+        (int)G.perm.size(), s.gp_perm, s.gp_slot, C.rowptr, C.sell_ptr, C.sell_col, s.Kc0, s.dinvKc, C.tag, s.gp_ptr,
+        s.gp_col, s.gp_val, s.gp_dinv);
+    CGP_LAUNCH_CHECK();
+    s.gp_nsub = G.nsub;
+    s.gp_ctas = G.nsub * G.per;
+    s.gp_nslices = G.nslices;
+    return CGP_OK;
+}
+
 int choose_coarse_solver(Solver& s, cudaStream_t st) {
     const cgp_params& p = s.prm;
     int mode = p.coarse_mode;
@@ -961,24 +1012,14 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
             // its subdomain plan, where the preconditioner is left to the library.  Not on one
             // cluster: with 16 subdomains the cavity's 33^2 rows took 110 iterations instead of
             // 152, but each 40 % longer (4 steps 6.25 instead of 5.60 ms)
-            s.rr_nsub = 0;
-            if (sh.ctas > kRRSingle && p.precond == CGP_PRECOND_AUTO && !s.onchip_bytes && s.rr_perm) {
-                std::vector<int32_t> rowptr(C.nv + 1), ptr(C.nslices + 1), col(C.nnz_sell);
-                std::vector<double> xy(2 * (size_t)C.nv), val(C.nnz_sell);
-                std::vector<uint8_t> in_space(C.nv);
-                CGP_CUDA(cudaStreamSynchronize(st));   // the assembled K_c
-                CGP_CUDA(cudaMemcpy(rowptr.data(), C.rowptr, sizeof(int32_t) * (C.nv + 1), cudaMemcpyDeviceToHost));
-                CGP_CUDA(cudaMemcpy(ptr.data(), C.sell_ptr, sizeof(int32_t) * (C.nslices + 1), cudaMemcpyDeviceToHost));
-                CGP_CUDA(cudaMemcpy(col.data(), C.sell_col, sizeof(int32_t) * C.nnz_sell, cudaMemcpyDeviceToHost));
-                CGP_CUDA(cudaMemcpy(xy.data(), C.xy, sizeof(double) * 2 * C.nv, cudaMemcpyDeviceToHost));
-                CGP_CUDA(cudaMemcpy(val.data(), s.Kc0, sizeof(double) * C.nnz_sell, cudaMemcpyDeviceToHost));
-                CGP_CUDA(cudaMemcpy(in_space.data(), C.tag, C.nv, cudaMemcpyDeviceToHost));
-                for (auto& t : in_space) t = (t & CGP_PHI_ZERO) ? 0 : 1;
-                RRHostPlan P;
-                if (rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh.ctas, 32 * sh.warps, s.pure_neumann, P)) {
-                    CGP_CUDA(cudaMemcpy(s.rr_perm, P.perm.data(), sizeof(int32_t) * P.perm.size(), cudaMemcpyHostToDevice));
-                    CGP_CUDA(cudaMemcpy(s.rr_einv, P.einv.data(), sizeof(double) * P.einv.size(), cudaMemcpyHostToDevice));
-                    s.rr_nsub = P.nsub;
+            s.rr_nsub = s.gp_nsub = 0;
+            const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm, plan_gp = !sh.ctas && s.gp_perm;
+            const bool fp64 = p.precision == CGP_FP64 || p.coarse_mode == CGP_COARSE_AUTO;   // (as below)
+            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_gp)) {
+                try {
+                    CGP_TRY(subdomain_plan(s, plan_rr ? &sh : nullptr, sms, st));
+                } catch (const std::bad_alloc&) {   // no host memory for the plan: Jacobi alone
+                    s.rr_nsub = s.gp_nsub = 0;
                 }
             }
         }
@@ -1123,7 +1164,8 @@ static int coarse_solve(Ctx& c) {
         }
         CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));   // counter + error word
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(s.coarse_grid, 1, 1);
+        const bool planned = s.gp_nsub && s.coarse_fp64;
+        cfg.gridDim = dim3(planned ? s.gp_ctas : s.coarse_grid, 1, 1);
         cfg.blockDim = dim3(kGridThreads, 1, 1);
         cfg.stream = c.st;
         cudaLaunchAttribute attr[1];
@@ -1131,6 +1173,12 @@ static int coarse_solve(Ctx& c) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+        if (planned) {
+            const GpPlan pl{32 * s.gp_nslices, s.gp_nslices, s.gp_nsub, s.gp_ctas, s.gp_perm, s.gp_ptr, s.gp_col,
+                            s.gp_val, s.gp_dinv, s.gp_first, s.gp_einv, s.gp_vec};
+            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid_plan, a, pl)));
+            return CGP_OK;
+        }
         PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid, a)));
         return CGP_OK;
     }
@@ -1842,7 +1890,7 @@ extern "C" int cgp_coarse_subdomains(const cgp_solver* h, int32_t* nsub) {
         set_error("null solver");
         return CGP_EINVAL;
     }
-    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub : 0);
+    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub + h->s.gp_nsub : 0);
     return CGP_OK;
 }
 
@@ -1863,7 +1911,7 @@ extern "C" int cgp_coarse_info(const cgp_solver* h, int32_t* kind, int32_t* ctas
             n = s.rr_ctas;
         } else {
             k = CGP_COARSE_PERSISTENT_MEM;
-            n = s.coarse_grid;
+            n = s.gp_nsub && s.coarse_fp64 ? s.gp_ctas : s.coarse_grid;
         }
     }
     if (kind) *kind = k;

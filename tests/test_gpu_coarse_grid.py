@@ -46,6 +46,7 @@ CASES = {
     "sq9": lambda: (square_mesh(9), 0), "sq63": lambda: (square_mesh(63), 0),
     "channel": lambda: (channel_cylinder_mesh(seed=2, h=0.05), 2), "sq197": lambda: (square_mesh(197), 0),
     "sq278": lambda: (square_mesh(278), 0), "sq280": lambda: (square_mesh(140), 1),
+    "channel_l3": lambda: (channel_cylinder_mesh(seed=2, h=0.02), 3),
 }
 
 
