@@ -269,6 +269,29 @@ static __global__ void __launch_bounds__(kOnchipThreads, 1) k_pcg_onchip(CoarseP
             if (lane == 0) wsum32[wid][k] = s;
         }
         __syncthreads();
+        const uint32_t dst = red32_remote + (uint32_t)(4 * ((par * 16 + rank) * kOnchipSlot));
+        const uint32_t mb = mbar_remote[lane < ncl ? lane : 0][par];
+        if constexpr (MR > 0) {
+            // warps 1 and 2, beside warp 0's scalars: subdomain g of this CTA = warps g wpg ..
+            // g wpg + wpg - 1; its sums (of A z, of r) go out as eight values (unused ones zero),
+            // four to a 16-byte store
+            if (wid == 1 || wid == 2) {
+                const bool sender = !aborted_now() && lane < ncl;
+                float g = lane < nw ? wsum32[lane][2 + wid] : 0.0f;
+                for (int o = 1; o < pl.wpg; o <<= 1) g += __shfl_down_sync(0xffffffffu, g, o);
+                float gv[kOnchipMaxSubPerCta];
+#pragma unroll
+                for (int k = 0; k < kOnchipMaxSubPerCta; ++k) {
+                    const float y = __shfl_sync(0xffffffffu, g, (k < spc ? k : 0) * pl.wpg);
+                    gv[k] = k < spc ? y : 0.0f;
+                }
+                const uint32_t to = dst + 4 * (wid == 1 ? kOnchipSubW : kOnchipSubR);
+                if (sender) {
+                    oc_st_async4(to, gv[0], gv[1], gv[2], gv[3], mb);
+                    oc_st_async4(to + 16, gv[4], gv[5], gv[6], gv[7], mb);
+                }
+            }
+        }
         if (wid == 0) {
             const bool live = !aborted_now();
             // 16 partials: xor rounds 8 .. 1 leave the total in lanes 0-15
@@ -281,33 +304,7 @@ static __global__ void __launch_bounds__(kOnchipThreads, 1) k_pcg_onchip(CoarseP
                 for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                 cs[k] = x;
             }
-            const bool sender = live && lane < ncl;
-            const uint32_t dst = red32_remote + (uint32_t)(4 * ((par * 16 + rank) * kOnchipSlot));
-            const uint32_t mb = mbar_remote[lane < ncl ? lane : 0][par];
-            if (sender) oc_st_async4(dst, cs[0], cs[1], cs[2], 0.0f, mb);
-            if constexpr (MR > 0) {
-                // subdomain g of this CTA = warps g wpg .. g wpg + wpg - 1; its sums go out as
-                // eight values per vector (unused ones zero), four to a 16-byte store
-                float gt = lane < nw ? wsum32[lane][3] : 0.0f, gu = lane < nw ? wsum32[lane][4] : 0.0f;
-                for (int o = 1; o < pl.wpg; o <<= 1) {
-                    gt += __shfl_down_sync(0xffffffffu, gt, o);
-                    gu += __shfl_down_sync(0xffffffffu, gu, o);
-                }
-                float tv[kOnchipMaxSubPerCta], uv[kOnchipMaxSubPerCta];
-#pragma unroll
-                for (int g = 0; g < kOnchipMaxSubPerCta; ++g) {
-                    const int from = (g < spc ? g : 0) * pl.wpg;
-                    const float y1 = __shfl_sync(0xffffffffu, gt, from), y2 = __shfl_sync(0xffffffffu, gu, from);
-                    tv[g] = g < spc ? y1 : 0.0f;
-                    uv[g] = g < spc ? y2 : 0.0f;
-                }
-                if (sender) {
-                    oc_st_async4(dst + 4 * kOnchipSubW, tv[0], tv[1], tv[2], tv[3], mb);
-                    oc_st_async4(dst + 4 * kOnchipSubW + 16, tv[4], tv[5], tv[6], tv[7], mb);
-                    oc_st_async4(dst + 4 * kOnchipSubR, uv[0], uv[1], uv[2], uv[3], mb);
-                    oc_st_async4(dst + 4 * kOnchipSubR + 16, uv[4], uv[5], uv[6], uv[7], mb);
-                }
-            }
+            if (live && lane < ncl) oc_st_async4(dst, cs[0], cs[1], cs[2], 0.0f, mb);
             // (the wait test hook expects 4 bytes more than anyone sends)
             if (lane == 0)
                 oc_mbar_arrive_expect(&mbar[par], (uint32_t)(ncl * (MR > 0 ? 4 * kOnchipSlot : 16) + 4 * halo_self +
@@ -365,16 +362,25 @@ static __global__ void __launch_bounds__(kOnchipThreads, 1) k_pcg_onchip(CoarseP
                 }
             }
             zpar ^= 1;
-            for (int idx = wid; idx < need_n; idx += nw) {
+            // (channel, 32,489 rows: with this and the subdomain sums on warps of their own 4.5
+            // instead of 4.7 us an iteration; two slices of the SpMV in flight gave another 1 %
+            // there and lost 0.6 % on 129^2 rows)
+            // two rows of E^+ a warp at a time: a half-warp's lane takes every sixteenth column,
+            // its s from the lane that holds it
+            const int half = lane >> 4, hl = lane & 15;
+            for (int i0 = 2 * wid; i0 < need_n; i0 += 2 * nw) {
+                const int idx = i0 + half < need_n ? i0 + half : i0;
                 const float* er = einv + idx * m;
                 float acc = 0.0f;
 #pragma unroll
-                for (int c = 0; c < cpl; ++c) {
-                    const int j = lane + 32 * c;
-                    if (j < m) acc = fmaf(er[j], sv[c], acc);
+                for (int c = 0; c < 2 * cpl; ++c) {
+                    const int j = hl + 16 * c;   // column 32 (c / 2) + 16 (c % 2) + hl
+                    const float sj = __shfl_sync(0xffffffffu, sv[c >> 1], hl + 16 * (c & 1));
+                    if (j < m) acc = fmaf(er[j], sj, acc);
                 }
-                acc = warp_sum(acc);
-                if (lane == 0) mu[needl[idx]] = acc;
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (hl == 0 && i0 + half < need_n) mu[needl[idx]] = acc;
             }
             __syncthreads();
             const float mw = mu[my_sub];
