@@ -169,7 +169,21 @@ static int layout(Solver& s, void* base, size_t* bytes) {
         const size_t ctas = std::min<size_t>(kRRMaxSub, (size_t)C.nslices / 8 + 16);
         s.rr_perm = cv.take<int32_t>(32 * ((size_t)C.nslices + 16 * ctas));
         s.rr_einv = cv.take<double>(ctas * ctas);
-        if (gp_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
+        if (s.lc > 0 && ml_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
+            size_t below = 0;
+            for (int l = 0; l < s.lc; ++l) below += (size_t)m->lev[l].nv;
+            const size_t sub = std::min(kMlMaxSub, m->lev[0].nv);
+            s.ml_perm = cv.take<int32_t>(m->lev[0].nv);
+            s.ml_first = cv.take<int32_t>(sub + 1);
+            s.ml_dinv = cv.take<double>(below);
+            s.ml_rs = cv.take<double>(below);
+            s.ml_ws = cv.take<double>(below);
+            s.ml_ss = cv.take<double>(below);
+            s.ml_z = cv.take<double>(below);
+            s.ml_einv = cv.take<double>(sub * sub);
+            s.ml_zs = cv.take<double>(sub);
+            s.ml_row = cv.take<double>(2 * sub);
+        } else if (gp_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
             const size_t slots = gp_slots(nc), ent = gp_entries(nnzc);
             s.gp_perm = cv.take<int32_t>(slots);
             s.gp_slot = cv.take<int32_t>(nc);

@@ -1,5 +1,6 @@
 // Memory-resident FP64 coarse solve over compact subdomains (Eq. 23), for systems that the
-// register-resident solve (coarse_rr.cuh) cannot hold: the same iteration, Chronopoulos and
+// register-resident solve (coarse_rr.cuh) cannot hold and whose level is the base mesh (coarse_ml.cuh
+// has the others): the same iteration, Chronopoulos and
 // Gear's PCG with M^{-1} = D^{-1} + Z E^+ Z^T, with its vectors in global memory.
 //
 // The host plan (gp_plan in rr_plan.cuh) sorts the rows into compact subdomains of whole

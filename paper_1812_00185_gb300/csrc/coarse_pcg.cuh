@@ -217,26 +217,31 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     return v;
 }
 
+// n / d by Newton's iteration for 1 / d from the 20-bit approximation (two steps: 80 bits, so
+// the quotient is within rounding of the exact one); not finite where d is 0 or not finite
+__device__ __forceinline__ double newton_quotient(double n, double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    r = fma(r, fma(-d, r, 1.0), r);
+    const double e = fma(-d, r, 1.0), q = n * r;
+    return fma(q, e, q);
+}
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 struct GridShared {
     double part[kSumMax][kGridThreads];
     double tot[kSumMax];
     SumShared res;
 };
 
-struct GridSync {
+struct GridBarrier {
     unsigned* count;
     int* err;
-    double* partials;
-    GridShared& sm;
     unsigned gen = 0;
-    int slot = 0;
     unsigned extra = 0;            // arrivals awaited beyond the grid's (1 under the wait test hook)
     unsigned limit = kSpinLimit;
-    __device__ GridSync(unsigned* c, int* e, double* p, GridShared& s, int wait_test = 0)
-        : count(c), err(e), partials(p), sm(s), extra(wait_test ? 1u : 0u),
-          limit(wait_test ? kSpinLimitTest : kSpinLimit) {}
-    __device__ int rank() const { return (int)blockIdx.x; }
-    __device__ int ranks() const { return (int)gridDim.x; }
+    __device__ GridBarrier(unsigned* c, int* e, int wait_test)
+        : count(c), err(e), extra(wait_test ? 1u : 0u), limit(wait_test ? kSpinLimitTest : kSpinLimit) {}
     __device__ bool sync() {
         __shared__ int ok;
         __syncthreads();
@@ -266,6 +271,16 @@ struct GridSync {
         __syncthreads();
         return ok != 0;
     }
+};
+
+struct GridSync : GridBarrier {
+    double* partials;
+    GridShared& sm;
+    int slot = 0;
+    __device__ GridSync(unsigned* c, int* e, double* p, GridShared& s, int wait_test = 0)
+        : GridBarrier(c, e, wait_test), partials(p), sm(s) {}
+    __device__ int rank() const { return (int)blockIdx.x; }
+    __device__ int ranks() const { return (int)gridDim.x; }
     // per-CTA partials [set][value][CTA]; after the grid barrier warp r of every CTA adds the
     // partials of value r in the same order (lane l takes l, l + 32, ...)
     template <int NR, int NO, class F>

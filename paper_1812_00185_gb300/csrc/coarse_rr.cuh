@@ -15,7 +15,8 @@
 // the stagnation window: 10,272 iterations to 1e-10 on the channel's 32,489-row system where
 // this form takes 1,243, and 2,878 against 580 on 129^2 vertices.)
 //
-// With a plan (rr_plan.cuh; the solver's default) the rows go to the CTAs as compact subdomains
+// With a plan (rr_plan.cuh; the solver's default where the coarse level is the base mesh, see
+// coarse_ml.cuh for the others) the rows go to the CTAs as compact subdomains
 // and the preconditioner is Jacobi plus an additive coarse correction, as in the on-chip solve:
 // M^{-1} = D^{-1} + Z E^+ Z^T with Z the CTAs' indicator vectors and E = Z^T K Z, all in FP64.
 // A CTA's sum of w joins the exchange of the other sums; from them s = Z^T r follows by the
@@ -154,17 +155,6 @@ __device__ __forceinline__ bool mbar_try(uint64_t* mb, uint32_t parity) {
 
 constexpr long long kRRWaitCycles = 4000000000LL;    // ~2 s: a wait this long means a lost signal
 constexpr long long kRRWaitCyclesTest = 20000000LL;  // ~10 ms, under the wait test hook
-
-// n / d by Newton's iteration for 1 / d from the 20-bit approximation (two steps: 80 bits, so
-// the quotient is within rounding of the exact one); not finite where d is 0 or not finite
-__device__ __forceinline__ double newton_quotient(double n, double d) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-    r = fma(r, fma(-d, r, 1.0), r);
-    const double e = fma(-d, r, 1.0), q = n * r;
-    return fma(q, e, q);
-}
-__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 constexpr int kRREinvMax = kRRCluster * kRRMaxSub;   // and kRRSingle^2 is less
 static_assert(kRRSingle * kRRSingle <= kRREinvMax, "rows of E^+ of one cluster");

@@ -73,14 +73,13 @@ std::vector<double> galerkin(int n, int m, const std::vector<int32_t>& rowptr, c
     return E;
 }
 
-// pseudo-inverse of the Galerkin matrix E (neumann: constants are its null space); false when a
-// pivot is not safely positive
-bool inverse(int m, std::vector<double> E, bool neumann, std::vector<double>& inv) {
+// Constants made regular: E + sigma v v^T with v = 1 / sqrt(m), whose inverse is E^+ + v v^T / sigma
+// (neumann: constants are E's null space).  A subdomain without rows of the space only meets
+// zeros.  Returns sigma, 0 when E is no matrix to invert.
+double regular(int m, std::vector<double>& E, bool neumann) {
     double trace = 0.0;
     for (int j = 0; j < m; ++j) trace += E[(size_t)j * m + j];
-    if (!(trace > 0.0) || !std::isfinite(trace)) return false;
-    // constants made regular: E + sigma v v^T with v = 1 / sqrt(m), whose inverse is
-    // E^+ + v v^T / sigma.  A subdomain without rows of the space only meets zeros.
+    if (!(trace > 0.0) || !std::isfinite(trace)) return 0.0;
     const double sigma = trace / m, shift = neumann ? sigma / m : 0.0;
     for (int j = 0; j < m; ++j) {
         for (int k = 0; k < j; ++k) {
@@ -90,6 +89,14 @@ bool inverse(int m, std::vector<double> E, bool neumann, std::vector<double>& in
         double& d = E[(size_t)j * m + j];
         d = d == 0.0 && !neumann ? sigma : d + shift;
     }
+    return sigma;
+}
+
+// pseudo-inverse of the Galerkin matrix E (neumann: constants are its null space); false when a
+// pivot is not safely positive
+bool inverse(int m, std::vector<double> E, bool neumann, std::vector<double>& inv) {
+    const double sigma = regular(m, E, neumann);
+    if (!(sigma > 0.0)) return false;
     // Cholesky, then the inverse column by column
     std::vector<double> L(E);
     for (int j = 0; j < m; ++j) {
@@ -233,6 +240,46 @@ bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
     P.first.push_back(P.nslices);
     P.nsub = m;
     P.einv.swap(inv);
+    return true;
+}
+
+bool ml_plan(int n, const std::vector<double>& xy, const std::vector<int32_t>& tri, const std::vector<uint8_t>& in_space,
+             int nsub, bool neumann, MlHostPlan& P) {
+    P = MlHostPlan{};
+    const int m = std::min(std::min(nsub, kMlMaxSub), n);
+    if (m < 2) return false;
+    std::vector<Point> pts = points(n, xy);
+    std::vector<int32_t> first(m + 1, n), sub(n), perm(n);
+    bisect(pts.data(), 0, n, 0, m, (n + m - 1) / m + 1, first.data());
+    for (int c = 0; c < m; ++c)
+        for (int k = first[c]; k < first[c + 1]; ++k) {
+            const int i = pts[k].id;
+            sub[i] = in_space[i] ? c : -1;
+            perm[k] = in_space[i] ? i : -2 - i;
+        }
+    // E from the triangles' element matrices: |T| g_a g_b with g the gradients of the hats
+    std::vector<double> E((size_t)m * m, 0.0);
+    for (size_t t = 0; 3 * t < tri.size(); ++t) {
+        const int32_t* v = &tri[3 * t];
+        double ex[3], ey[3];   // edge opposite to each corner
+        for (int a = 0; a < 3; ++a) {
+            const size_t b = v[(a + 1) % 3], c = v[(a + 2) % 3];
+            ex[a] = xy[2 * c] - xy[2 * b];
+            ey[a] = xy[2 * c + 1] - xy[2 * b + 1];
+        }
+        const double area4 = 2.0 * std::fabs(ex[0] * ey[1] - ey[0] * ex[1]);
+        for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b)
+                if (sub[v[a]] >= 0 && sub[v[b]] >= 0)
+                    E[(size_t)sub[v[a]] * m + sub[v[b]]] += (ex[a] * ex[b] + ey[a] * ey[b]) / area4;
+    }
+    const double sigma = regular(m, E, neumann);
+    if (!(sigma > 0.0)) return false;
+    P.nsub = m;
+    P.shift = neumann ? 1.0 / (sigma * m) : 0.0;
+    P.perm.swap(perm);
+    P.first.swap(first);
+    P.e.swap(E);
     return true;
 }
 

@@ -1,7 +1,10 @@
 // Host plans of the FP64 coarse solves over compact subdomains: the register-resident one
-// (coarse_rr.cuh: which row every thread holds) and the memory-resident one (coarse_gp.cuh: the
-// order of the rows), with the coarse space of their preconditioner.
+// (coarse_rr.cuh: which row every thread holds), the memory-resident one (coarse_gp.cuh: the
+// order of the rows) and, where the coarse level has levels below it, the multilevel one
+// (coarse_ml.cuh), with the coarse space of their preconditioner.
 #pragma once
+
+#include <cuda_runtime.h>
 
 #include <cstdint>
 #include <vector>
@@ -48,5 +51,51 @@ struct GpHostPlan {
 bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
              const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
              const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P);
+
+// Plan of the multilevel solve (coarse_ml.cuh): the base mesh's vertices in nsub compact
+// subdomains, and their Galerkin matrix (made regular), which the device inverts.
+constexpr int kMlMaxSub = 608;
+// Systems that one cluster of the register-resident solve does not hold (its 8 slices per CTA);
+// 4,225 rows: 0.73-0.94 ms with one to three levels below, 1.52-1.58 ms register-resident.
+inline bool ml_wanted(int nslices) { return nslices > 128; }
+struct MlHostPlan {
+    int nsub = 0;
+    std::vector<int32_t> perm;      // vertices by subdomain: i, or -2 - i (outside the space)
+    std::vector<int32_t> first;     // nsub + 1
+    std::vector<double> e;          // nsub x nsub
+    double shift = 0.0;             // E^+ = e^{-1} - shift
+};
+
+// False (P.nsub = 0) when there is nothing to invert.
+bool ml_plan(int n, const std::vector<double>& xy, const std::vector<int32_t>& tri, const std::vector<uint8_t>& in_space,
+             int nsub, bool neumann, MlHostPlan& P);
+
+// device views of the multilevel solve
+constexpr int kMlMaxLevels = 4;   // levels below the coarse one
+
+struct MlLevel {
+    int n = 0;                          // its vertices
+    const int32_t* rowptr = nullptr;    // the pattern of the level ABOVE: its rows 0 .. n - 1 restrict
+    const int32_t* ptr = nullptr;
+    const int32_t* col = nullptr;
+    const int2* parents = nullptr;      // of the vertices that the level above adds
+    const double* dinv = nullptr;       // 1 / diagonal, 0 where phi = 0
+    double* rs = nullptr;               // restricted residual
+    double* ws = nullptr;               // restricted w = A u
+    double* ss = nullptr;               // restricted s
+    double* z = nullptr;                // preconditioned, all levels up to this one (base; uppermost if stored)
+};
+
+struct MlPlan {
+    int levels = 0, nsub = 0;           // 0: no plan
+    MlLevel lev[kMlMaxLevels];
+    const int32_t* perm = nullptr;      // base vertices by subdomain (those with phi = 0: -2 - i)
+    const int32_t* first = nullptr;     // nsub + 1
+    const double* einv = nullptr;       // nsub x nsub
+    double* zs = nullptr;               // the subdomains' sums
+    bool stored = false;                // the uppermost of the levels stores its z
+    int group = 256;           // threads per subdomain: a CTA or a warp
+    const uint8_t* tag = nullptr;       // of the coarse level
+};
 
 }  // namespace cgp

@@ -5,6 +5,7 @@
 #include "krylov.cuh"
 #include "mlp.cuh"
 #include "onchip_plan.cuh"
+#include "rr_plan.cuh"
 
 namespace cgp {
 
@@ -82,6 +83,11 @@ struct Solver {
     int gp_nsub = 0, gp_ctas = 0, gp_nslices = 0;
     int32_t *gp_perm = nullptr, *gp_slot = nullptr, *gp_ptr = nullptr, *gp_first = nullptr, *gp_col = nullptr;
     double *gp_val = nullptr, *gp_dinv = nullptr, *gp_einv = nullptr, *gp_vec = nullptr;
+    // the multilevel solve's (coarse_ml.cuh; ml.nsub = 0: no plan): view, CTAs, workspace arrays
+    MlPlan ml{};
+    int ml_ctas = 0, ml_threads = 0;
+    int32_t *ml_perm = nullptr, *ml_first = nullptr;
+    double *ml_dinv = nullptr, *ml_rs = nullptr, *ml_ws = nullptr, *ml_ss = nullptr, *ml_z = nullptr, *ml_einv = nullptr, *ml_zs = nullptr, *ml_row = nullptr;
     bool coarse_fp64 = true;
     cudaStream_t branch = nullptr;                 // second stream of a step (work beside the coarse solve)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;      // the coarse solve's inner iterations run in FP64

@@ -7,6 +7,7 @@
 
 #include "coarse_pcg.cuh"
 #include "coarse_gp.cuh"
+#include "coarse_ml.cuh"
 #include "coarse_rr.cuh"
 #include "coarse_onchip.cuh"
 #include "flows.cuh"
@@ -880,6 +881,81 @@ static int subdomain_plan(Solver& s, const RRShape* sh, int sms, cudaStream_t st
     return CGP_OK;
 }
 
+// Plan of the multilevel solve (coarse_ml.cuh); s.ml.nsub stays 0 where the base mesh's coarse
+// matrix cannot be inverted safely.
+static int multilevel_plan(Solver& s, int sms, cudaStream_t st) {
+    const Level& C = s.mesh->lev[s.lc];
+    const Level& B = s.mesh->lev[0];
+    // a CTA per SM, its 8 to 32 warps with a slice of the coarse level each where that goes
+    const int per_cta = (C.nslices + sms - 1) / sms;
+    const int warps = per_cta <= 8 ? 8 : per_cta <= 16 ? 16 : kMlThreads / 32;
+    int per_sm = 0;
+    CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ml_kernel(32 * warps), 32 * warps,
+                                                           ml_shared_bytes(kMlMaxSub)));
+    if (per_sm < 1) return CGP_OK;
+    std::vector<double> xy(2 * (size_t)B.nv);
+    std::vector<int32_t> tri(3 * (size_t)B.nt);
+    std::vector<uint8_t> in_space(B.nv);
+    CGP_CUDA(cudaMemcpy(xy.data(), B.xy, sizeof(double) * 2 * B.nv, cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(tri.data(), B.tri, sizeof(int32_t) * 3 * B.nt, cudaMemcpyDeviceToHost));
+    CGP_CUDA(cudaMemcpy(in_space.data(), B.tag, B.nv, cudaMemcpyDeviceToHost));
+    for (auto& t : in_space) t = (t & CGP_PHI_ZERO) ? 0 : 1;
+    const int group = warps == kMlThreads / 32 && B.nv > 64 * kMlMaxSub ? 256 : 32;
+    MlHostPlan P;
+    if (!ml_plan(B.nv, xy, tri, in_space, kMlPerCta * sms, s.pure_neumann, P)) return CGP_OK;
+    auto up = [st](auto* dst, const auto& v) {
+        return cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, st);
+    };
+    CGP_CUDA(up(s.ml_perm, P.perm));
+    CGP_CUDA(up(s.ml_first, P.first));
+    CGP_CUDA(up(s.ml_einv, P.e));
+    // its inverse; the place of the subdomains' sums holds the verdict
+    CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), st));
+    CGP_CUDA(cudaMemsetAsync(s.ml_zs, 0, sizeof(double), st));
+    int* const verdict = reinterpret_cast<int*>(s.ml_zs);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.gridDim = dim3(sms, 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.dynamicSmemBytes = sizeof(double) * (size_t)P.nsub * ((P.nsub + sms - 1) / sms);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CGP_CUDA(cudaLaunchKernelEx(&cfg, k_ml_inverse, P.nsub, s.ml_einv, s.ml_row, s.bar_count, s.bar_err, verdict));
+    k_ml_symmetric<<<P.nsub, 128, 0, st>>>(P.nsub, s.ml_einv, P.shift);
+    CGP_LAUNCH_CHECK();
+    int bad = 0;
+    CGP_CUDA(cudaMemcpyAsync(&bad, verdict, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CGP_CUDA(cudaStreamSynchronize(st));
+    if (bad) return CGP_OK;
+    s.ml = MlPlan{};
+    size_t at = 0;
+    for (int l = 0; l < s.lc; ++l) {
+        const Level &L = s.mesh->lev[l], &up1 = s.mesh->lev[l + 1];
+        k_ml_diag<<<blocks_for(L.nv), kBlock, 0, st>>>(L.nv, L.xy, L.tri, L.vt_ptr, L.vt_list, L.tag, s.ml_dinv + at);
+        s.ml.lev[l] = MlLevel{L.nv, up1.rowptr, up1.sell_ptr, up1.sell_col, reinterpret_cast<const int2*>(up1.parents),
+                              s.ml_dinv + at, s.ml_rs + at, s.ml_ws + at, s.ml_ss + at, s.ml_z + at};
+        at += (size_t)L.nv;
+    }
+    CGP_LAUNCH_CHECK();
+    s.ml.levels = s.lc;
+    s.ml.perm = s.ml_perm;
+    s.ml.first = s.ml_first;
+    s.ml.einv = s.ml_einv;
+    s.ml.zs = s.ml_zs;
+    // large levels form the uppermost z once (a grid barrier more, a third of the gathers less):
+    // 1,050,625 rows 99 instead of 134 us an iteration, 263,169 39 instead of 47; 130,321 the same
+    s.ml.stored = per_cta > 32;
+    s.ml.group = group;
+    s.ml.tag = C.tag;
+    s.ml.nsub = P.nsub;
+    s.ml_ctas = sms;
+    s.ml_threads = 32 * warps;
+    return CGP_OK;
+}
+
 int choose_coarse_solver(Solver& s, cudaStream_t st) {
     const cgp_params& p = s.prm;
     int mode = p.coarse_mode;
@@ -1012,14 +1088,18 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
             // its subdomain plan, where the preconditioner is left to the library.  Not on one
             // cluster: with 16 subdomains the cavity's 33^2 rows took 110 iterations instead of
             // 152, but each 40 % longer (4 steps 6.25 instead of 5.60 ms)
-            s.rr_nsub = s.gp_nsub = 0;
+            s.rr_nsub = s.gp_nsub = s.ml.nsub = 0;
             const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm, plan_gp = !sh.ctas && s.gp_perm;
             const bool fp64 = p.precision == CGP_FP64 || p.coarse_mode == CGP_COARSE_AUTO;   // (as below)
-            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_gp)) {
+            const bool plan_ml = sh.ctas != kRRSingle && s.ml_perm;
+            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_gp || plan_ml)) {
                 try {
-                    CGP_TRY(subdomain_plan(s, plan_rr ? &sh : nullptr, sms, st));
+                    if (plan_ml) CGP_TRY(multilevel_plan(s, sms, st));
+                    if (s.ml.nsub) s.rr_ctas = 0;
+                    else if (plan_rr || plan_gp) CGP_TRY(subdomain_plan(s, plan_rr ? &sh : nullptr, sms, st));
                 } catch (const std::bad_alloc&) {   // no host memory for the plan: Jacobi alone
-                    s.rr_nsub = s.gp_nsub = 0;
+                    s.rr_nsub = s.gp_nsub = s.ml.nsub = 0;
+                    s.rr_ctas = sh.ctas;
                 }
             }
         }
@@ -1164,8 +1244,8 @@ static int coarse_solve(Ctx& c) {
         }
         CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));   // counter + error word
         cudaLaunchConfig_t cfg = {};
-        const bool planned = s.gp_nsub && s.coarse_fp64;
-        cfg.gridDim = dim3(planned ? s.gp_ctas : s.coarse_grid, 1, 1);
+        const bool planned = s.gp_nsub && s.coarse_fp64, multilevel = s.ml.nsub && s.coarse_fp64;
+        cfg.gridDim = dim3(multilevel ? s.ml_ctas : planned ? s.gp_ctas : s.coarse_grid, 1, 1);
         cfg.blockDim = dim3(kGridThreads, 1, 1);
         cfg.stream = c.st;
         cudaLaunchAttribute attr[1];
@@ -1173,6 +1253,12 @@ static int coarse_solve(Ctx& c) {
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
+        if (multilevel) {
+            cfg.blockDim = dim3(s.ml_threads, 1, 1);
+            cfg.dynamicSmemBytes = ml_shared_bytes(s.ml.nsub);
+            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, ml_kernel(s.ml_threads), a, s.ml)));
+            return CGP_OK;
+        }
         if (planned) {
             const GpPlan pl{32 * s.gp_nslices, s.gp_nslices, s.gp_nsub, s.gp_ctas, s.gp_perm, s.gp_ptr, s.gp_col,
                             s.gp_val, s.gp_dinv, s.gp_first, s.gp_einv, s.gp_vec};
@@ -1890,7 +1976,7 @@ extern "C" int cgp_coarse_subdomains(const cgp_solver* h, int32_t* nsub) {
         set_error("null solver");
         return CGP_EINVAL;
     }
-    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub + h->s.gp_nsub : 0);
+    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub + h->s.gp_nsub + h->s.ml.nsub : 0);
     return CGP_OK;
 }
 
@@ -1911,7 +1997,7 @@ extern "C" int cgp_coarse_info(const cgp_solver* h, int32_t* kind, int32_t* ctas
             n = s.rr_ctas;
         } else {
             k = CGP_COARSE_PERSISTENT_MEM;
-            n = s.gp_nsub && s.coarse_fp64 ? s.gp_ctas : s.coarse_grid;
+            n = !s.coarse_fp64 ? s.coarse_grid : s.ml.nsub ? s.ml_ctas : s.gp_nsub ? s.gp_ctas : s.coarse_grid;
         }
     }
     if (kind) *kind = k;
