@@ -130,11 +130,13 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * subdomains (phi = 0 vertices in none) and E^+ the pseudo-inverse of E = Z^T K_c Z, built
  * once at cgp_assemble; asked for by name, only the ONCHIP coarse solver has it (cgp_assemble
  * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs;
- * in FP64 PERSISTENT solves of systems beyond one cluster (about 4,000 rows) an additive
+ * in FP64 PERSISTENT solves the inverse of the matrix for systems of up to 1,600 rows (iterations
+ * are then sweeps of refinement; not for CGP_MIXED, with the learned guess or with max_it_poisson
+ * below 64), and beyond that an additive
  * multilevel preconditioner over the levels below the coarse one (Bramble, Pasciak and Xu) with
- * the subdomain correction on the base mesh, or, where the coarse level is the base mesh, the
- * correction itself (one subdomain per CTA or SM, up to 4 million rows); JACOBI elsewhere and
- * with the learned guess on systems too large for registers.  The solution is the same to the
+ * the subdomain correction on the base mesh, or, where the coarse level is the base mesh and
+ * has more than about 4,000 vertices, the correction itself (one subdomain per CTA or SM, up to 4
+ * million rows); JACOBI elsewhere and with the learned guess on systems too large for registers.  The solution is the same to the
  * solve's tolerance; only the iteration count changes. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 

@@ -165,6 +165,12 @@ static int layout(Solver& s, void* base, size_t* bytes) {
     s.dinvKcf = cv.take<float>(nc);
     s.cw64 = cv.take<double>(5 * nc + 1410);   // 5 vectors, or the register-resident solve's words (coarse_rr.cuh)
     // its plan: a thread per row of at most one slice more per CTA than the rows need, and E^+
+    if (s.prm.precond == CGP_PRECOND_AUTO && s.prm.precision == CGP_FP64 && s.nc <= kDirectMaxRows &&
+        (s.prm.coarse_mode == CGP_COARSE_AUTO || s.prm.coarse_mode == CGP_COARSE_PERSISTENT) &&
+        s.prm.max_it_poisson >= kDirectMinCap && s.prm.guess != CGP_GUESS_LEARNED) {
+        s.direct_inv = cv.take<double>(nc * nc);
+        s.direct_row = cv.take<double>(2 * nc);
+    }
     if (s.prm.precond == CGP_PRECOND_AUTO) {
         const size_t ctas = std::min<size_t>(kRRMaxSub, (size_t)C.nslices / 8 + 16);
         s.rr_perm = cv.take<int32_t>(32 * ((size_t)C.nslices + 16 * ctas));

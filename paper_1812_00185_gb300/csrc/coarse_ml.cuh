@@ -58,14 +58,14 @@ __global__ void k_ml_diag(int n, const double* __restrict__ xy, const int32_t* _
 // In place, the inverse of the symmetric positive definite m x m matrix e by Gauss and Jordan's
 // elimination without pivoting, a cooperative launch of one CTA per SM that holds its rows (every
 // G-th) in shared memory; the owner of a pivot row hands it on through `row` (2 x m), one grid
-// barrier a step.  *bad: a pivot is not safely positive, or a wait ran out.  608 rows: 2 ms, and 45
-// ms on one host core.
-__global__ void __launch_bounds__(256) k_ml_inverse(int m, double* __restrict__ e, double* __restrict__ row,
+// barrier a step.  *bad: a pivot is not safely positive, or a wait ran out.
+constexpr int kInverseThreads = 512, kInverseRows = 32;   // rows of a CTA at most
+__global__ void __launch_bounds__(kInverseThreads) k_ml_inverse(int m, double* __restrict__ e, double* __restrict__ row,
                                                     unsigned* count, int* err, int* bad) {
     extern __shared__ double mine[];
     GridBarrier bar(count, err, 0);
     const int G = (int)gridDim.x, cta = (int)blockIdx.x, own = cta < m ? (m - cta + G - 1) / G : 0;
-    __shared__ double diag;
+    __shared__ double diag, f[kInverseRows];
     for (int q = 0; q < own; ++q)
         for (int j = threadIdx.x; j < m; j += blockDim.x) mine[(size_t)q * m + j] = e[(size_t)(cta + q * G) * m + j];
     __syncthreads();
@@ -89,12 +89,16 @@ __global__ void __launch_bounds__(256) k_ml_inverse(int m, double* __restrict__ 
             if (threadIdx.x == 0) *bad = 1;
             return;
         }
-        for (int q = 0; q < own; ++q) {
-            if (cta + q * G == p) continue;
-            double* r = mine + (size_t)q * m;
-            const double f = r[p];
-            __syncthreads();
-            for (int j = threadIdx.x; j < m; j += blockDim.x) r[j] = fma(-f, __ldcg(pass + j), j == p ? 0.0 : r[j]);
+        // column p of the other rows, then their update, each entry of the pivot row read once
+        if (threadIdx.x < own) f[threadIdx.x] = cta + threadIdx.x * G == p ? 0.0 : mine[(size_t)threadIdx.x * m + p];
+        __syncthreads();
+        for (int j = threadIdx.x; j < m; j += blockDim.x) {
+            const double v = __ldcg(pass + j);
+            for (int q = 0; q < own; ++q) {
+                double& r = mine[(size_t)q * m + j];
+                if (j != p) r = fma(-f[q], v, r);
+                else if (cta + q * G != p) r = -f[q] * v;
+            }
         }
         __syncthreads();
     }

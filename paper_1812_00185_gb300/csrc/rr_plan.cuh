@@ -52,12 +52,18 @@ bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
              const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
              const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P);
 
+// Systems solved with the inverse of their matrix (coarse_direct.cuh).  Making it takes 6 ms at
+// assembly for 1,089 rows and 12 ms for 1,600, and grows with the cube; the solve saves 0.7 ms each
+// time.  A caller's iteration cap below kDirectMinCap is one on PCG iterations.
+constexpr int kDirectMaxRows = 1600, kDirectMinCap = 64;
+
 // Plan of the multilevel solve (coarse_ml.cuh): the base mesh's vertices in nsub compact
 // subdomains, and their Galerkin matrix (made regular), which the device inverts.
 constexpr int kMlMaxSub = 608;
-// Systems that one cluster of the register-resident solve does not hold (its 8 slices per CTA);
-// 4,225 rows: 0.73-0.94 ms with one to three levels below, 1.52-1.58 ms register-resident.
-inline bool ml_wanted(int nslices) { return nslices > 128; }
+// Every system too large for the inverse of its matrix.  Measured against the register-resident
+// solve, to 1e-10: 1,681 rows 0.54 ms (0.75), the channel's 2,181 0.66 (1.50), 4,225 rows with one
+// to three levels below 0.73-0.94 (1.52-1.58).
+inline bool ml_wanted(int nslices) { return 32 * nslices > kDirectMaxRows; }
 struct MlHostPlan {
     int nsub = 0;
     std::vector<int32_t> perm;      // vertices by subdomain: i, or -2 - i (outside the space)

@@ -88,6 +88,9 @@ struct Solver {
     int ml_ctas = 0, ml_threads = 0;
     int32_t *ml_perm = nullptr, *ml_first = nullptr;
     double *ml_dinv = nullptr, *ml_rs = nullptr, *ml_ws = nullptr, *ml_ss = nullptr, *ml_z = nullptr, *ml_einv = nullptr, *ml_zs = nullptr, *ml_row = nullptr;
+    // the small systems' inverse (coarse_direct.cuh; direct_ctas = 0: not used)
+    int direct_ctas = 0;
+    double *direct_inv = nullptr, *direct_row = nullptr;
     bool coarse_fp64 = true;
     cudaStream_t branch = nullptr;                 // second stream of a step (work beside the coarse solve)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;      // the coarse solve's inner iterations run in FP64

@@ -2,10 +2,12 @@
 // orchestration: eager launches with host-polled loop control, or a CUDA graph whose
 // Krylov loops are conditional WHILE nodes driven by the kernels themselves.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <new>
 
 #include "coarse_pcg.cuh"
+#include "coarse_direct.cuh"
 #include "coarse_gp.cuh"
 #include "coarse_ml.cuh"
 #include "coarse_rr.cuh"
@@ -881,6 +883,64 @@ static int subdomain_plan(Solver& s, const RRShape* sh, int sms, cudaStream_t st
     return CGP_OK;
 }
 
+// In place, the symmetric m x m matrix e's inverse less `shift` (row: 2 m doubles); *ok is false
+// where it cannot be inverted safely.  Ends with a synchronisation of the stream.
+static int invert(Solver& s, int m, double* e, double* row, double shift, int sms, cudaStream_t st, bool* ok) {
+    int* const verdict = reinterpret_cast<int*>(s.coarse_partials);
+    CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), st));
+    CGP_CUDA(cudaMemsetAsync(verdict, 0, sizeof(int), st));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    if ((m + sms - 1) / sms > kInverseRows) {
+        *ok = false;
+        return CGP_OK;
+    }
+    cfg.gridDim = dim3(sms, 1, 1);
+    cfg.blockDim = dim3(kInverseThreads, 1, 1);
+    cfg.dynamicSmemBytes = sizeof(double) * (size_t)m * ((m + sms - 1) / sms);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CGP_CUDA(cudaFuncSetAttribute(k_ml_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+    CGP_CUDA(cudaLaunchKernelEx(&cfg, k_ml_inverse, m, e, row, s.bar_count, s.bar_err, verdict));
+    k_ml_symmetric<<<m, 128, 0, st>>>(m, e, shift);
+    CGP_LAUNCH_CHECK();
+    int bad = 0;
+    CGP_CUDA(cudaMemcpyAsync(&bad, verdict, sizeof(int), cudaMemcpyDeviceToHost, st));
+    CGP_CUDA(cudaStreamSynchronize(st));
+    *ok = !bad;
+    return CGP_OK;
+}
+
+// The inverse of a small coarse system's matrix (coarse_direct.cuh); s.direct_ctas stays 0 where
+// there is none.
+static int direct_plan(Solver& s, int sms, cudaStream_t st) {
+    const Level& C = s.mesh->lev[s.lc];
+    const size_t shared = sizeof(double) * (size_t)C.nv * ((C.nv + sms - 1) / sms);
+    int optin = 0, dev = 0;
+    CGP_CUDA(cudaGetDevice(&dev));
+    CGP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    if (shared + 1024 > (size_t)optin) return CGP_OK;
+    std::vector<double> dinv(C.nv);
+    CGP_CUDA(cudaMemcpyAsync(dinv.data(), s.dinvKc, sizeof(double) * C.nv, cudaMemcpyDeviceToHost, st));
+    CGP_CUDA(cudaStreamSynchronize(st));
+    // constants made regular as in rr_plan.cu: K + sigma v v^T, v = 1 / sqrt(n), sigma the mean diagonal
+    double trace = 0.0;
+    for (double d : dinv) trace += 1.0 / d;
+    if (!(trace > 0.0) || !std::isfinite(trace)) return CGP_OK;
+    const double sigma = trace / C.nv;
+    CGP_CUDA(cudaMemsetAsync(s.direct_inv, 0, sizeof(double) * (size_t)C.nv * C.nv, st));
+    k_direct_dense<<<blocks_for(C.nv), kBlock, 0, st>>>(sell_of(C), s.Kc0, C.rowptr, s.pure_neumann ? sigma / C.nv : 0.0,
+                                                        s.direct_inv);
+    CGP_LAUNCH_CHECK();
+    bool ok = false;
+    CGP_TRY(invert(s, C.nv, s.direct_inv, s.direct_row, s.pure_neumann ? 1.0 / (sigma * C.nv) : 0.0, sms, st, &ok));
+    if (ok) s.direct_ctas = sms;
+    return CGP_OK;
+}
+
 // Plan of the multilevel solve (coarse_ml.cuh); s.ml.nsub stays 0 where the base mesh's coarse
 // matrix cannot be inverted safely.
 static int multilevel_plan(Solver& s, int sms, cudaStream_t st) {
@@ -909,27 +969,9 @@ static int multilevel_plan(Solver& s, int sms, cudaStream_t st) {
     CGP_CUDA(up(s.ml_perm, P.perm));
     CGP_CUDA(up(s.ml_first, P.first));
     CGP_CUDA(up(s.ml_einv, P.e));
-    // its inverse; the place of the subdomains' sums holds the verdict
-    CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), st));
-    CGP_CUDA(cudaMemsetAsync(s.ml_zs, 0, sizeof(double), st));
-    int* const verdict = reinterpret_cast<int*>(s.ml_zs);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.gridDim = dim3(sms, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = sizeof(double) * (size_t)P.nsub * ((P.nsub + sms - 1) / sms);
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    CGP_CUDA(cudaLaunchKernelEx(&cfg, k_ml_inverse, P.nsub, s.ml_einv, s.ml_row, s.bar_count, s.bar_err, verdict));
-    k_ml_symmetric<<<P.nsub, 128, 0, st>>>(P.nsub, s.ml_einv, P.shift);
-    CGP_LAUNCH_CHECK();
-    int bad = 0;
-    CGP_CUDA(cudaMemcpyAsync(&bad, verdict, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CGP_CUDA(cudaStreamSynchronize(st));
-    if (bad) return CGP_OK;
+    bool ok = false;
+    CGP_TRY(invert(s, P.nsub, s.ml_einv, s.ml_row, P.shift, sms, st, &ok));
+    if (!ok) return CGP_OK;
     s.ml = MlPlan{};
     size_t at = 0;
     for (int l = 0; l < s.lc; ++l) {
@@ -1091,7 +1133,9 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
             s.rr_nsub = s.gp_nsub = s.ml.nsub = 0;
             const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm, plan_gp = !sh.ctas && s.gp_perm;
             const bool fp64 = p.precision == CGP_FP64 || p.coarse_mode == CGP_COARSE_AUTO;   // (as below)
-            const bool plan_ml = sh.ctas != kRRSingle && s.ml_perm;
+            s.direct_ctas = 0;
+            if (s.direct_inv) CGP_TRY(direct_plan(s, sms, st));
+            const bool plan_ml = !s.direct_ctas && s.ml_perm;
             if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_gp || plan_ml)) {
                 try {
                     if (plan_ml) CGP_TRY(multilevel_plan(s, sms, st));
@@ -1235,6 +1279,20 @@ static int coarse_solve(Ctx& c) {
             cfg.blockDim = dim3(kOnchipThreads, 1, 1);
             cfg.dynamicSmemBytes = s.onchip_bytes;
             PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, onchip_kernel(s.onchip.nsub), a, s.onchip)));
+            return CGP_OK;
+        }
+        if (s.direct_ctas) {
+            CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));
+            cudaLaunchAttribute attr[1];
+            cudaLaunchConfig_t cfg = {};
+            attr[0].id = cudaLaunchAttributeCooperative;
+            attr[0].val.cooperative = 1;
+            cfg.gridDim = dim3(s.direct_ctas, 1, 1);
+            cfg.blockDim = dim3(kDirectThreads, 1, 1);
+            cfg.stream = c.st;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_direct_solve, a, (const double*)s.direct_inv)));
             return CGP_OK;
         }
         if (s.rr_ctas && s.coarse_fp64) {
@@ -1993,6 +2051,8 @@ extern "C" int cgp_coarse_info(const cgp_solver* h, int32_t* kind, int32_t* ctas
         if (s.onchip_bytes) {
             k = CGP_COARSE_ONCHIP;
             n = cl = s.cluster_size;
+        } else if (s.direct_ctas) {
+            n = s.direct_ctas;
         } else if (s.rr_ctas && s.coarse_fp64) {
             n = s.rr_ctas;
         } else {
