@@ -129,24 +129,23 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * M^{-1} = D^{-1} + Z E^+ Z^T with Z the indicator vectors of up to 128 compact vertex
  * subdomains (phi = 0 vertices in none) and E^+ the pseudo-inverse of E = Z^T K_c Z, built
  * once at cgp_assemble; asked for by name, only the ONCHIP coarse solver has it (cgp_assemble
- * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs;
- * in FP64 PERSISTENT solves the inverse of the matrix for systems of up to 1,600 rows (iterations
- * are then sweeps of refinement; not for CGP_MIXED, with the learned guess or with max_it_poisson
- * below 64), and beyond that an additive
- * multilevel preconditioner over the levels below the coarse one (Bramble, Pasciak and Xu) with
- * the subdomain correction on the base mesh, or, where the coarse level is the base mesh and
- * has more than about 4,000 vertices, the correction itself (one subdomain per CTA or SM, up to 4
- * million rows); JACOBI elsewhere and with the learned guess on systems too large for registers.  The solution is the same to the
- * solve's tolerance; only the iteration count changes. */
+ * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs.  In FP64 PERSISTENT
+ * solves AUTO takes, by size: the inverse of the matrix up to 1,600 rows (iterations are then
+ * sweeps of refinement; not for CGP_MIXED, with the learned guess, or with max_it_poisson below
+ * 64); beyond that an additive multilevel preconditioner over the levels below the coarse one
+ * (Bramble, Pasciak and Xu) with the subdomain correction on the base mesh; or, where the coarse
+ * level is the base mesh and has more than about 4,000 vertices, the correction itself (one
+ * subdomain per CTA or SM, up to 4 million rows).  JACOBI elsewhere, and with the learned guess on
+ * systems too large for registers.  The solution is the same to the solve's tolerance; only the
+ * iteration count changes. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 
 /* Coarse Poisson solver kinds.  KERNELS: two kernel launches per PCG iteration (graph
  * WHILE loop).  PERSISTENT: the whole solve in one cooperative launch over the GPU with a
  * bounded software grid barrier; in FP64, when the mesh fits one 32-row slice per warp with
- * at most 16 warps per SM, each thread keeps its row and its PCG vectors
- * in registers (not with the multilevel preconditioner).  PERSISTENT_MEM: the same without
- * register residency.  CLUSTER: the whole
- * solve in one launch of one thread-block cluster, vectors in global memory, reductions
+ * at most 16 warps per SM, each thread keeps its row and its PCG vectors in registers (not with
+ * the multilevel preconditioner).  PERSISTENT_MEM: the same without register residency.  CLUSTER:
+ * the whole solve in one launch of one thread-block cluster, vectors in global memory, reductions
  * through distributed shared memory.  ONCHIP (CGP_MIXED only): the FP32 inner solve on one
  * cluster of 8 or 16 CTAs with the FP32 matrix and the vectors held in distributed shared
  * memory and hardware cluster barriers (cgp_assemble fails with CGP_EINVAL if the coarse

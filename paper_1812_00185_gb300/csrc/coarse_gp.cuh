@@ -1,7 +1,7 @@
 // Memory-resident FP64 coarse solve over compact subdomains (Eq. 23), for systems that the
-// register-resident solve (coarse_rr.cuh) cannot hold and whose level is the base mesh (coarse_ml.cuh
-// has the others): the same iteration, Chronopoulos and
-// Gear's PCG with M^{-1} = D^{-1} + Z E^+ Z^T, with its vectors in global memory.
+// register-resident solve (coarse_rr.cuh) cannot hold and whose level is the base mesh (the others
+// are coarse_ml.cuh's): the same iteration, Chronopoulos and Gear's PCG with M^{-1} = D^{-1} +
+// Z E^+ Z^T, with its vectors in global memory.
 //
 // The host plan (gp_plan in rr_plan.cuh) sorts the rows into compact subdomains of whole
 // 32-row slices, kGridCtasPerSm CTAs each, and the solve runs on a copy of the matrix in that
