@@ -132,11 +132,10 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * fails with CGP_EINVAL otherwise).  AUTO: COARSE where the ONCHIP solver runs.  In FP64 PERSISTENT
  * solves AUTO takes, by size: the inverse of the matrix up to 1,600 rows (iterations are then
  * sweeps of refinement; not for CGP_MIXED, with the learned guess, or with max_it_poisson below
- * 64); beyond that an additive multilevel preconditioner over the levels below the coarse one
- * (Bramble, Pasciak and Xu) with the subdomain correction on the base mesh; or, where the coarse
- * level is the base mesh and has more than about 4,000 vertices, the correction itself (one
- * subdomain per CTA or SM, up to 4 million rows).  JACOBI elsewhere, and with the learned guess on
- * systems too large for registers.  The solution is the same to the solve's tolerance; only the
+ * 64); beyond that an additive multilevel preconditioner over the coarse level and the levels
+ * below it (Bramble, Pasciak and Xu) with the subdomain correction on the base mesh (not with the
+ * learned guess, which has the correction with one subdomain per CTA in the register-resident
+ * solve).  JACOBI elsewhere.  The solution is the same to the solve's tolerance; only the
  * iteration count changes. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 

@@ -175,7 +175,7 @@ static int layout(Solver& s, void* base, size_t* bytes) {
         const size_t ctas = std::min<size_t>(kRRMaxSub, (size_t)C.nslices / 8 + 16);
         s.rr_perm = cv.take<int32_t>(32 * ((size_t)C.nslices + 16 * ctas));
         s.rr_einv = cv.take<double>(ctas * ctas);
-        if (s.lc > 0 && ml_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
+        if (ml_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
             size_t below = 0;
             for (int l = 0; l < s.lc; ++l) below += (size_t)m->lev[l].nv;
             const size_t sub = std::min(kMlMaxSub, m->lev[0].nv);
@@ -185,21 +185,10 @@ static int layout(Solver& s, void* base, size_t* bytes) {
             s.ml_rs = cv.take<double>(below);
             s.ml_ws = cv.take<double>(below);
             s.ml_ss = cv.take<double>(below);
-            s.ml_z = cv.take<double>(below);
+            s.ml_z = cv.take<double>(s.lc > 0 ? below : nc);
             s.ml_einv = cv.take<double>(sub * sub);
             s.ml_zs = cv.take<double>(sub);
             s.ml_row = cv.take<double>(2 * sub);
-        } else if (gp_wanted(C.nslices) && s.prm.guess != CGP_GUESS_LEARNED) {
-            const size_t slots = gp_slots(nc), ent = gp_entries(nnzc);
-            s.gp_perm = cv.take<int32_t>(slots);
-            s.gp_slot = cv.take<int32_t>(nc);
-            s.gp_ptr = cv.take<int32_t>(slots / 32 + 1);
-            s.gp_first = cv.take<int32_t>((size_t)s.max_grid + 1);
-            s.gp_col = cv.take<int32_t>(ent);
-            s.gp_val = cv.take<double>(ent);
-            s.gp_dinv = cv.take<double>(slots);
-            s.gp_einv = cv.take<double>((size_t)kRRMaxSub * kRRMaxSub);
-            s.gp_vec = cv.take<double>(6 * slots);
         }
     }
     if (s.prm.guess == CGP_GUESS_LEARNED) {

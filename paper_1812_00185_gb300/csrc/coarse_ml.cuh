@@ -1,5 +1,5 @@
-// Memory-resident FP64 coarse solve with an additive multilevel preconditioner (Eq. 23), for a
-// coarse level that has mesh levels below it.
+// Memory-resident FP64 coarse solve with an additive multilevel preconditioner (Eq. 23) over the
+// coarse level and the mesh levels below it, if any.
 //
 // Chronopoulos and Gear's PCG as in coarse_pcg.cuh, with the preconditioner of Bramble, Pasciak
 // and Xu (Math. Comp. 55, 1990) over the nested levels 0 .. L (L: the coarse level):
@@ -28,6 +28,10 @@
 //      66,049  2               74  (403)       23  (10.8)          1.71  (4.35)
 //     491,401  2              152  (1,034)     55  (30)            8.3   (31)
 //   1,050,625  3              127  (1,516)    100  (54)           12.8   (81)
+//      16,641  none            96  (242)       14  (8.8)           1.38  (2.12)
+//     263,169  none           347  (669)       33  (23)           11.3   (15.3)
+// (in brackets up to 66,049 rows the register-resident solve, beyond a memory-resident one on rows
+// sorted into 152 subdomains.)  Without a level below, M^{-1} = D^{-1} + Z E^+ Z^T on the level itself.
 #pragma once
 
 #include "coarse_pcg.cuh"
@@ -267,6 +271,7 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
     const size_t n = (size_t)A.n;
     double *x = a.x, *r = a.w64, *u = r + n, *w = u + n, *p = w + n, *s = p + n;
     const int top = pl.levels - 1;   // the level below the coarse one
+    const bool flat = top < 0;       // the coarse level is the base mesh: M^{-1} = D^{-1} + Z E^+ Z^T
     // this group's subdomain of the base mesh; kMlPerCta groups of a CTA have one each (as warps,
     // those after the ones that add up the sums)
     const int gs = pl.group, gt = tid & (gs - 1), gi = gs == 32 ? wid - 4 : tid / gs;
@@ -316,6 +321,10 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
             double t = 0.0;
             base_rows([&](int i) {
                 if (i < 0) return;
+                if (flat) {
+                    t += ldcg(from + i);
+                    return;
+                }
                 const double q = ml_restrict(pl.lev[0], from, i);
                 __stcg(pl.lev[0].ws + i, q);
                 t += q;
@@ -347,7 +356,8 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
                 mu = fma(-alpha, mq, mu);
             }
             base_rows([&](int i) {
-                if (i >= 0) __stcg(pl.lev[0].z + i, fma(__ldg(pl.lev[0].dinv + i), step(pl.lev[0], i), mu));
+                if (i >= 0 && flat) __stcg(pl.lev[0].z + i, mu);
+                else if (i >= 0) __stcg(pl.lev[0].z + i, fma(__ldg(pl.lev[0].dinv + i), step(pl.lev[0], i), mu));
                 else __stcg(pl.lev[0].z - 2 - i, 0.0);
             });
         }
@@ -367,6 +377,7 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
             }
             return sy.sync();
         };
+        if (flat) return rows([&](int i) { return ldcg(pl.lev[0].z + i); });
         if (pl.stored && top > 0) {
             const MlLevel& q = pl.lev[top];
             rows_of(q.n, [&](int i) {

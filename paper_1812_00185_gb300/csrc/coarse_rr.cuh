@@ -15,8 +15,8 @@
 // the stagnation window: 10,272 iterations to 1e-10 on the channel's 32,489-row system where
 // this form takes 1,243, and 2,878 against 580 on 129^2 vertices.)
 //
-// With a plan (rr_plan.cuh; the solver's default where the coarse level is the base mesh, see
-// coarse_ml.cuh for the others) the rows go to the CTAs as compact subdomains
+// With a plan (rr_plan.cuh; the default with the learned guess, whose second start coarse_ml.cuh
+// does not take) the rows go to the CTAs as compact subdomains
 // and the preconditioner is Jacobi plus an additive coarse correction, as in the on-chip solve:
 // M^{-1} = D^{-1} + Z E^+ Z^T with Z the CTAs' indicator vectors and E = Z^T K Z, all in FP64.
 // A CTA's sum of w joins the exchange of the other sums; from them s = Z^T r follows by the

@@ -167,82 +167,6 @@ bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
     return true;
 }
 
-bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
-             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
-             const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P) {
-    P = GpHostPlan{};
-    const int m = std::min(nsub, kRRMaxSub);
-    if (m < 2 || n < 32 * m) return false;
-    std::vector<Point> pts = points(n, xy);
-    std::vector<int32_t> first(m + 1, n), sub(n);
-    bisect(pts.data(), 0, n, 0, m, (n + m - 1) / m + 1, first.data());
-    for (int c = 0; c < m; ++c)
-        for (int k = first[c]; k < first[c + 1]; ++k) sub[pts[k].id] = in_space[pts[k].id] ? c : -1;
-    std::vector<double> inv;
-    if (!inverse(m, galerkin(n, m, rowptr, sell_ptr, sell_col, val, sub), neumann, inv)) return false;
-    // the order within a subdomain: rows longer than most first (their slices are wider), then by
-    // the cells of a grid of about 48 rows each, so that a slice's columns lie close together
-    std::vector<int64_t> hist(64, 0);
-    for (int i = 0; i < n; ++i) ++hist[std::min(63, rowptr[i + 1] - rowptr[i])];
-    const int usual = (int)(std::max_element(hist.begin(), hist.end()) - hist.begin());
-    P.slot_of.assign(n, 0);
-    P.ptr.push_back(0);
-    std::vector<int32_t> slices(m + 1, 0), key, count;
-    for (int c = 0; c < m; ++c) {
-        const int lo = first[c], rows = first[c + 1] - lo;
-        double mn[2] = {INFINITY, INFINITY}, mx[2] = {-INFINITY, -INFINITY};
-        for (int k = lo; k < lo + rows; ++k)
-            for (int d = 0; d < 2; ++d) {
-                mn[d] = std::min(mn[d], pts[k].x[d]);
-                mx[d] = std::max(mx[d], pts[k].x[d]);
-            }
-        const int side = std::max(1, (int)std::sqrt(rows / 48.0));
-        auto cell = [&](int k, int d) {
-            const double w = mx[d] - mn[d];
-            return w > 0.0 ? std::min(side - 1, (int)((pts[k].x[d] - mn[d]) / w * side)) : 0;
-        };
-        key.assign(rows, 0);
-        count.assign(2 * side * side + 1, 0);
-        for (int k = 0; k < rows; ++k) {
-            const int cx = cell(lo + k, 0), cy = cell(lo + k, 1), len = rowptr[pts[lo + k].id + 1] - rowptr[pts[lo + k].id];
-            key[k] = (len > usual ? 0 : side * side) + cy * side + (cy & 1 ? side - 1 - cx : cx);
-            ++count[key[k] + 1];
-        }
-        for (size_t q = 1; q < count.size(); ++q) count[q] += count[q - 1];
-        const int s0 = (int)P.ptr.size() - 1, ns = (rows + 31) / 32;
-        P.perm.resize(32 * (size_t)(s0 + ns), -1);
-        for (int k = 0; k < rows; ++k) {
-            const int slot = 32 * s0 + count[key[k]]++;
-            P.perm[slot] = pts[lo + k].id;
-            P.slot_of[pts[lo + k].id] = slot;
-        }
-        for (int q = 0; q < ns; ++q) {
-            int w = 0;
-            for (int l = 0; l < 32; ++l) {
-                const int i = P.perm[32 * (size_t)(s0 + q) + l];
-                if (i >= 0) w = std::max(w, rowptr[i + 1] - rowptr[i]);
-            }
-            const int64_t end = (int64_t)P.ptr.back() + 32 * w;
-            if (end > INT32_MAX) {
-                P = GpHostPlan{};
-                return false;
-            }
-            P.ptr.push_back((int32_t)end);
-        }
-        slices[c + 1] = s0 + ns;
-    }
-    P.nslices = (int)P.ptr.size() - 1;
-    // CTAs per subdomain: as many as give every warp of theirs a slice
-    P.per = std::max(1, std::min(max_per, P.nslices / (8 * m)));
-    for (int c = 0; c < m; ++c)
-        for (int q = 0; q < P.per; ++q)
-            P.first.push_back(slices[c] + (int32_t)((int64_t)(slices[c + 1] - slices[c]) * q / P.per));
-    P.first.push_back(P.nslices);
-    P.nsub = m;
-    P.einv.swap(inv);
-    return true;
-}
-
 bool ml_plan(int n, const std::vector<double>& xy, const std::vector<int32_t>& tri, const std::vector<uint8_t>& in_space,
              int nsub, bool neumann, MlHostPlan& P) {
     P = MlHostPlan{};

@@ -1,7 +1,6 @@
 // Host plans of the FP64 coarse solves over compact subdomains: the register-resident one
-// (coarse_rr.cuh: which row every thread holds), the memory-resident one (coarse_gp.cuh: the
-// order of the rows) and, where the coarse level has levels below it, the multilevel one
-// (coarse_ml.cuh), with the coarse space of their preconditioner.
+// (coarse_rr.cuh: which row every thread holds) and the multilevel one (coarse_ml.cuh), with the
+// coarse space of their preconditioner.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -12,14 +11,6 @@
 namespace cgp {
 
 constexpr int kRRMaxSub = 160;   // subdomains (one per CTA): five per lane of a warp
-
-// The memory-resident solve has a plan for systems of more slices than any launch of the
-// register-resident one holds by design (16 per SM of about 150), up to a size whose host plan
-// (about 0.1 s per million rows, once per solver) is soon earned back.
-constexpr int kGpMinSlices = 2048, kGpMaxSlices = 1 << 17;
-inline bool gp_wanted(int nslices) { return nslices > kGpMinSlices && nslices <= kGpMaxSlices; }
-inline size_t gp_slots(int64_t n) { return (size_t)n + 32 * (size_t)kRRMaxSub; }
-inline size_t gp_entries(int64_t nnz_sell) { return (size_t)nnz_sell + (size_t)nnz_sell / 4 + 32 * 64 * (size_t)kRRMaxSub; }
 
 struct RRHostPlan {
     int nsub = 0;                  // 0: no plan (the slices in order, Jacobi alone)
@@ -36,22 +27,6 @@ bool rr_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_
              const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
              const std::vector<uint8_t>& in_space, int ctas, int threads, bool neumann, RRHostPlan& P);
 
-// Plan of the memory-resident solve: nsub compact subdomains of whole 32-row slices, `per` CTAs
-// each, and the slices' widths in the new order.
-struct GpHostPlan {
-    int nsub = 0, per = 0, nslices = 0;
-    std::vector<int32_t> perm;      // slot -> row, or -1 (padding)
-    std::vector<int32_t> slot_of;   // row -> slot
-    std::vector<int32_t> ptr;       // nslices + 1: first entry of every slice
-    std::vector<int32_t> first;     // nsub per + 1: first slice of every CTA
-    std::vector<double> einv;
-};
-
-// False (P.nsub = 0) when E is not safely invertible.
-bool gp_plan(int n, const std::vector<int32_t>& rowptr, const std::vector<int32_t>& sell_ptr,
-             const std::vector<int32_t>& sell_col, const std::vector<double>& val, const std::vector<double>& xy,
-             const std::vector<uint8_t>& in_space, int nsub, int max_per, bool neumann, GpHostPlan& P);
-
 // Systems solved with the inverse of their matrix (coarse_direct.cuh).  Making it takes 6 ms at
 // assembly for 1,089 rows and 12 ms for 1,600, and grows with the cube; the solve saves 0.7 ms each
 // time.  A caller's iteration cap below kDirectMinCap is one on PCG iterations.
@@ -61,8 +36,8 @@ constexpr int kDirectMaxRows = 1600, kDirectMinCap = 64;
 // subdomains, and their Galerkin matrix (made regular), which the device inverts.
 constexpr int kMlMaxSub = 608;
 // Every system too large for the inverse of its matrix.  Measured against the register-resident
-// solve, to 1e-10: 1,681 rows 0.54 ms (0.75), the channel's 2,181 0.66 (1.50), 4,225 rows with one
-// to three levels below 0.73-0.94 (1.52-1.58).
+// solve, to 1e-10: 1,681 rows 0.54 ms with a level below, 0.73 without (0.76), the channel's 2,181
+// 0.66 and 0.73 (1.50), 4,225 rows 0.73-0.94 (1.42-1.58), 66,049 rows without a level below 3.2 (3.8).
 inline bool ml_wanted(int nslices) { return 32 * nslices > kDirectMaxRows; }
 struct MlHostPlan {
     int nsub = 0;

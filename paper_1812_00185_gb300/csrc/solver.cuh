@@ -79,10 +79,6 @@ struct Solver {
     int rr_nsub = 0;              // subdomains of its plan (rr_plan.cuh; 0: Jacobi alone)
     int32_t* rr_perm = nullptr;
     double* rr_einv = nullptr;
-    // plan of the memory-resident FP64 solve (rr_plan.cuh; gp_nsub = 0: none) and its arrays
-    int gp_nsub = 0, gp_ctas = 0, gp_nslices = 0;
-    int32_t *gp_perm = nullptr, *gp_slot = nullptr, *gp_ptr = nullptr, *gp_first = nullptr, *gp_col = nullptr;
-    double *gp_val = nullptr, *gp_dinv = nullptr, *gp_einv = nullptr, *gp_vec = nullptr;
     // the multilevel solve's (coarse_ml.cuh; ml.nsub = 0: no plan): view, CTAs, workspace arrays
     MlPlan ml{};
     int ml_ctas = 0, ml_threads = 0;

@@ -8,7 +8,6 @@
 
 #include "coarse_pcg.cuh"
 #include "coarse_direct.cuh"
-#include "coarse_gp.cuh"
 #include "coarse_ml.cuh"
 #include "coarse_rr.cuh"
 #include "coarse_onchip.cuh"
@@ -834,10 +833,9 @@ static cudaLaunchConfig_t cluster_config(int csize, cudaStream_t st, cudaLaunchA
     return cfg;
 }
 
-// Host plan of the FP64 coarse solve over compact subdomains (rr_plan.cuh): of the register-
-// resident launch `sh`, or (null) of the memory-resident solve.  No plan (Jacobi alone) where the
-// coarse matrix cannot be inverted safely.
-static int subdomain_plan(Solver& s, const RRShape* sh, int sms, cudaStream_t st) {
+// Host plan of the register-resident FP64 coarse solve over compact subdomains (rr_plan.cuh).  No
+// plan (Jacobi alone) where the coarse matrix cannot be inverted safely.
+static int subdomain_plan(Solver& s, const RRShape& sh, cudaStream_t st) {
     const Level& C = s.mesh->lev[s.lc];
     std::vector<int32_t> rowptr(C.nv + 1), ptr(C.nslices + 1), col(C.nnz_sell);
     std::vector<double> xy(2 * (size_t)C.nv), val(C.nnz_sell);
@@ -853,33 +851,11 @@ static int subdomain_plan(Solver& s, const RRShape* sh, int sms, cudaStream_t st
     auto up = [](auto* dst, const auto& v) {
         return cudaMemcpy(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
     };
-    if (sh) {
-        RRHostPlan P;
-        if (!rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh->ctas, 32 * sh->warps, s.pure_neumann, P)) return CGP_OK;
-        CGP_CUDA(up(s.rr_perm, P.perm));
-        CGP_CUDA(up(s.rr_einv, P.einv));
-        s.rr_nsub = P.nsub;
-        return CGP_OK;
-    }
-    int per_sm = 0;
-    CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_grid_plan, kGridThreads, 0));
-    GpHostPlan G;
-    if (per_sm < 1 || !gp_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sms, std::min(per_sm, kGridCtasPerSm),
-                               s.pure_neumann, G))
-        return CGP_OK;
-    if (G.perm.size() > gp_slots(C.nv) || (size_t)G.ptr.back() > gp_entries(C.nnz_sell)) return CGP_OK;
-    CGP_CUDA(up(s.gp_perm, G.perm));
-    CGP_CUDA(up(s.gp_slot, G.slot_of));
-    CGP_CUDA(up(s.gp_ptr, G.ptr));
-    CGP_CUDA(up(s.gp_first, G.first));
-    CGP_CUDA(up(s.gp_einv, G.einv));
-    k_gp_matrix<<<blocks_for((int64_t)G.perm.size()), kBlock, 0, st>>>(
-        (int)G.perm.size(), s.gp_perm, s.gp_slot, C.rowptr, C.sell_ptr, C.sell_col, s.Kc0, s.dinvKc, C.tag, s.gp_ptr,
-        s.gp_col, s.gp_val, s.gp_dinv);
-    CGP_LAUNCH_CHECK();
-    s.gp_nsub = G.nsub;
-    s.gp_ctas = G.nsub * G.per;
-    s.gp_nslices = G.nslices;
+    RRHostPlan P;
+    if (!rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh.ctas, 32 * sh.warps, s.pure_neumann, P)) return CGP_OK;
+    CGP_CUDA(up(s.rr_perm, P.perm));
+    CGP_CUDA(up(s.rr_einv, P.einv));
+    s.rr_nsub = P.nsub;
     return CGP_OK;
 }
 
@@ -946,9 +922,10 @@ static int direct_plan(Solver& s, int sms, cudaStream_t st) {
 static int multilevel_plan(Solver& s, int sms, cudaStream_t st) {
     const Level& C = s.mesh->lev[s.lc];
     const Level& B = s.mesh->lev[0];
-    // a CTA per SM, its 8 to 32 warps with a slice of the coarse level each where that goes
+    // a CTA per SM, its 8 to 32 warps with a slice of the coarse level each where that goes (16 up to
+    // 20 slices: 17 slices took 26 us an iteration on 32 warps, 16 slices 18 us on 16)
     const int per_cta = (C.nslices + sms - 1) / sms;
-    const int warps = per_cta <= 8 ? 8 : per_cta <= 16 ? 16 : kMlThreads / 32;
+    const int warps = per_cta <= 8 ? 8 : per_cta <= 20 ? 16 : kMlThreads / 32;
     int per_sm = 0;
     CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ml_kernel(32 * warps), 32 * warps,
                                                            ml_shared_bytes(kMlMaxSub)));
@@ -982,6 +959,10 @@ static int multilevel_plan(Solver& s, int sms, cudaStream_t st) {
         at += (size_t)L.nv;
     }
     CGP_LAUNCH_CHECK();
+    if (s.lc == 0) {
+        s.ml.lev[0].n = C.nv;
+        s.ml.lev[0].z = s.ml_z;
+    }
     s.ml.levels = s.lc;
     s.ml.perm = s.ml_perm;
     s.ml.first = s.ml_first;
@@ -1130,19 +1111,19 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
             // its subdomain plan, where the preconditioner is left to the library.  Not on one
             // cluster: with 16 subdomains the cavity's 33^2 rows took 110 iterations instead of
             // 152, but each 40 % longer (4 steps 6.25 instead of 5.60 ms)
-            s.rr_nsub = s.gp_nsub = s.ml.nsub = 0;
-            const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm, plan_gp = !sh.ctas && s.gp_perm;
+            s.rr_nsub = s.ml.nsub = 0;
+            const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm;
             const bool fp64 = p.precision == CGP_FP64 || p.coarse_mode == CGP_COARSE_AUTO;   // (as below)
             s.direct_ctas = 0;
             if (s.direct_inv) CGP_TRY(direct_plan(s, sms, st));
             const bool plan_ml = !s.direct_ctas && s.ml_perm;
-            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_gp || plan_ml)) {
+            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_ml)) {
                 try {
                     if (plan_ml) CGP_TRY(multilevel_plan(s, sms, st));
                     if (s.ml.nsub) s.rr_ctas = 0;
-                    else if (plan_rr || plan_gp) CGP_TRY(subdomain_plan(s, plan_rr ? &sh : nullptr, sms, st));
+                    else if (plan_rr) CGP_TRY(subdomain_plan(s, sh, st));
                 } catch (const std::bad_alloc&) {   // no host memory for the plan: Jacobi alone
-                    s.rr_nsub = s.gp_nsub = s.ml.nsub = 0;
+                    s.rr_nsub = s.ml.nsub = 0;
                     s.rr_ctas = sh.ctas;
                 }
             }
@@ -1302,8 +1283,8 @@ static int coarse_solve(Ctx& c) {
         }
         CGP_CUDA(cudaMemsetAsync(s.bar_count, 0, 2 * sizeof(unsigned int), c.st));   // counter + error word
         cudaLaunchConfig_t cfg = {};
-        const bool planned = s.gp_nsub && s.coarse_fp64, multilevel = s.ml.nsub && s.coarse_fp64;
-        cfg.gridDim = dim3(multilevel ? s.ml_ctas : planned ? s.gp_ctas : s.coarse_grid, 1, 1);
+        const bool multilevel = s.ml.nsub && s.coarse_fp64;
+        cfg.gridDim = dim3(multilevel ? s.ml_ctas : s.coarse_grid, 1, 1);
         cfg.blockDim = dim3(kGridThreads, 1, 1);
         cfg.stream = c.st;
         cudaLaunchAttribute attr[1];
@@ -1315,12 +1296,6 @@ static int coarse_solve(Ctx& c) {
             cfg.blockDim = dim3(s.ml_threads, 1, 1);
             cfg.dynamicSmemBytes = ml_shared_bytes(s.ml.nsub);
             PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, ml_kernel(s.ml_threads), a, s.ml)));
-            return CGP_OK;
-        }
-        if (planned) {
-            const GpPlan pl{32 * s.gp_nslices, s.gp_nslices, s.gp_nsub, s.gp_ctas, s.gp_perm, s.gp_ptr, s.gp_col,
-                            s.gp_val, s.gp_dinv, s.gp_first, s.gp_einv, s.gp_vec};
-            PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid_plan, a, pl)));
             return CGP_OK;
         }
         PL(c, CGP_PROF_POIS_CLUSTER, CGP_CUDA(cudaLaunchKernelEx(&cfg, k_pcg_grid, a)));
@@ -2034,7 +2009,7 @@ extern "C" int cgp_coarse_subdomains(const cgp_solver* h, int32_t* nsub) {
         set_error("null solver");
         return CGP_EINVAL;
     }
-    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub + h->s.gp_nsub + h->s.ml.nsub : 0);
+    if (nsub) *nsub = h->s.onchip_bytes ? h->s.onchip.nsub : (h->s.coarse_fp64 ? h->s.rr_nsub + h->s.ml.nsub : 0);
     return CGP_OK;
 }
 
@@ -2057,7 +2032,7 @@ extern "C" int cgp_coarse_info(const cgp_solver* h, int32_t* kind, int32_t* ctas
             n = s.rr_ctas;
         } else {
             k = CGP_COARSE_PERSISTENT_MEM;
-            n = !s.coarse_fp64 ? s.coarse_grid : s.ml.nsub ? s.ml_ctas : s.gp_nsub ? s.gp_ctas : s.coarse_grid;
+            n = !s.coarse_fp64 ? s.coarse_grid : s.ml.nsub ? s.ml_ctas : s.coarse_grid;
         }
     }
     if (kind) *kind = k;

@@ -77,3 +77,22 @@ def test_two_part_mesh_falls_back_to_jacobi(lib):
     assert rc == cg.CGP_OK and np.linalg.norm(b - A @ phi) <= 1.01 * TOL * np.linalg.norm(b)
     s.close()
     m.close()
+
+
+# the base mesh itself: M^{-1} = D^{-1} + Z E^+ Z^T, a warp or 8 warps per subdomain
+FLAT = {"sq40": lambda: square_mesh(40), "channel": lambda: channel_cylinder_mesh(seed=3, h=0.012),
+        "sq64": lambda: square_mesh(64), "sq197": lambda: square_mesh(197)}
+
+
+@pytest.mark.parametrize("name", FLAT)
+def test_base_mesh_solve_meets_its_tolerance(lib, name):
+    from paper_1812_00185_gb300 import binding as cg
+    m, s, A, fixed = _system(cg, FLAT[name](), 0)
+    assert s.coarse_info()[0] == cg.CGP_COARSE_PERSISTENT_MEM and s.coarse_subdomains() == 4 * s.coarse_info()[1]
+    b = _rhs(A.shape[0], fixed, 14)
+    first = cg.cgp_poisson_solve(s.handle, b)
+    phi, it, rc = cg.cgp_poisson_solve(s.handle, b)
+    assert rc == cg.CGP_OK and 0 < it < 400 and np.array_equal(phi, first[0])
+    assert np.linalg.norm(b - A @ phi) <= 1.01 * TOL * np.linalg.norm(b)
+    s.close()
+    m.close()
