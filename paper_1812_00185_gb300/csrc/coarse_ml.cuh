@@ -435,7 +435,7 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
             status = CGP_ETIMEOUT;
             break;
         }
-        const double stop2 = 0.25 * a.tol2 * bb;
+        const double stop2 = 0.25 * a.tol2 * bb, stall = stall_level(rr_final, stop2);
         double gamma = 0.0, d = 0.0, rr_best = INFINITY;
         int best_k = 0, leave = 0;
         for (int k = 0;; ++k) {
@@ -465,7 +465,7 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
                         best_k = k;
                     }
                     if (!finite_bits(q[0]) || q[0] == 0.0) return 2;
-                    return k - best_k > stagnation_window(k, rr_best <= 1e4 * stop2) || iters >= a.maxit ? 1 : 0;
+                    return k - best_k > stagnation_window(k, rr_best <= stall) || iters >= a.maxit ? 1 : 0;
                 })) {
                 status = CGP_ETIMEOUT;
                 break;

@@ -45,12 +45,17 @@ constexpr int kGridCtasPerSm = 4;
 constexpr unsigned kSpinLimit = 1u << 24;   // polls of one grid barrier before giving up (~seconds)
 constexpr unsigned kSpinLimitTest = 1u << 14;   // the same under the wait test hook (milliseconds)
 constexpr int kStagnation = 2000;           // FP64 inner iterations without halving the best residual
-// ... unless the best residual is within 100 of the target: there a run of an eighth of the
-// iterations' usual 33 halvings, k / 4, is a stall at the recurrence's attainable accuracy, and a
-// restart from the true residual has little left to do.  (One of three seeded loads on 1025^2
-// rows stalled just above 1e-10 and waited out the 2000: 3,572 iterations instead of 1,920.)
-__device__ __forceinline__ int stagnation_window(int k, bool near_target) {
-    return !near_target ? kStagnation : (k / 4 < 200 ? 200 : (k / 4 < kStagnation ? k / 4 : kStagnation));
+// ... unless this run of the recurrence has itself brought <r, r> down by 1e12 and to within 1e4 of
+// its target (norms: 1e6 and 100).  A run of an eighth of the iterations' usual 33 halvings, k / 4,
+// is then a stall at the recurrence's attainable accuracy, and a restart from the true residual has
+// little left to do.  (One of three seeded loads on 1025^2 rows stalled just above 1e-10 and waited
+// out the 2000: 3,572 iterations instead of 1,920.)  A run that starts near its target is not
+// stalled when it is slow: with the second condition alone, warm starts with a smooth residual were
+// restarted again and again (1025^2 rows, Jacobi, smooth residuals 20 and 50 times the target away:
+// 5,132 and 6,783 iterations instead of 1,417 and 1,428).
+__device__ __forceinline__ double stall_level(double rr_start, double stop2) { return fmin(1e-12 * rr_start, 1e4 * stop2); }
+__device__ __forceinline__ int stagnation_window(int k, bool may_stall) {
+    return !may_stall ? kStagnation : (k / 4 < 200 ? 200 : (k / 4 < kStagnation ? k / 4 : kStagnation));
 }
 constexpr int kStagnation32 = 300;          // the same for the FP32 inner solve of the mixed form
 
@@ -382,18 +387,19 @@ __device__ __forceinline__ T row_spmv(const SellView& A, const double* __restric
 
 // Inner FP64 PCG (Chronopoulos-Gear, w = A u formed every iteration as in coarse_rr.cuh) on
 // A x = b from the residual r and u = D^{-1} r in V (written before the last barrier), with
-// gamma = <r, u>; x itself is V.e.  Two passes over the rows per iteration: w = A u with the
+// gamma = <r, u> and rr_start = <r, r>; x itself is V.e.  Two passes over the rows per iteration: w = A u with the
 // reduction, then the vector updates.  Returns false on a barrier timeout.  iters counts
 // iterations across calls.  outcome: 0 = ended normally (target met, or stagnation),
 // 1 = breakdown before an update (the iterate is intact), 2 = a non-finite value after an
 // update (the iterate is not).
 template <class Sync>
 __device__ bool inner_pcg(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<double>& V, const double* __restrict__ dinv,
-                          int s_begin, int s_end, double gamma, double stop2, int& iters, int& outcome) {
+                          int s_begin, int s_end, double gamma, double rr_start, double stop2, int& iters, int& outcome) {
     outcome = 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const SellView& A = a.A;
     double d = 0.0, rr_best = INFINITY, part[3] = {0.0, 0.0, 0.0};
+    const double stall = stall_level(rr_start, stop2);
     int best_k = 0;
     for (int k = 0;; ++k) {
         // w = A u, <w, u> (u is complete)
@@ -424,7 +430,7 @@ __device__ bool inner_pcg(const CoarsePcgArgs& a, Sync& sy, const InnerVecs<doub
                     best_k = k;
                 }
                 if (!isfinite(q[0]) || q[0] == 0.0) return 2;
-                return k - best_k > stagnation_window(k, rr_best <= 1e4 * stop2) || iters >= a.maxit ? 1 : 0;
+                return k - best_k > stagnation_window(k, rr_best <= stall) || iters >= a.maxit ? 1 : 0;
             }))
             return false;
         if (flag) {
@@ -754,7 +760,7 @@ __device__ void coarse_pcg_body(const CoarsePcgArgs& a, Sync& sy) {
             }
         } else {
             // FP64: the inner recurrence updates x itself; the next outer pass re-checks the true residual
-            ok = inner_pcg(a, sy, V64, a.dinv, s_begin, s_end, tot[2], 0.25 * tol2 * bb, iters, outcome);
+            ok = inner_pcg(a, sy, V64, a.dinv, s_begin, s_end, tot[2], rr0, 0.25 * tol2 * bb, iters, outcome);
         }
         if (!ok) {
             status = CGP_ETIMEOUT;

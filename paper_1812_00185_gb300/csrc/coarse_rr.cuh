@@ -568,7 +568,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         // leave in the shared flag: 1 = target met or restart, 2 = not finite
         const double stop2 = 0.25 * a.tol2 * bb;
         double p_i = 0.0, s_i = 0.0, rg = 0.0, c = 0.0;
-        const long long near_bits = __double_as_longlong(1e4 * stop2);
+        const long long stall_bits = __double_as_longlong(stall_level(rr_final, stop2));
         long long half_best = 0x7fe0000000000000ll;   // bits of half the smallest <r, r> so far
         double gd[2] = {0.0, 0.0};   // gamma and d of the last update
         int best_k = 0, leave = 0;
@@ -603,8 +603,8 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                             half_best = rb - (1ll << 52);
                             best_k = k;
                         }
-                        const bool near_target = half_best + (1ll << 52) <= near_bits;
-                        if (!finite_bits(q[0]) || k - best_k > stagnation_window(k, near_target) || iters >= a.maxit) {
+                        const bool may_stall = half_best + (1ll << 52) <= stall_bits;
+                        if (!finite_bits(q[0]) || k - best_k > stagnation_window(k, may_stall) || iters >= a.maxit) {
                             q[0] = 0.0;
                             q[1] = 1.0;
                         }
