@@ -582,7 +582,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
             });
             const bool ok = sy.reduce(
                 r_i * u_i, w_i * u_i, r_i * r_i, in_space ? w_i : 0.0, kRRAdvance, bad, o, mu, [&](double tg, double td, double trr, double (&q)[4]) {
-                    const double dn = td - tg * tg * c;
+                    const double dn = td - tg * (tg * c);   // (tg^2 alone leaves the range of FP64)
                     q[0] = newton_quotient(tg, dn);
                     q[1] = tg * rg;
                     q[2] = tg;
