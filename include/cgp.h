@@ -384,14 +384,15 @@ void cgp_mlp_destroy(cgp_mlp* m);
  * every scratch word lives in one fixed file-scope device array of about 4.3 MB that each
  * device loading the library keeps until the process exits.
  *  - A in SELL-32 form (see cgp_mesh_get_level: slice s = rows 32s..32s+31, entries of a
- *    slice column-major, width = its longest row, padding with value 0): sell_ptr
- *    (nslices+1 offsets), sell_col, val; dinv = 1/diag(A).  n <= 65536 rows, else
+ *    slice column-major, width = its longest row, padding with value 0 and any column of
+ *    [0, n), also for the lanes beyond row n - 1): sell_ptr (nslices+1 offsets), sell_col, val;
+ *    dinv = 1/diag(A).  n <= 65536 rows, else
  *    CGP_EINVAL.  All pointers are device memory owned by the caller.
  *  - x: initial guess on entry, solution on exit.  info: 2 device int32 written at the end
  *    of the solve: iterations, status (CGP_OK, CGP_ENOTCONV, CGP_EBREAKDOWN, ...).
  *  - Asynchronous on `stream`.  The first call on a device looks up the array's device
  *    address and the launch size (make it before any stream capture); later calls only
- *    enqueue a memset of the barrier counter, the solve and a status copy.  The address is
+ *    enqueue a memset in the scratch array, the solve and a status copy.  The address is
  *    kept per device and context: after cudaDeviceReset the next call looks it up again
  *    (that call, too, belongs before any capture).
  *  - Every call shares the one array: calls whose solves may overlap on the GPU (different

@@ -437,12 +437,13 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         const int sl = (int)blockIdx.x * nw + wid;
         i = sl * 32 + lane;
         row = i < A.n;
-        if (sl < A.nslices) {
+        if (row) {   // (the lanes beyond the last row have nothing but padding)
             base = __ldg(A.ptr + sl) + lane;
             w_ = (__ldg(A.ptr + sl + 1) - base + lane) >> 5;
         }
     }
-    // ---- row data, loaded once
+    // ---- row data, loaded once.  An entry of value 0 (padding) reads the row's own word, which is
+    // always there: a padding column of no row would be awaited for ever.
     int col[kRRWidth];
     double av[kRRWidth];
     double dinv_i = 0.0;
@@ -451,8 +452,8 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         col[k] = 0;
         av[k] = 0.0;
         if (k < w_) {
-            col[k] = __ldg(A.col + base + 32 * k);
             av[k] = __ldg(a.val + base + 32 * k);
+            col[k] = av[k] != 0.0 ? __ldg(A.col + base + 32 * k) : i;
         }
     }
     if (row) {
@@ -500,7 +501,8 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
             }
         for (int k = kRRWidth; k < w_ && !bad; ++k) {   // entries beyond the registers
             const int e = base + 32 * k;
-            const int c = __ldg(A.col + e);
+            const double val = __ldg(a.val + e);
+            const int c = val != 0.0 ? __ldg(A.col + e) : i;
             double x;
             unsigned long long tg;
             ld_word(ubuf + 2 * (size_t)c, x, tg);
@@ -511,7 +513,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                 }
                 ld_word(ubuf + 2 * (size_t)c, x, tg);
             }
-            s0 += __ldg(a.val + e) * x;
+            s0 += val * x;
         }
         return s0 + s1;
     };
