@@ -748,10 +748,11 @@ static int cheb_mixed(Ctx& c, SellView A, const double* val, const float* valf, 
 
 // Steps of the FP64 semi-iteration for a mass solve to `tol` (two more than the energy-norm
 // bound asks for, since the test that follows is on the residual), or 0 where the caller's
-// iteration cap does not allow them: then PCG alone, as capped.
+// iteration cap does not allow them: then PCG alone, as capped.  The cap is one on the steps and
+// the PCG iterations after them together (and leaves those at least one).
 static int cheb64_steps(const Solver& s) {
     const int n = cheb_steps_for(0.25 * s.prm.tol_mass);
-    return n <= s.prm.max_it_mass ? n : 0;
+    return n < s.prm.max_it_mass ? n : 0;
 }
 
 // FP64 mass-matrix solve (Eqs. 25, 26) from x = 0: the same semi-iteration in FP64, then the
@@ -778,7 +779,7 @@ static int cheb_fp64(Ctx& c, SellView A, const double* val, const double* dinv, 
         rho = rho1;
     }
     CGP_LAUNCH_CHECK();
-    return pcg<NC>(c, A, val, dinv, b, x, ks, tol, maxit, false, false, pid);
+    return pcg<NC>(c, A, val, dinv, b, x, ks, tol, maxit - steps, false, false, pid);
 }
 
 // BiCGStab with FP32 inner solves (mixed form); the FP32 matrix is refreshed first
