@@ -557,13 +557,19 @@ constexpr int kTile = 32;
 
 // The 64 x 128 weight gradient of layer 2 (and its bias) as a register-tiled product: 256
 // threads hold 8 x 4 outputs each (o = og + 8 j, k = kg + 32 j), so 12 16-byte shared-memory
-// reads feed 128 FMAs; at most kWgradBlocks CTAs, two per SM.  Sums of 32 rows are added to the
-// running ones, which keeps the rounding of a two-level sum.
+// reads feed 128 FMAs; two CTAs per SM.  Sums of 32 rows are added to the running ones, those of
+// at most kRowsPerBlock rows, which keeps the rounding of a two-level sum: beyond kWgradBlocks
+// CTAs of that many rows (311,296) there are more CTAs, not longer FP32 sums.  (8.4M rows with 304
+// CTAs: equal terms added up to 1.3e-5 off, against 9e-7.)
 constexpr int kWgradBlocks = 304;
 
 inline int wgrad64_rows(int64_t rows) {   // rows per CTA, whole tiles
     const int64_t r = (rows + kWgradBlocks - 1) / kWgradBlocks;
-    return (int)((r + kTile - 1) / kTile * kTile);
+    return (int)std::min<int64_t>((r + kTile - 1) / kTile * kTile, kRowsPerBlock);
+}
+inline int wgrad64_blocks(int64_t rows) {
+    const int r = wgrad64_rows(rows);
+    return (int)((rows + r - 1) / r);
 }
 
 __global__ void __launch_bounds__(256, 2) k_mlp_wgrad64(int n, int batch, int rows, const float* __restrict__ ga,
@@ -771,7 +777,7 @@ extern "C" int cgp_mlp_create(const cgp_mesh* mesh, int32_t level, int32_t max_b
         m->grad = cv.take<float>(kMlpParams);
         m->adam_m = cv.take<float>(kMlpParams);
         m->adam_v = cv.take<float>(kMlpParams);
-        m->wpart = cv.take<float>(std::max((size_t)kWgradBlocks * kHid * (2 * kHid + 1), nblk * kHid * 9));
+        m->wpart = cv.take<float>(std::max((size_t)std::max(kWgradBlocks, wgrad64_blocks(nb)) * kHid * (2 * kHid + 1), nblk * kHid * 9));
         m->gA = cv.take<float>(kHid * nb);
         m->gB = cv.take<float>(kHid * nb);
         m->gM = cv.take<float>(kHid * nb);
@@ -887,7 +893,7 @@ static int mlp_backward(cgp_mlp* m, const double* r, const double* q, const doub
     CGP_TRY(mlp_forward_train(B, L, r, q, batch, st));
     const int g = blocks_for(nb), g256 = blocks_for(nb, 256);   // two vertices per thread of 128
     const dim3 gm((n + 31) / 32, batch), gw((n + kRowsPerBlock - 1) / kRowsPerBlock, batch);
-    const int rows64 = wgrad64_rows(nb), nblk64 = (int)((nb + rows64 - 1) / rows64);
+    const int rows64 = wgrad64_rows(nb), nblk64 = wgrad64_blocks(nb);
     const int nblk = (int)(gw.x * gw.y);
     int gl = (int)(nb / kBlock + 1);
     if (gl > 1024) gl = 1024;
