@@ -880,7 +880,15 @@ static int invert(Solver& s, int m, double* e, double* row, double shift, int sm
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    CGP_CUDA(cudaFuncSetAttribute(k_ml_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes));
+    // the most there is, not what this launch needs: the attribute is the function's, and another
+    // thread may be assembling a smaller system
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    CGP_CUDA(cudaGetDevice(&dev));
+    CGP_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    CGP_CUDA(cudaFuncGetAttributes(&fa, k_ml_inverse));
+    CGP_CUDA(cudaFuncSetAttribute(k_ml_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  optin - (int)fa.sharedSizeBytes));
     CGP_CUDA(cudaLaunchKernelEx(&cfg, k_ml_inverse, m, e, row, s.bar_count, s.bar_err, verdict));
     k_ml_symmetric<<<m, 128, 0, st>>>(m, e, shift);
     CGP_LAUNCH_CHECK();
