@@ -6,6 +6,7 @@
 // so every row is written by one thread and the sums are deterministic (no atomics).
 #include <algorithm>
 #include <cstring>
+#include <new>
 
 #include "flows.cuh"
 #include "guess_proj.cuh"
@@ -320,40 +321,18 @@ extern "C" int cgp_workspace_size(const cgp_mesh* mesh, const cgp_params* params
     return layout(s, nullptr, bytes);
 }
 
-extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void* workspace, size_t ws_bytes,
-                            cgp_stream_t stream, cgp_solver** out) {
-    clear_error();
-    if (!out) {
-        set_error("out is NULL");
-        return CGP_EINVAL;
-    }
-    *out = nullptr;
-    CGP_TRY(check_params(mesh, params));
-    cudaStream_t st = (cudaStream_t)stream;
-    cgp_solver* h = new cgp_solver();
-    Solver& s = h->s;
-    setup_dims(s, mesh, params);
-    size_t need = 0;
-    layout(s, nullptr, &need);
-    if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255)) {
-        set_error("workspace too small or not 256-byte aligned (%zu < %zu bytes)", ws_bytes, need);
-        delete h;
-        return CGP_ENOMEM;
-    }
-    layout(s, workspace, &need);
-    s.ws_bytes = ws_bytes;
+// everything of cgp_assemble after the workspace's layout; the caller destroys the solver on failure
+static int assemble_into(Solver& s, cudaStream_t st) {
+    const cgp_mesh* mesh = s.mesh;
+    const cgp_params* params = &s.prm;
     const Level& F = mesh->lev[s.lf];
     const Level& C = mesh->lev[s.lc];
-    auto fail = [&](int rc) {
-        cgp_solver_destroy(h);
-        return rc;
-    };
     // pure-Neumann coarse problem unless some coarse vertex has phi = 0
     {
         std::vector<uint8_t> tagc(C.nv);
         if (cudaMemcpy(tagc.data(), C.tag, C.nv, cudaMemcpyDeviceToHost) != cudaSuccess) {
             set_error("tag copy failed");
-            return fail(CGP_ECUDA);
+            return CGP_ECUDA;
         }
         s.pure_neumann = true;
         for (uint8_t t : tagc)
@@ -364,7 +343,7 @@ extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void
     if (cudaMemsetAsync(s.M, 0, (char*)s.geo - (char*)s.M, st) != cudaSuccess ||
         cudaMemsetAsync(s.Mc, 0, (char*)s.geoc - (char*)s.Mc, st) != cudaSuccess) {
         set_error("workspace initialisation failed");
-        return fail(CGP_ECUDA);
+        return CGP_ECUDA;
     }
     k_static_rows<<<blocks_for(F.nv), kBlock, 0, st>>>(F.nv, F.rowptr, F.col, F.sell_ptr, F.vt_ptr, F.vt_list, F.tri, s.geo,
                                                        s.M, s.K, s.Cx, s.Cy, s.CxT, s.CyT, s.vtslot);
@@ -390,11 +369,11 @@ extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void
     }
     if (cudaGetLastError() != cudaSuccess) {
         set_error("assembly launch failed");
-        return fail(CGP_ECUDA);
+        return CGP_ECUDA;
     }
     {
         int rc = choose_coarse_solver(s, st);
-        if (rc != CGP_OK) return fail(rc);
+        if (rc != CGP_OK) return rc;
     }
     if (cudaMemsetAsync(s.tickets, 0, 64 * sizeof(unsigned int), st) != cudaSuccess ||
         cudaMemsetAsync(s.ks, 0, (KS_COUNT + 1) * sizeof(KrylovState), st) != cudaSuccess ||
@@ -406,10 +385,10 @@ extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void
         (s.proj && cudaMemsetAsync(s.proj, 0, sizeof(ProjState), st) != cudaSuccess) ||
         (s.mlp_gate && cudaMemsetAsync(s.mlp_gate, 0, 4 * sizeof(int), st) != cudaSuccess)) {
         set_error("workspace initialisation failed");
-        return fail(CGP_ECUDA);
+        return CGP_ECUDA;
     }
     int rc = init_state(&s, st);
-    if (rc != CGP_OK) return fail(rc);
+    if (rc != CGP_OK) return rc;
     if (cudaStreamCreateWithFlags(&s.side, cudaStreamNonBlocking) != cudaSuccess ||
         cudaStreamCreateWithFlags(&s.branch, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&s.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -417,11 +396,51 @@ extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void
         cudaMallocHost(&s.h_flag, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&s.h_view, sizeof(Solver::HostView)) != cudaSuccess) {
         set_error("stream / pinned flag creation failed");
-        return fail(CGP_ECUDA);
+        return CGP_ECUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) {
         set_error("assembly failed on the device: %s", cudaGetErrorString(cudaGetLastError()));
-        return fail(CGP_ECUDA);
+        return CGP_ECUDA;
+    }
+    return CGP_OK;
+}
+
+extern "C" int cgp_assemble(const cgp_mesh* mesh, const cgp_params* params, void* workspace, size_t ws_bytes,
+                            cgp_stream_t stream, cgp_solver** out) {
+    clear_error();
+    if (!out) {
+        set_error("out is NULL");
+        return CGP_EINVAL;
+    }
+    *out = nullptr;
+    CGP_TRY(check_params(mesh, params));
+    cgp_solver* h = new (std::nothrow) cgp_solver();
+    if (!h) {
+        set_error("no host memory for the solver");
+        return CGP_ENOMEM;
+    }
+    Solver& s = h->s;
+    setup_dims(s, mesh, params);
+    size_t need = 0;
+    layout(s, nullptr, &need);
+    if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255)) {
+        set_error("workspace too small or not 256-byte aligned (%zu < %zu bytes)", ws_bytes, need);
+        delete h;
+        return CGP_ENOMEM;
+    }
+    layout(s, workspace, &need);
+    s.ws_bytes = ws_bytes;
+    int rc;
+    try {
+        rc = assemble_into(s, (cudaStream_t)stream);
+    } catch (const std::bad_alloc&) {   // of a host copy or plan
+        set_error("no host memory to assemble with");
+        rc = CGP_ENOMEM;
+    }
+    if (rc != CGP_OK) {
+        cudaStreamSynchronize((cudaStream_t)stream);   // the workspace is the caller's again
+        cgp_solver_destroy(h);
+        return rc;
     }
     *out = h;
     return CGP_OK;

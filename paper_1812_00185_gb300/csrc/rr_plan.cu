@@ -1,7 +1,7 @@
 // Host plans of the FP64 coarse solves over compact subdomains (see rr_plan.cuh).
 #include <algorithm>
 #include <cmath>
-#include <system_error>
+#include <exception>
 #include <thread>
 #include <utility>
 
@@ -42,7 +42,7 @@ void bisect(Point* p, int lo, int hi, int p0, int p1, int cap, int32_t* first) {
     if (here > 100000) {
         try {
             other = std::thread(bisect, p, lo, mid, p0, p0 + left, cap, first);
-        } catch (const std::system_error&) {   // no thread to be had: one after the other
+        } catch (const std::exception&) {   // no thread or no memory for one: one after the other
         }
     }
     if (!other.joinable()) bisect(p, lo, mid, p0, p0 + left, cap, first);

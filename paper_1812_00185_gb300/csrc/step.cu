@@ -1124,17 +1124,17 @@ int choose_coarse_solver(Solver& s, cudaStream_t st) {
             const bool plan_rr = sh.ctas > kRRSingle && s.rr_perm;
             const bool fp64 = p.precision == CGP_FP64 || p.coarse_mode == CGP_COARSE_AUTO;   // (as below)
             s.direct_ctas = 0;
-            if (s.direct_inv) CGP_TRY(direct_plan(s, sms, st));
-            const bool plan_ml = !s.direct_ctas && s.ml_perm;
-            if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_ml)) {
-                try {
+            try {
+                if (s.direct_inv) CGP_TRY(direct_plan(s, sms, st));
+                const bool plan_ml = !s.direct_ctas && s.ml_perm;
+                if (p.precond == CGP_PRECOND_AUTO && fp64 && !s.onchip_bytes && (plan_rr || plan_ml)) {
                     if (plan_ml) CGP_TRY(multilevel_plan(s, sms, st));
                     if (s.ml.nsub) s.rr_ctas = 0;
                     else if (plan_rr) CGP_TRY(subdomain_plan(s, sh, st));
-                } catch (const std::bad_alloc&) {   // no host memory for the plan: Jacobi alone
-                    s.rr_nsub = s.ml.nsub = 0;
-                    s.rr_ctas = sh.ctas;
                 }
+            } catch (const std::bad_alloc&) {   // no host memory for the plan: Jacobi alone
+                s.rr_nsub = s.ml.nsub = s.direct_ctas = 0;
+                s.rr_ctas = sh.ctas;
             }
         }
         // mixed form, AUTO, no room on chip: the grid-wide FP64 solve (one reduction per
