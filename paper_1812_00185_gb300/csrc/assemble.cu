@@ -164,7 +164,7 @@ static int layout(Solver& s, void* base, size_t* bytes) {
     s.geoc = cv.take<double>((size_t)7 * C.nt);
     s.Kc0f = cv.take<float>(nnzc);
     s.dinvKcf = cv.take<float>(nc);
-    s.cw64 = cv.take<double>(5 * nc + 1410);   // 5 vectors, or the register-resident solve's words (coarse_rr.cuh)
+    s.cw64 = cv.take<double>(std::max<size_t>(5 * nc, rr_work_doubles((int)nc)));   // 5 vectors, or the register-resident solve's words
     // its plan: a thread per row of at most one slice more per CTA than the rows need, and E^+
     if (s.prm.precond == CGP_PRECOND_AUTO && s.prm.precision == CGP_FP64 && s.nc <= kDirectMaxRows &&
         (s.prm.coarse_mode == CGP_COARSE_AUTO || s.prm.coarse_mode == CGP_COARSE_PERSISTENT) &&

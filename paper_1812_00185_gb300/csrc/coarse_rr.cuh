@@ -63,7 +63,6 @@ constexpr int kRRMaxWarps = 16;      // warps (slices) per CTA: 512 threads of u
 constexpr int kRRMinWarps = 4;       // the reductions use three warps
 constexpr int kRRCluster = 8;        // CTAs per cluster of a launch of several clusters: 8, or 4
 constexpr int kRRSingle = 16;        // CTAs of a launch of one cluster (small systems)
-constexpr int kRRMaxClusters = 64;   // clusters of a launch: two polled words per lane
 
 struct RRShape {
     int ctas = 0, cluster = 0, warps = 0;   // ctas = 0: the system does not fit
@@ -102,12 +101,6 @@ inline RRShape rr_shape(int nslices, const RRCapacity& cap) {
     }
     return s;
 }
-
-// Work area (doubles): words [2][3][kRRMaxClusters], words of the CTAs' Z^T w [2][kRRMaxSub], the
-// error word (2 doubles), u words [n].  Zeroed before every launch: generation 0 is never awaited.
-constexpr size_t kRRZWords = 12 * (size_t)kRRMaxClusters;
-constexpr size_t kRRHead = kRRZWords + 4 * (size_t)kRRMaxSub + 2;
-inline size_t rr_work_doubles(int n) { return kRRHead + 2 * (size_t)n; }
 
 // one 16-byte {value, tag} word, single-copy atomic, at L2
 __device__ __forceinline__ void st_word(double* p, double v, unsigned long long tag) {

@@ -5,12 +5,20 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdint>
 #include <vector>
 
 namespace cgp {
 
 constexpr int kRRMaxSub = 160;   // subdomains (one per CTA): five per lane of a warp
+constexpr int kRRMaxClusters = 64;   // clusters of a launch: two polled words per lane
+
+// Work area (doubles): words [2][3][kRRMaxClusters], words of the CTAs' Z^T w [2][kRRMaxSub], the
+// error word (2 doubles), u words [n].  Zeroed before every launch: generation 0 is never awaited.
+constexpr size_t kRRZWords = 12 * (size_t)kRRMaxClusters;
+constexpr size_t kRRHead = kRRZWords + 4 * (size_t)kRRMaxSub + 2;
+inline size_t rr_work_doubles(int n) { return kRRHead + 2 * (size_t)n; }
 
 struct RRHostPlan {
     int nsub = 0;                  // 0: no plan (the slices in order, Jacobi alone)
