@@ -148,6 +148,7 @@ __device__ __forceinline__ bool mbar_try(uint64_t* mb, uint32_t parity) {
 
 constexpr long long kRRWaitCycles = 4000000000LL;    // ~2 s: a wait this long means a lost signal
 constexpr long long kRRWaitCyclesTest = 20000000LL;  // ~10 ms, under the wait test hook
+constexpr long long kRRDrainCycles = 100000LL;       // ~50 us, after a wait that ran out
 
 constexpr int kRREinvMax = kRRCluster * kRRMaxSub;   // and kRRSingle^2 is less
 static_assert(kRRSingle * kRRSingle <= kRREinvMax, "rows of E^+ of one cluster");
@@ -641,6 +642,14 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
     }
     if (row) a.x[i] = x_i;
     cgrp::this_cluster().sync();   // no CTA leaves while its shared memory may be written
+    if (status == CGP_ETIMEOUT) {
+        // a CTA whose wait ran out has not seen every store that was sent to it: all are on their way
+        // now, and 50 us outlast the latest of them
+        const long long t0 = clock64();
+        while (clock64() - t0 < kRRDrainCycles) {
+        }
+        cgrp::this_cluster().sync();
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         KrylovState* st = a.st;
         st->iter = iters;
