@@ -200,15 +200,14 @@ __global__ void __launch_bounds__(256) k_mlp_nmean64_bwd(int n, const int32_t* _
 // order; with VOUT also hv[b][i][o] = relu(a[b][o][i]) (the vertex-major copy the next
 // 1-ring mean gathers).  W (bf16, row-major FOUT x 2*FIN) is staged per block as FP32
 // columns wt[k][o]: lane l of a warp loads 8 consecutive k of row o = l (16 bytes) and
-// writes them down column l, so the transposed writes are free of bank conflicts.  With
-// FOUT >= 32 two threads share a vertex (the first half of the block takes outputs
+// writes them down column l, so the transposed writes are free of bank conflicts.
+// Two threads share a vertex (the first half of the block takes outputs
 // [0, FOUT/2), the second half the rest, so a warp reads one wt row as a broadcast), and each
 // thread has two vertices, so a weight read from shared memory feeds two FMAs (one read per
 // FMA held the kernel at the shared-memory pipe's rate).  Each thread loads its inputs in
 // chunks, the next chunk while it multiplies the current one, so the latency of the
 // feature-major input loads overlaps the FMAs.
-template <int FOUT>
-__host__ __device__ constexpr int dense_vertices_per_block() { return 128; }   // of 128 threads
+constexpr int kDenseVertices = 128;   // per block of 128 threads
 
 template <int FIN, int FOUT, bool RELU_IN, bool VOUT>
 __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_bfloat16* __restrict__ W,
@@ -216,16 +215,13 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
                                                    const float* __restrict__ m, float* __restrict__ a,
                                                    float* __restrict__ hv) {
     constexpr int K = 2 * FIN;
-    constexpr int VB = dense_vertices_per_block<FOUT>();
-    constexpr int OS = FOUT >= 32 ? 2 : 1;              // threads per vertex
-    constexpr int V = OS * VB / 128;                    // vertices per thread
+    constexpr int OS = 2;                               // threads per vertex
+    constexpr int V = OS * kDenseVertices / 128;        // vertices per thread
     constexpr int FO = FOUT / OS;                       // outputs per thread
-    constexpr int LD = FOUT == 1 ? 1 : FOUT + 4;        // row stride of wt (16-byte rows)
-    constexpr int KCMAX = FO == 1 ? 32 : 8;
-    constexpr int KC = FIN < KCMAX ? FIN : KCMAX;       // inputs loaded per chunk
+    constexpr int LD = FOUT + 4;                        // row stride of wt (16-byte rows)
+    constexpr int KC = FIN < 8 ? FIN : 8;               // inputs loaded per chunk
     constexpr int NV8 = K * FOUT / 8;                   // 16-byte pieces of W
-    static_assert(FOUT % OS == 0 && (FO == 1 || FO % 4 == 0) && FIN % KC == 0 && K % 8 == 0, "dense layer shape");
-    static_assert(!VOUT || FO % 4 == 0, "vertex-major copy in 16-byte stores");
+    static_assert(FOUT % OS == 0 && FO % 4 == 0 && FIN % KC == 0 && K % 8 == 0, "dense layer shape");
     __shared__ __align__(16) float wt[K][LD];
     const uint4* W8 = reinterpret_cast<const uint4*>(W);
 #pragma unroll
@@ -253,7 +249,7 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
     float acc[V][FO];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-        const int64_t t = blockIdx.x * (int64_t)VB + threadIdx.x % TV + v * TV;
+        const int64_t t = blockIdx.x * (int64_t)kDenseVertices + threadIdx.x % TV + v * TV;
         in[v] = t < (int64_t)n * batch;
         b[v] = in[v] ? (int)(t / n) : 0;
         i[v] = in[v] ? (int)(t % n) : 0;
@@ -283,23 +279,16 @@ __global__ void __launch_bounds__(128) k_mlp_dense(int n, int batch, const __nv_
 #pragma unroll
         for (int u = 0; u < KC; ++u) {
             const float* wr = &wt[c * KC + u][o0];
-            if constexpr (FO % 4 == 0) {
 #pragma unroll
-                for (int o = 0; o < FO; o += 4) {
-                    const float4 w4 = *reinterpret_cast<const float4*>(wr + o);
+            for (int o = 0; o < FO; o += 4) {
+                const float4 w4 = *reinterpret_cast<const float4*>(wr + o);
 #pragma unroll
-                    for (int v = 0; v < V; ++v) {
-                        acc[v][o] += w4.x * xs[v][u];
-                        acc[v][o + 1] += w4.y * xs[v][u];
-                        acc[v][o + 2] += w4.z * xs[v][u];
-                        acc[v][o + 3] += w4.w * xs[v][u];
-                    }
+                for (int v = 0; v < V; ++v) {
+                    acc[v][o] += w4.x * xs[v][u];
+                    acc[v][o + 1] += w4.y * xs[v][u];
+                    acc[v][o + 2] += w4.z * xs[v][u];
+                    acc[v][o + 3] += w4.w * xs[v][u];
                 }
-            } else {
-#pragma unroll
-                for (int v = 0; v < V; ++v)
-#pragma unroll
-                    for (int o = 0; o < FO; ++o) acc[v][o] += wr[o] * xs[v][u];
             }
         }
     };
@@ -711,21 +700,20 @@ void MlpBuffers::carve(Carve& cv, int n_, int batch) {
     a1 = cv.take<float>(kHid * nb);
     m1 = cv.take<float>(kHid * nb);
     a2 = cv.take<float>(kHid * nb);
-    m2 = cv.take<float>(kHid * nb);
+    pz = cv.take<float2>(nb);
     hv = cv.take<float>(kHid * nb);
-    out = cv.take<float>(nb);
     params_bf = cv.take<__nv_bfloat16>(kMlpParams);
     params = cv.take<float>(kMlpParams);
 }
 
-// the training forward pass up to layer 3's (p, z) (in B.m2): every activation kept
+// the training forward pass up to layer 3's (p, z): every activation kept
 // (feature-major) for mlp_backward
 static int mlp_forward_train(const MlpBuffers& B, const Level& L, const double* r, const double* q, int batch,
                              cudaStream_t st) {
     const int n = B.n;
     const int64_t nb = (int64_t)n * batch;
     const int g = blocks_for(nb);
-    const int gh = blocks_for(nb, dense_vertices_per_block<kHid>());
+    const int gh = blocks_for(nb, kDenseVertices);
     k_mlp_scales<<<dim3(kScaleBlocks, batch), kBlock, 0, st>>>(n, r, q, B.spart);
     k_mlp_scales_fin<<<batch, 32, 0, st>>>(n, kScaleBlocks, B.spart, B.scale);
     k_mlp_features<<<g, kBlock, 0, st>>>(n, batch, r, q, L.xy, B.scale, B.h0);
@@ -736,7 +724,7 @@ static int mlp_forward_train(const MlpBuffers& B, const Level& L, const double* 
     k_mlp_nmean64<<<gm, 256, 0, st>>>(n, L.rowptr, L.col, B.hv, B.m1);
     k_mlp_dense<kHid, kHid, true, false><<<gh, 128, 0, st>>>(n, batch, B.params_bf + kOffW2, B.params + kOffB2, B.a1,
                                                               B.m1, B.a2, nullptr);
-    k_mlp_l3_pz<<<g, kBlock, 0, st>>>(n, batch, B.params_bf + kOffW3, B.a2, reinterpret_cast<float2*>(B.m2));
+    k_mlp_l3_pz<<<g, kBlock, 0, st>>>(n, batch, B.params_bf + kOffW3, B.a2, B.pz);
     CGP_LAUNCH_CHECK();
     return CGP_OK;
 }
@@ -897,9 +885,8 @@ static int mlp_backward(cgp_mlp* m, const double* r, const double* q, const doub
     const int nblk = (int)(gw.x * gw.y);
     int gl = (int)(nb / kBlock + 1);
     if (gl > 1024) gl = 1024;
-    const float2* pz = reinterpret_cast<const float2*>(B.m2);
     float2* gs = reinterpret_cast<float2*>(m->gM);   // free until layer 2's mean part
-    k_mlp_loss<<<gl, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, B.params + kOffB3, pz, q, tgt, B.scale, m->g3,
+    k_mlp_loss<<<gl, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, B.params + kOffB3, B.pz, q, tgt, B.scale, m->g3,
                                       m->partials, m->ticket, m->loss);
     // layer 3: gA = dL/da2, then dW3, db3
     k_mlp_l3_bwd<<<g, kBlock, 0, st>>>(n, batch, L.rowptr, L.col, B.params_bf + kOffW3, m->g3, B.a2, gs, m->gA);

@@ -27,9 +27,9 @@ struct MlpBuffers {
     double* spart = nullptr;                    // [batch][kScaleBlocks][2]: block partial sums of r^2, q^2
     float *h0 = nullptr, *m0 = nullptr;         // [batch][4][n]
     float *a1 = nullptr, *m1 = nullptr;         // [batch][64][n] pre-activations / neighbour means
-    float *a2 = nullptr, *m2 = nullptr;
+    float* a2 = nullptr;
+    float2* pz = nullptr;                       // [batch][n]: layer 3's products (training)
     float* hv = nullptr;                        // [batch][n][64]: vertex-major copy for the 1-ring means
-    float* out = nullptr;                       // [batch][n]
     __nv_bfloat16* params_bf = nullptr;         // bfloat16 copy used by the forward kernels
     float* params = nullptr;                    // FP32 master (biases are read from here)
     void carve(Carve& cv, int n, int batch);
