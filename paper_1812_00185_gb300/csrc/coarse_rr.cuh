@@ -431,13 +431,17 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         const int sl = (int)blockIdx.x * nw + wid;
         i = sl * 32 + lane;
         row = i < A.n;
-        if (row) {   // (the lanes beyond the last row have nothing but padding)
+        if (row) {
+            // up to the last entry that is not 0, so that no word is awaited for padding, whose
+            // column may be no row's (and none for the lanes beyond the last row)
             base = __ldg(A.ptr + sl) + lane;
-            w_ = (__ldg(A.ptr + sl + 1) - base + lane) >> 5;
+            const int width = (__ldg(A.ptr + sl + 1) - base + lane) >> 5;
+#pragma unroll 8
+            for (int k = 0; k < width; ++k)
+                if (__ldg(a.val + base + 32 * k) != 0.0) w_ = k + 1;
         }
     }
-    // ---- row data, loaded once.  An entry of value 0 (padding) reads the row's own word, which is
-    // always there: a padding column of no row would be awaited for ever.
+    // ---- row data, loaded once
     int col[kRRWidth];
     double av[kRRWidth];
     double dinv_i = 0.0;
@@ -446,8 +450,8 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
         col[k] = 0;
         av[k] = 0.0;
         if (k < w_) {
+            col[k] = __ldg(A.col + base + 32 * k);
             av[k] = __ldg(a.val + base + 32 * k);
-            col[k] = av[k] != 0.0 ? __ldg(A.col + base + 32 * k) : i;
         }
     }
     if (row) {
@@ -495,8 +499,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
             }
         for (int k = kRRWidth; k < w_ && !bad; ++k) {   // entries beyond the registers
             const int e = base + 32 * k;
-            const double val = __ldg(a.val + e);
-            const int c = val != 0.0 ? __ldg(A.col + e) : i;
+            const int c = __ldg(A.col + e);
             double x;
             unsigned long long tg;
             ld_word(ubuf + 2 * (size_t)c, x, tg);
@@ -507,7 +510,7 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
                 }
                 ld_word(ubuf + 2 * (size_t)c, x, tg);
             }
-            s0 += val * x;
+            s0 += __ldg(a.val + e) * x;
         }
         return s0 + s1;
     };
