@@ -439,6 +439,8 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
         double gamma = 0.0, d = 0.0, rr_best = INFINITY;
         int best_k = 0, leave = 0;
         for (int k = 0;; ++k) {
+            // 1 / gamma', off the reduction's chain
+            const double rg = k && wid == 0 ? newton_quotient(1.0, gamma) : 0.0;
             v[1] = 0.0;
             for (int sl = s_begin + wid; sl < s_end; sl += nw) {
                 const int i = sl * 32 + lane;
@@ -453,7 +455,7 @@ static __global__ void __launch_bounds__(kT, 1) k_pcg_grid_ml(CoarsePcgArgs a, M
             }
             // out: alpha, beta, gamma, d; flag as in inner_pcg
             if (!sy.reduce(v, o, flag, t, [&](const double (&s)[3], double (&q)[4]) -> int {
-                    const double rg = k ? newton_quotient(1.0, gamma) : 0.0, beta = s[0] * rg;
+                    const double beta = s[0] * rg;
                     q[3] = k ? fma(-beta * beta, d, s[1]) : s[1];
                     q[2] = s[0];
                     q[1] = beta;

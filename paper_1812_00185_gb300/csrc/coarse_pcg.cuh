@@ -224,10 +224,12 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
 
 // n / d by Newton's iteration for 1 / d from the 20-bit approximation (two steps: 80 bits, so
 // the quotient is within rounding of the exact one); not finite where d is 0 or not finite.  The
-// approximation takes subnormal d for 0 and has 0 for 1 / d from 2^1022 on: there a division.
+// approximation takes subnormal d for 0 and has 0 for 1 / d from 2^1022 on: there a division (a
+// call, or its chain takes part in every quotient).
+static __device__ __noinline__ double divided(double n, double d) { return n / d; }
 __device__ __forceinline__ double newton_quotient(double n, double d) {
     const unsigned ex = (unsigned)__double2hiint(d) >> 20 & 0x7ffu;
-    if (ex - 1u >= 0x7fcu && ex != 0x7ffu) return n / d;
+    if (ex - 1u >= 0x7fcu && ex != 0x7ffu) return divided(n, d);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     r = fma(r, fma(-d, r, 1.0), r);
