@@ -136,7 +136,13 @@ enum { CGP_RESTRICT_INJECT = 0, CGP_RESTRICT_PT = 1 };
  * below it (Bramble, Pasciak and Xu) with the subdomain correction on the base mesh (not with the
  * learned guess, which has the correction with one subdomain per CTA in the register-resident
  * solve).  JACOBI elsewhere.  The solution is the same to the solve's tolerance; only the
- * iteration count changes. */
+ * iteration count changes.
+ * What AUTO prepares for FP64 solves costs cgp_assemble time and workspace (GB300): the inverse
+ * 5.8 ms and n^2 doubles at n = 1,089 rows, 12.5 ms and 20 MB at 1,600; the multilevel plan 3 ms for
+ * small base meshes, 9 ms for one of 66,049 vertices, 19 ms for 263,169, and 3 to 7 MB; JACOBI 0.2 to
+ * 0.9 ms.  Against JACOBI an inverse has paid for itself after 8 to 17 solves.  A solver that makes
+ * few solves of its own, only prolongs, or only runs in a batch (whose coarse solves use Jacobi
+ * whatever was prepared) is cheaper with JACOBI. */
 enum { CGP_PRECOND_AUTO = 0, CGP_PRECOND_JACOBI = 1, CGP_PRECOND_COARSE = 2 };
 
 /* Coarse Poisson solver kinds.  KERNELS: two kernel launches per PCG iteration (graph
@@ -186,7 +192,8 @@ int cgp_mesh_get_level(const cgp_mesh* mesh, int32_t level, double* xy, int32_t*
 void cgp_mesh_destroy(cgp_mesh* mesh);
 
 /* ---- solver ---- */
-/* Workspace bytes cgp_assemble needs for this mesh and parameters. */
+/* Workspace bytes cgp_assemble needs for this mesh and parameters (precond = AUTO: with room for what
+ * it prepares, see there). */
 int cgp_workspace_size(const cgp_mesh* mesh, const cgp_params* params, size_t* bytes);
 /* Assemble the static P1 operators (Eqs. 17-20) on the velocity level and, by
  * rediscretisation, on the pressure-increment level (Section 2.2), and set the
@@ -300,7 +307,7 @@ void cgp_solver_destroy(cgp_solver* s);
  *  - whole step (CGP_BATCH_WHOLE_STEP, the default when every instance qualifies: injection
  *    restriction, a zero or previous-increment coarse guess, a one-launch coarse solver):
  *    every batched step is ONE persistent launch in which thread-block clusters take
- *    instances from a queue, largest first, and run each instance's whole step of Eqs. 21-26
+ *    instances from a queue, longest step (by an estimate) first, and run each instance's whole step of Eqs. 21-26
  *    (momentum rows and FP64 BiCGStab, coarse right-hand side and the instance's coarse PCG,
  *    prolongation, Chebyshev mass solves of Eqs. 25-26 with the eigenvalue bounds [1/2, 2] of
  *    Jacobi-scaled P1 mass matrices, FP32 steps inside FP64 refinement in mixed instances,
@@ -329,7 +336,8 @@ int cgp_batch_mode(const cgp_batch* b, int32_t* mode);
  * cgp_get_fields on each solver. */
 int cgp_batch_step(cgp_batch* b, int32_t n_steps, cgp_stream_t stream);
 /* Chosen shape, clusters per launch, and the autotuner's trial times (ms; -1 = not run) for
- * the candidates (cluster, threads) = (1,256),(1,512),(1,1024),(2,256),...,(8,1024). */
+ * the candidates (cluster, threads) = (1,256),(1,512),(1,1024),(2,256),...,(8,1024), and in the
+ * whole-step form (16,256),(16,512). */
 int cgp_batch_info(const cgp_batch* b, int32_t* cluster_size, int32_t* threads, int32_t* nclusters, float* trial_ms,
                    int32_t n_trials);
 void cgp_batch_destroy(cgp_batch* b);

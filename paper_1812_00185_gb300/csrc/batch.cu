@@ -3,7 +3,7 @@
 // Whole-step form (the default whenever every instance qualifies: injection restriction, a
 // zero or previous-increment coarse guess, a one-launch coarse solver): one batched step is
 // ONE persistent clustered launch (k_batch_step, batch_step.cuh) in which every cluster takes
-// instances from a queue, largest first, and runs each one's entire step; the cluster size
+// instances from a queue, longest step first, and runs each one's entire step; the cluster size
 // and threads per CTA are autotuned on the batch's own first step (the instances' state is
 // saved and restored around the trials).  The launch is captured in a CUDA graph.
 //
@@ -11,7 +11,7 @@
 //   for every instance, on its own stream (independent graph branches):
 //       Eq. 21 momentum solve, Eqs. 22-23 right-hand side        (step_pre)
 //   ONE persistent launch: the coarse Poisson solves of all instances; clusters take
-//       instances from a queue, largest first                    (k_pcg_batch)
+//       instances from a queue, longest step first               (k_pcg_batch)
 //   for every instance, on its own stream:
 //       Eqs. 24-26, end of step                                  (step_post)
 // The cluster size and the threads per CTA of the persistent launch are chosen by an

@@ -1,6 +1,6 @@
 // The whole CGP step of many independent instances in ONE persistent launch (a form beyond
 // the paper).  Every thread-block cluster of the launch takes instances from a queue (the
-// host orders them largest first) and advances each by one complete step of Eqs. 21-26;
+// host orders them by an estimate of their step, longest first) and advances each by one complete step of Eqs. 21-26;
 // the cluster's CTAs share the rows, reduce through distributed shared memory, and
 // synchronise with the hardware cluster barrier between phases; clusters never wait on one
 // another.

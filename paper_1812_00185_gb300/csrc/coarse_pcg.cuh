@@ -837,7 +837,7 @@ static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_cluster(Coars
 }
 
 // Coarse solves of many independent CGP instances in ONE persistent launch: every cluster
-// of the launch takes instances from a queue (the host orders them largest first) and
+// of the launch takes instances from a queue (the host orders them longest step first) and
 // solves each with the ClusterSync body; clusters never wait on one another.
 static __global__ void __launch_bounds__(kClusterThreads, 1) k_pcg_batch(const CoarsePcgArgs* __restrict__ args, int ninst,
                                                                   unsigned int* queue) {
