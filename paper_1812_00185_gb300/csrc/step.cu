@@ -849,13 +849,14 @@ static int subdomain_plan(Solver& s, const RRShape& sh, cudaStream_t st) {
     CGP_CUDA(cudaMemcpy(val.data(), s.Kc0, sizeof(double) * C.nnz_sell, cudaMemcpyDeviceToHost));
     CGP_CUDA(cudaMemcpy(in_space.data(), C.tag, C.nv, cudaMemcpyDeviceToHost));
     for (auto& t : in_space) t = (t & CGP_PHI_ZERO) ? 0 : 1;
-    auto up = [](auto* dst, const auto& v) {
-        return cudaMemcpy(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
+    auto up = [st](auto* dst, const auto& v) {   // on the stream of the solves
+        return cudaMemcpyAsync(dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice, st);
     };
     RRHostPlan P;
     if (!rr_plan(C.nv, rowptr, ptr, col, val, xy, in_space, sh.ctas, 32 * sh.warps, s.pure_neumann, P)) return CGP_OK;
     CGP_CUDA(up(s.rr_perm, P.perm));
     CGP_CUDA(up(s.rr_einv, P.einv));
+    CGP_CUDA(cudaStreamSynchronize(st));   // P goes
     s.rr_nsub = P.nsub;
     return CGP_OK;
 }
