@@ -13,7 +13,7 @@ from workloads import WORKLOADS
 pytestmark = [pytest.mark.gpu, pytest.mark.slow]
 
 
-@pytest.mark.parametrize("name", ["channel1m_k2", "cavity512_k1", "cavity512_k2", "cavity512_k3"])
+@pytest.mark.parametrize("name", ["channel1m_k2", "cavity512_k1"])
 def test_fp64_default_matches_oracle(lib, name):
     from paper_1812_00185_gb300 import binding as cg
     from paper_1812_00185_gb300.forms import workload_params
