@@ -647,11 +647,10 @@ static __global__ void __launch_bounds__(kWarps * 32, 1) k_pcg_grid_rr(CoarsePcg
     cgrp::this_cluster().sync();   // no CTA leaves while its shared memory may be written
     if (status == CGP_ETIMEOUT) {
         // a CTA whose wait ran out has not seen every store that was sent to it: all are on their way
-        // now, and 50 us outlast the latest of them
+        // now, and 50 us outlast the latest of them (no further meeting: the others may be gone)
         const long long t0 = clock64();
         while (clock64() - t0 < kRRDrainCycles) {
         }
-        cgrp::this_cluster().sync();
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         KrylovState* st = a.st;
